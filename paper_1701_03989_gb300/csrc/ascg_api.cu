@@ -1248,7 +1248,7 @@ void set_last_error(const std::string& msg) { g_err = msg; }
 
 ascg_status check_options(const ascg_options& o) { return check_opts(o); }
 
-ascg_status op_split_desc(ascg_op op, SysDesc* d, int* device) {
+ascg_status op_split_desc(ascg_op op, SysDesc* d, int* device, double* row_len) {
   if (!op) return fail(ASCG_ERR_INVALID, "op is NULL");
   std::memset(d, 0, sizeof(*d));
   d->n = op->n;
@@ -1257,6 +1257,7 @@ ascg_status op_split_desc(ascg_op op, SysDesc* d, int* device) {
   d->o_val = op->o_val;
   d->diag = op->diag;
   *device = op->device;
+  *row_len = (double)op->o_len / (double)op->n;
   return ASCG_OK;
 }
 }  // namespace ascg

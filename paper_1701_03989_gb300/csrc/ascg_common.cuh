@@ -44,6 +44,73 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+__device__ __forceinline__ unsigned biased_exp(double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu; }
+
+// t + sum_k a_k x[c_k] over the `width` sliced-ELL entries of one row (v, c at
+// the lane's first entry, stride kSlice), one FMA each in stored order. In
+// groups of kRowGroup entries: while a group's FMAs run, the next group's
+// gathers and the loads of A of the group after it are in flight, so that a
+// warp alone on its scheduler waits on its FMA chain and not on memory.
+constexpr int kRowGroup = 4;
+__device__ __forceinline__ double row_chain(const double* __restrict__ v, const int32_t* __restrict__ c, int width,
+                                            const double* __restrict__ x, double t) {
+  constexpr int G = kRowGroup;
+  double a0[G], a1[G], x0[G];
+  int c1[G];
+#pragma unroll
+  for (int q = 0; q < G; ++q) {
+    a0[q] = a1[q] = x0[q] = 0.0;
+    c1[q] = 0;
+  }
+  {
+    int c0[G];
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+      if (q < width) {
+        c0[q] = __ldg(c + kSlice * q);
+        a0[q] = __ldg(v + kSlice * q);
+      }
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+      if (G + q < width) {
+        c1[q] = __ldg(c + kSlice * (G + q));
+        a1[q] = __ldg(v + kSlice * (G + q));
+      }
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+      if (q < width) x0[q] = __ldg(x + c0[q]);
+  }
+  for (int k = 0; k < width; k += G) {
+    double x1[G], a2[G];
+    int c2[G];
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+      x1[q] = a2[q] = 0.0;
+      c2[q] = 0;
+    }
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+      if (k + G + q < width) x1[q] = __ldg(x + c1[q]);
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+      if (k + 2 * G + q < width) {
+        c2[q] = __ldg(c + kSlice * (k + 2 * G + q));
+        a2[q] = __ldg(v + kSlice * (k + 2 * G + q));
+      }
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+      if (k + q < width) t = fma(a0[q], x0[q], t);
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+      a0[q] = a1[q];
+      a1[q] = a2[q];
+      x0[q] = x1[q];
+      c1[q] = c2[q];
+    }
+  }
+  return t;
+}
+
 // Raises a kernel's dynamic shared-memory limit to `bytes` on the current
 // device, once per device (devices 0..63; others every call). The device's
 // flag is set only after the attribute call succeeded, so a caller that sees
@@ -235,11 +302,16 @@ bool gram_tc_fits(int64_t n);
 // Y (rows x w used, leading dimension ldY, rows a multiple of 1024): items
 // are whole 1024-row chunks of one system each (GramItem rows in Y, nrows a
 // multiple of 1024, at most 8 chunks); items of systems with sys_w 0 skip.
-// Each item gets its system's column exponents (emax_all: nsys x 33 ints,
-// zeroed and filled here) and writes w(w+1)/2 partials.
+// Each item takes its system's column exponents (emax_all: 33 ints per
+// system, filled by launch_tc_items_exponents or the matrix powers steps) and
+// writes w(w+1)/2 partials, of which the pairs of its system's own sys_w
+// columns hold values.
 cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramItem* items,
-                                 int nitems, const int* sys_w, int nsys, int* emax_all, double* partials,
+                                 int nitems, const int* sys_w, const int* emax_all, double* partials,
                                  cudaStream_t s);
+// The column exponents of every item's system (emax_all zeroed here), by a pass over Y.
+cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramItem* items, int nitems,
+                                      const int* sys_w, int nsys, int* emax_all, cudaStream_t s);
 // Recovery (eq. coords) on the tensor cores: x += Y x', r = Y r', p = Y p' in
 // one pass, with the Gram's digit split of Y (col_emax: the Gram's column
 // exponents, device int[kMaxW]) and coefficients (coords: device double[3w],
@@ -278,8 +350,10 @@ struct RowItem {
   int pad_;
 };
 // Matrix powers step j (monomial basis) of every system q with j < sys_steps[q].
+// emax_all (nsys x kMaxW ints, zeroed before step 0, or nullptr): the largest
+// biased exponent of every column formed, and of columns 0 and 1.
 cudaError_t launch_mpk_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
-                             cudaStream_t s);
+                             int* emax_all, cudaStream_t s);
 // b - A x of the systems with sel[q] != 0: into Y columns 1 and 0, or into column 2.
 cudaError_t launch_residual_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sel,
                                   int into_col2, cudaStream_t s);

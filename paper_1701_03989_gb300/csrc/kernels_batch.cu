@@ -21,38 +21,55 @@ __device__ __forceinline__ bool item_row(const RowItem* items, int64_t* row, int
 // Matrix powers step j in the monomial basis (theta = sigma = 0, gamma = 1;
 // eq. (polybasiscg)) for every system q with j < sys_steps[q]: column 2j+2 =
 // A column 2j and, while j + 1 < sbar_q, column 2j+3 = A column 2j+1, A = D + O.
-__global__ void __launch_bounds__(kRowItem) mpk_items_kernel(const SysDesc* __restrict__ descs,
-                                                             const RowItem* __restrict__ items,
-                                                             const int* __restrict__ sys_steps, int j) {
-  int64_t row;
-  int q;
-  if (!item_row(items, &row, &q)) return;
-  const int steps = sys_steps[q];
-  if (j >= steps) return;  // uniform over the CTA
-  const SysDesc d = descs[q];
-  const double* pj = d.Y + (int64_t)(2 * j) * d.ldY;
-  const double* rj = d.Y + (int64_t)(2 * j + 1) * d.ldY;
+//
+// One warp per 32-row slice and chain (P or R), 128 threads: the two chains of
+// two slices. A row's sum is one chain of dependent FMAs, 64 cycles each on
+// GB300, so a long row costs its length in latency however idle the GPU is:
+// the two chains on two warps halve that, and small CTAs spread a small
+// system over four times as many SMs. The second warp of a slice finds A in L1.
+// row_chain keeps two groups of A and one of gathers in flight; 8 CTAs per SM
+// (64 registers) beat 7 (72) by 4 % and 10 (48, spilling) by 18 %. FP64-bound:
+// 1.71M warp FMAs (10 systems, two banded of 117 and 129 entries a row) take
+// 111 us, 0.79 of the FP64 pipe. 32 systems of 1e3..1e5 rows, targets 1e-8 and
+// 1e-12: 236.4 -> 195.1 ms a batch with the exponents folded in below (one
+// thread per row with both chains, and a pass over the bases for the
+// exponents before).
+constexpr int kMpkRows = 64;                     // rows per CTA
+constexpr int kMpkSplit = kRowItem / kMpkRows;   // CTAs per row item
+__global__ void __launch_bounds__(2 * kMpkRows, 8) mpk_items_kernel(const SysDesc* __restrict__ descs,
+                                                                 const RowItem* __restrict__ items,
+                                                                 const int* __restrict__ sys_steps, int j,
+                                                                 int* __restrict__ emax_all) {
+  const RowItem it = items[blockIdx.x / kMpkSplit];
+  const int lane = threadIdx.x & 31, ch = (threadIdx.x >> 5) & 1;
+  const int first = (blockIdx.x % kMpkSplit) * kMpkRows + (int)(threadIdx.x >> 6) * kSlice;  // in the item
+  if (first >= it.nrows) return;  // uniform over the warp
+  const SysDesc d = descs[it.sys];
+  const int64_t row = (int64_t)it.row0 + first + lane;
+  const bool on = first + lane < it.nrows;
   const int64_t sl = row >> 5;
-  const int l = (int)(row & 31);
   const int64_t b = d.o_ptr[sl];
   const int width = (int)((d.o_ptr[sl + 1] - b) >> 5);
-  const double* v = d.o_val + b + l;
-  const int32_t* c = d.o_col + b + l;
-  const double dg = d.diag[row];
-  double tp = dg * pj[row];
-  if (j + 1 < steps) {
-    double tr = dg * rj[row];
-    for (int k = 0; k < width; ++k) {
-      const double a = __ldg(v + kSlice * k);
-      const int cc = __ldg(c + kSlice * k);
-      tp = fma(a, __ldg(pj + cc), tp);
-      tr = fma(a, __ldg(rj + cc), tr);
-    }
-    d.Y[(int64_t)(2 * j + 3) * d.ldY + row] = tr;
-  } else {
-    for (int k = 0; k < width; ++k) tp = fma(__ldg(v + kSlice * k), __ldg(pj + __ldg(c + kSlice * k)), tp);
+  const double dg = on ? d.diag[row] : 0.0;
+  const double* x = d.Y + (int64_t)(2 * j + ch) * d.ldY;
+  pdl_wait();  // the step before (its column of Y) and the lanes' tables
+  pdl_release();
+  const int steps = sys_steps[it.sys];
+  if (j + ch >= steps) return;  // no step j, or no R chain in the last one; uniform over the warp
+  const double xi = on ? x[row] : 0.0;
+  const double t = row_chain(d.o_val + b + lane, d.o_col + b + lane, width, x, dg * xi);
+  if (on) d.Y[(int64_t)(2 * j + 2 + ch) * d.ldY + row] = t;
+  if (!emax_all) return;
+  // the largest biased exponent of the column written (and, at step 0, of the
+  // input columns) for the tensor-core Gram: one reduction without return per
+  // warp, in place of another pass over the basis
+  int* em = emax_all + (int64_t)it.sys * kMaxW;
+  const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(t) : 0u);
+  if (lane == 0) atomicMax(em + 2 * j + 2 + ch, (int)e);
+  if (j == 0) {
+    const unsigned e0 = __reduce_max_sync(0xffffffffu, biased_exp(xi));
+    if (lane == 0) atomicMax(em + ch, (int)e0);
   }
-  d.Y[(int64_t)(2 * j + 2) * d.ldY + row] = tp;
 }
 
 // Residual of the systems with sel[q] != 0: into columns 1 (r) and 0 (p) of Y
@@ -111,6 +128,8 @@ __global__ void __launch_bounds__(kRowItem) recover_items_kernel(const SysDesc* 
                                                                  const RowItem* __restrict__ items,
                                                                  const int* __restrict__ sys_w,
                                                                  const double* __restrict__ coords, int64_t c_stride) {
+  pdl_wait();
+  pdl_release();
   int64_t row;
   int q;
   if (!item_row(items, &row, &q)) return;
@@ -157,10 +176,9 @@ cudaError_t launch_fill_uniform(double* v, int64_t count, uint64_t seed, cudaStr
 }
 
 cudaError_t launch_mpk_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
-                             cudaStream_t s) {
+                             int* emax_all, cudaStream_t s) {
   if (nitems < 1) return cudaSuccess;
-  mpk_items_kernel<<<nitems, kRowItem, 0, s>>>(descs, items, sys_steps, j);
-  return cudaGetLastError();
+  return launch_pdl(mpk_items_kernel, nitems * kMpkSplit, 2 * kMpkRows, s, descs, items, sys_steps, j, emax_all);
 }
 
 cudaError_t launch_residual_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sel,
@@ -183,8 +201,7 @@ cudaError_t launch_recover_items(int W, const SysDesc* descs, const RowItem* ite
   switch (W) {
 #define ASCG_RB(WW)                                                                             \
   case WW:                                                                                      \
-    recover_items_kernel<WW><<<nitems, kRowItem, 0, s>>>(descs, items, sys_w, coords, c_stride); \
-    return cudaGetLastError();
+    return launch_pdl(recover_items_kernel<WW>, nitems, kRowItem, s, descs, items, sys_w, coords, c_stride);
     ASCG_RB(3) ASCG_RB(5) ASCG_RB(7) ASCG_RB(9) ASCG_RB(11) ASCG_RB(13) ASCG_RB(15) ASCG_RB(17) ASCG_RB(19)
     ASCG_RB(21) ASCG_RB(23) ASCG_RB(25) ASCG_RB(27) ASCG_RB(29) ASCG_RB(31) ASCG_RB(33)
 #undef ASCG_RB

@@ -765,10 +765,9 @@ cudaError_t launch_block_ctrl_batch(const double* G, int64_t g_stride, const dou
                                     double* coords, int64_t c_stride, double* res_hist, int res_cap, double* ab_hist,
                                     int ab_cap, double* spec, unsigned* counters, cudaStream_t s) {
   if (count < 1 || max_sbar < 1) return cudaSuccess;
-  block_ctrl_kernel<<<dim3(adaptive ? max_sbar + 1 : 1, count), 128, 0, s>>>(
-      G, theta, sigma, gamma, st, coords, nullptr, res_hist, res_cap, ab_hist, ab_cap, g_stride, c_stride, spec,
-      counters);
-  return cudaGetLastError();
+  return launch_pdl_ex(block_ctrl_kernel, dim3(adaptive ? max_sbar + 1 : 1, count), dim3(128), 0, s, G, theta, sigma,
+                       gamma, st, coords, nullptr, res_hist, res_cap, ab_hist, ab_cap, g_stride, c_stride, spec,
+                       counters);
 }
 
 cudaError_t launch_block_advance(const BlockState* prev, BlockState* cur, int max_iters, cudaStream_t s) {

@@ -172,6 +172,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_items_kernel(const SysDe
                                                                       const int* __restrict__ sys_w,
                                                                       double* __restrict__ partials) {
   constexpr int NP = MOM ? kMomSlots : W * (W + 1) / 2;
+  pdl_wait();
+  pdl_release();
   const GramItem it = items[blockIdx.x];
   if (sys_w[it.sys] == 0) return;  // uniform over the CTA
   const SysDesc& d = descs[it.sys];
@@ -215,6 +217,8 @@ __global__ void __launch_bounds__(128) gram_items_moment_finalize_kernel(const d
                                                                          const int* __restrict__ sys_nitems,
                                                                          const int* __restrict__ sys_w,
                                                                          double* __restrict__ G, int64_t g_stride) {
+  pdl_wait();
+  pdl_release();
   const int q = blockIdx.x;
   const int w = sys_w[q];
   if (w == 0) return;
@@ -280,6 +284,8 @@ __global__ void __launch_bounds__(256) gram_items_finalize_kernel(int W, const d
                                                                   const int* __restrict__ sys_nitems,
                                                                   const int* __restrict__ sys_w, double* __restrict__ G,
                                                                   int64_t g_stride) {
+  pdl_wait();
+  pdl_release();
   const int q = blockIdx.x;
   const int w = sys_w[q];
   if (w == 0) return;
@@ -358,10 +364,8 @@ cudaError_t launch_gram_items(int W, const SysDesc* descs, const GramItem* items
 #define ASCG_GI(WW)                                                                              \
   case WW:                                                                                       \
     if (moments)                                                                                 \
-      gram_items_kernel<WW, true><<<grid, kGramThreads, 0, s>>>(descs, items, sys_w, partials);  \
-    else                                                                                         \
-      gram_items_kernel<WW><<<grid, kGramThreads, 0, s>>>(descs, items, sys_w, partials);        \
-    return cudaGetLastError();
+      return launch_pdl_ex(gram_items_kernel<WW, true>, grid, dim3(kGramThreads), 0, s, descs, items, sys_w, partials); \
+    return launch_pdl_ex(gram_items_kernel<WW>, grid, dim3(kGramThreads), 0, s, descs, items, sys_w, partials);
     ASCG_GI(3) ASCG_GI(5) ASCG_GI(7) ASCG_GI(9) ASCG_GI(11) ASCG_GI(13) ASCG_GI(15) ASCG_GI(17) ASCG_GI(19)
     ASCG_GI(21) ASCG_GI(23) ASCG_GI(25) ASCG_GI(27) ASCG_GI(29) ASCG_GI(31) ASCG_GI(33)
 #undef ASCG_GI
@@ -375,10 +379,9 @@ cudaError_t launch_gram_items_finalize(int W, const double* partials, const int*
                                        cudaStream_t s) {
   if (count < 1) return cudaSuccess;
   if (moments)
-    gram_items_moment_finalize_kernel<<<count, 128, 0, s>>>(partials, sys_item0, sys_nitems, sys_w, G, g_stride);
-  else
-    gram_items_finalize_kernel<<<count, 256, 0, s>>>(W, partials, sys_item0, sys_nitems, sys_w, G, g_stride);
-  return cudaGetLastError();
+    return launch_pdl(gram_items_moment_finalize_kernel, count, 128, s, partials, sys_item0, sys_nitems, sys_w, G,
+                      g_stride);
+  return launch_pdl(gram_items_finalize_kernel, count, 256, s, W, partials, sys_item0, sys_nitems, sys_w, G, g_stride);
 }
 
 cudaError_t launch_gram_moments(int64_t n, int w, const double* Y, int64_t ldY, double* partials, int* nparts,

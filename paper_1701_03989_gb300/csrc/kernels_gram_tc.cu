@@ -537,11 +537,12 @@ __device__ __forceinline__ void drain_quarter(uint32_t tq, int a, int w, uint32_
 
 // The Gram partial of the chunks ch = c_lo, c_lo + c_step, ... < c_hi of the
 // rows [row_base, row_base + n_local) of the tensor map's matrix (chunk ch
-// starts at row row_base + ch * kTChunk), with the column exponents col_emax,
-// written to out[w (w + 1) / 2]. Run by a whole CTA of kTcThreads. guard: the
+// starts at row row_base + ch * kTChunk), over the first w columns (the others
+// count as zero) with the column exponents col_emax, written to out[w_out
+// (w_out + 1) / 2], w <= w_out. Run by a whole CTA of kTcThreads. guard: the
 // wait limit, where a wait that ran out is reported, and the stall test's
 // stage (see TcGuard).
-__device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w, int64_t row_base, int64_t c_lo,
+__device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w_out, int w, int64_t row_base, int64_t c_lo,
                                              int64_t c_hi, int64_t c_step, int64_t n_local,
                                              const int* __restrict__ col_emax, double* __restrict__ out,
                                              const TcGuard guard) {
@@ -723,11 +724,11 @@ done:
   __syncthreads();
   const int ok = !*s_err;
   if (!ok && tid == 0 && guard.err) atomicExch(guard.err, (int)ASCG_ERR_TIMEOUT);
-  const int np = w * (w + 1) / 2;
+  const int np = w_out * (w_out + 1) / 2;
   for (int p = tid; p < np; p += kTcThreads) {
     int a = 0, rem = p;
-    while (rem >= w - a) {
-      rem -= w - a;
+    while (rem >= w_out - a) {
+      rem -= w_out - a;
       ++a;
     }
     const int b = a + rem;
@@ -756,7 +757,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   pdl_wait();
   pdl_release();
   if (guard.gate && !*guard.gate) return;  // uniform, before any barrier or tensor memory
-  gram_tc_body(&ymap, w, 0, blockIdx.x, (n + kTChunk - 1) / kTChunk, gridDim.x, n, col_emax,
+  gram_tc_body(&ymap, w, w, 0, blockIdx.x, (n + kTChunk - 1) / kTChunk, gridDim.x, n, col_emax,
                partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), guard);
 }
 
@@ -769,9 +770,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                          const int* __restrict__ sys_w, const int* __restrict__ emax_all,
                          double* __restrict__ partials) {
   const GramItem it = items[blockIdx.x];
-  if (sys_w[it.sys] == 0) return;  // uniform over the CTA, before any barrier
+  pdl_wait();
+  pdl_release();
+  const int wq = sys_w[it.sys];
+  if (wq == 0) return;  // uniform over the CTA, before any barrier
   const int64_t nch = it.nrows / kTChunk;
-  gram_tc_body(&ymap, w, it.row0, 0, nch, 1, nch * kTChunk, emax_all + (int64_t)it.sys * kTW,
+  gram_tc_body(&ymap, w, wq, it.row0, 0, nch, 1, nch * kTChunk, emax_all + (int64_t)it.sys * kTW,
                partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), TcGuard{kWaitLimit, -1, nullptr, nullptr});
 }
 
@@ -1244,7 +1248,7 @@ cudaError_t launch_gram_tc(int64_t n, int w, const double* Y, int64_t ldY, int* 
 }
 
 cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramItem* items,
-                                 int nitems, const int* sys_w, int nsys, int* emax_all, double* partials,
+                                 int nitems, const int* sys_w, const int* emax_all, double* partials,
                                  cudaStream_t s) {
   if (nitems < 1) return cudaSuccess;
   if (!gram_tc_applies(w) || !gram_tc_aligned(Y, ldY) || rows < 1 || rows > 0x7fffffffll || rows > ldY ||
@@ -1255,12 +1259,16 @@ cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t ro
   CUtensorMap map;
   e = encode_map(&map, Y, rows, w, ldY);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(emax_all, 0, sizeof(int) * kTW * nsys, s);
+  return launch_pdl_ex(gram_tc_items_kernel, dim3(nitems), dim3(kTcThreads), kTcSmem, s, map, w, items, sys_w, emax_all,
+                       partials);
+}
+
+cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramItem* items, int nitems,
+                                      const int* sys_w, int nsys, int* emax_all, cudaStream_t s) {
+  if (nitems < 1) return cudaSuccess;
+  const cudaError_t e = cudaMemsetAsync(emax_all, 0, sizeof(int) * kTW * nsys, s);
   if (e != cudaSuccess) return e;
   tc_items_exponent_kernel<<<nitems, 256, 0, s>>>(w, Y, ldY, items, sys_w, emax_all);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  gram_tc_items_kernel<<<nitems, kTcThreads, kTcSmem, s>>>(map, w, items, sys_w, emax_all, partials);
   return cudaGetLastError();
 }
 

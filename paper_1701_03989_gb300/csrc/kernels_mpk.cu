@@ -22,8 +22,6 @@ namespace ascg {
 
 namespace {
 
-__device__ __forceinline__ unsigned biased_exp(double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu; }
-
 // emax_part (optional, int[kMaxW][emax_ld]): lane 0 of each warp stores the
 // warp's largest biased exponent of each column written (and, for j = 0, of
 // the input columns 0 and 1) at emax_part[col * emax_ld + warp]; plain stores,

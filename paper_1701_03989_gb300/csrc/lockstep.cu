@@ -44,7 +44,7 @@ namespace ascg {
 
 // Defined in ascg_api.cu.
 ascg_status check_options(const ascg_options& o);
-ascg_status op_split_desc(ascg_op op, SysDesc* d, int* device);
+ascg_status op_split_desc(ascg_op op, SysDesc* d, int* device, double* row_len);
 
 namespace {
 
@@ -190,6 +190,7 @@ struct LaneSys {
   int64_t tag = 0;
   int64_t off = 0;   // first row of the system's range in the shared basis matrix
   size_t bytes = 0;  // basis bytes: (2 s_max + 1) 8 round_up(n, 1024)
+  double row_len = 0.0;  // mean entries per row of O, padding included
   int m = 0, kb = 0, s_prev = 0, nb_info = 0, wasted = 0, sbar = 0;
   double bnorm = 0.0, eps_star = 0.0, rel_upd = 0.0, rnorm0 = 0.0, rel_true = 0.0;
   bool active = false, done = false;
@@ -384,7 +385,7 @@ class Lockstep {
     if (!(eps_target >= 0.0 && std::isfinite(eps_target)))
       return lfail(ASCG_ERR_INVALID, "eps_target must be finite and >= 0");
     int dev = 0, cur = 0;
-    LS_TRY(op_split_desc(op, &out->d, &dev));
+    LS_TRY(op_split_desc(op, &out->d, &dev, &out->row_len));
     LS_CUDA(cudaGetDevice(&cur));
     if (dev != cur) return lfail(ASCG_ERR_INVALID, "every operator must live on the current device");
     out->op = op;
@@ -530,7 +531,7 @@ class Lockstep {
     const bool item_gram = n_tc < count_active();
     const bool tc_gram = n_tc > 0;
     const int Wb = 2 * max_sbar + 1;
-    int nl = max_sbar + 2 + (item_gram ? 2 : 0) + (tc_gram ? 3 : 0);
+    int nl = max_sbar + 2 + (item_gram ? 2 : 0) + (tc_gram ? 2 : 0);
     // The block's work: the state records in, the matrix powers steps, the
     // Gram (item launch and tensor-core lanes), the controller, the recovery,
     // the state records out. The host fills the pinned records before each
@@ -596,7 +597,10 @@ class Lockstep {
     int* d_tcn = d_int_ + kTcNItems * lanes_;
     const int nr = (int)ritems_.size(), ng = (int)gitems_.size(), nt = (int)titems_.size();
     const int Wb = 2 * max_sbar + 1;
-    for (int j = 0; j < max_sbar; ++j) LS_CUDA(launch_mpk_items(d_desc_, d_ritems_, nr, d_steps, j, s_));
+    // the steps record the column exponents that the tensor-core Gram needs
+    if (tc_gram) LS_CUDA(cudaMemsetAsync(d_emax_, 0, sizeof(int) * kMaxW * hi_, s_));
+    for (int j = 0; j < max_sbar; ++j)
+      LS_CUDA(launch_mpk_items(d_desc_, d_ritems_, nr, d_steps, j, tc_gram ? d_emax_ : nullptr, s_));
     if (item_gram) {
       // pair groups: enough CTAs to cover the SMs twice
       const int groups = std::max(1, std::min(16, (2 * gram_grid() + ng - 1) / std::max(ng, 1)));
@@ -604,7 +608,7 @@ class Lockstep {
       LS_CUDA(launch_gram_items_finalize(Wb, d_partials_, d_item0, d_nitems, d_wi, hi_, d_G_, kGStride, moments_, s_));
     }
     if (tc_gram) {  // every tensor-core lane in one launch over the shared basis matrix
-      LS_CUDA(launch_gram_tc_items(Wb, ybase_, yld_, yld_, d_titems_, nt, d_wtc, hi_, d_emax_, d_tpart_, s_));
+      LS_CUDA(launch_gram_tc_items(Wb, ybase_, yld_, yld_, d_titems_, nt, d_wtc, d_emax_, d_tpart_, s_));
       LS_CUDA(launch_gram_items_finalize(Wb, d_tpart_, d_tc0, d_tcn, d_wtc, hi_, d_G_, kGStride, false, s_));
     }
     LS_CUDA(launch_block_ctrl_batch(d_G_, kGStride, d_params_, d_params_ + kMaxS, d_params_ + 2 * kMaxS, d_bst_,
@@ -943,11 +947,20 @@ class Lockstep {
         h_tcn[q] = (int)titems_.size() - h_tc0[q];
       }
       const int64_t n = lane_[q].d.n;
-      for (int64_t r = 0; r < n; r += kRowItem)
-        ritems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(kRowItem, n - r), 0});
       const int64_t gr = gram_item_rows(n);
       for (int64_t r = 0; r < n; r += gr) gitems_.push_back(GramItem{r, (int)std::min<int64_t>(gr, n - r), q});
       h_nitems[q] = (int)gitems_.size() - h_item0[q];
+    }
+    // row items, the longest rows first: an item's time is its rows' length, so
+    // the last CTAs of a launch are the short ones
+    std::vector<int> order;
+    for (int q = 0; q < hi_; ++q)
+      if (used_[q]) order.push_back(q);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return lane_[a].row_len > lane_[b].row_len; });
+    for (int q : order) {
+      const int64_t n = lane_[q].d.n;
+      for (int64_t r = 0; r < n; r += kRowItem)
+        ritems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(kRowItem, n - r), 0});
     }
     LS_TRY(grow_items((int64_t)ritems_.size(), (int64_t)gitems_.size()));
     LS_TRY(grow_titems((int64_t)titems_.size()));
@@ -1497,6 +1510,8 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
     LS_CUDA(cudaMemcpyAsync(B.items, items.data(), sizeof(GramItem) * ng, cudaMemcpyHostToDevice, s));
     LS_CUDA(cudaMemcpyAsync(B.titems, titems.data(), sizeof(GramItem) * nt, cudaMemcpyHostToDevice, s));
     LS_CUDA(cudaMemcpyAsync(B.ints, ints, sizeof(ints), cudaMemcpyHostToDevice, s));
+    // a solve's exponents come from its matrix powers steps: not timed
+    LS_CUDA(launch_tc_items_exponents(w, B.Y, ld, B.titems, nt, B.ints, 1, B.emax, s));
     LS_CUDA(cudaStreamSynchronize(s));  // the host arrays above are locals
     const int groups = std::max(1, std::min(16, (2 * gram_grid() + ng - 1) / ng));
     std::vector<float> a(kReps), b(kReps);
@@ -1510,7 +1525,7 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
       LS_CUDA(cudaEventElapsedTime(&ms, B.e0, B.e1));
       if (rep > 0) a[rep - 1] = ms;
       LS_CUDA(cudaEventRecord(B.e0, s));
-      LS_CUDA(launch_gram_tc_items(w, B.Y, ld, ld, B.titems, nt, B.ints, 1, B.emax, B.tpart, s));
+      LS_CUDA(launch_gram_tc_items(w, B.Y, ld, ld, B.titems, nt, B.ints, B.emax, B.tpart, s));
       LS_CUDA(launch_gram_items_finalize(w, B.tpart, B.ints + 3, B.ints + 4, B.ints, 1, B.G, kMaxW * kMaxW, false, s));
       LS_CUDA(cudaEventRecord(B.e1, s));
       LS_CUDA(cudaEventSynchronize(B.e1));
