@@ -443,7 +443,7 @@ typedef struct {
  * 8 bytes of Gram partials per FP64 Gram item (1024 to 8192 rows, about n/16
  * as a power of two) and per tensor-core Gram item (8192 rows). The basis
  * matrix takes the budget less the partials' share and is allocated here;
- * the partial and row-table buffers (about 16 bytes per 256 rows) grow on
+ * the partial and row-table buffers (at most 80 bytes per 256 rows) grow on
  * demand within that share.
  * max_systems: most systems running at once (1 .. 2^20). cuda_stream: the
  * caller's stream, which orders submissions after the caller's work; the

@@ -111,6 +111,18 @@ __device__ __forceinline__ double row_chain(const double* __restrict__ v, const 
   return t;
 }
 
+// Whether a matrix powers step over n rows of row_len entries on average runs
+// each chain (P, R) in a warp of its own, or both in one thread. One warp per
+// chain halves a row's dependent FMAs and keeps more loads in flight, but
+// reads A twice (through L1) and takes twice the warps. Measured, us per
+// step, both in one thread / a warp each: 2D n = 4096 3.3 / 2.6, 65536 3.84 /
+// 3.83, 262144 8.4 / 8.8, 1048576 21.8 / 33.6; banded of 128 entries a row n
+// = 20000 48.4 / 14.8, 400000 185 / 173; of 16, n = 200000 17.1 / 14.6, n =
+// 400000 27.5 / 28.9; of 24, n = 400000 39.1 / 40.6, of 48 72.7 / 70.7.
+inline bool mpk_by_chain(int64_t n, double row_len) {
+  return n <= 65536 || row_len >= 32.0 || (row_len >= 12.0 && n <= 262144);
+}
+
 // Raises a kernel's dynamic shared-memory limit to `bytes` on the current
 // device, once per device (devices 0..63; others every call). The device's
 // flag is set only after the attribute call succeeded, so a caller that sees
@@ -347,8 +359,10 @@ struct RowItem {
   int sys;
   int row0;
   int nrows;
-  int pad_;
+  int by_chain;  // matrix powers items: see mpk_by_chain
 };
+// Rows of a matrix powers item: one CTA of 128 threads.
+constexpr int kMpkChainRows = 64, kMpkBothRows = 128;
 // Matrix powers step j (monomial basis) of every system q with j < sys_steps[q].
 // emax_all (nsys x kMaxW ints, zeroed before step 0, or nullptr): the largest
 // biased exponent of every column formed, and of columns 0 and 1.

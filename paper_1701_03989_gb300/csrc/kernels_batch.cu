@@ -22,53 +22,90 @@ __device__ __forceinline__ bool item_row(const RowItem* items, int64_t* row, int
 // eq. (polybasiscg)) for every system q with j < sys_steps[q]: column 2j+2 =
 // A column 2j and, while j + 1 < sbar_q, column 2j+3 = A column 2j+1, A = D + O.
 //
-// One warp per 32-row slice and chain (P or R), 128 threads: the two chains of
-// two slices. A row's sum is one chain of dependent FMAs, 64 cycles each on
-// GB300, so a long row costs its length in latency however idle the GPU is:
-// the two chains on two warps halve that, and small CTAs spread a small
-// system over four times as many SMs. The second warp of a slice finds A in L1.
-// row_chain keeps two groups of A and one of gathers in flight; 8 CTAs per SM
-// (64 registers) beat 7 (72) by 4 % and 10 (48, spilling) by 18 %. FP64-bound:
-// 1.71M warp FMAs (10 systems, two banded of 117 and 129 entries a row) take
-// 111 us, 0.79 of the FP64 pipe. 32 systems of 1e3..1e5 rows, targets 1e-8 and
-// 1e-12: 236.4 -> 195.1 ms a batch with the exponents folded in below (one
-// thread per row with both chains, and a pass over the bases for the
-// exponents before).
-constexpr int kMpkRows = 64;                     // rows per CTA
-constexpr int kMpkSplit = kRowItem / kMpkRows;   // CTAs per row item
-__global__ void __launch_bounds__(2 * kMpkRows, 8) mpk_items_kernel(const SysDesc* __restrict__ descs,
-                                                                 const RowItem* __restrict__ items,
-                                                                 const int* __restrict__ sys_steps, int j,
-                                                                 int* __restrict__ emax_all) {
-  const RowItem it = items[blockIdx.x / kMpkSplit];
-  const int lane = threadIdx.x & 31, ch = (threadIdx.x >> 5) & 1;
-  const int first = (blockIdx.x % kMpkSplit) * kMpkRows + (int)(threadIdx.x >> 6) * kSlice;  // in the item
-  if (first >= it.nrows) return;  // uniform over the warp
+// An item is one CTA of 128 threads. by_chain (mpk_by_chain): one warp per
+// 32-row slice and chain (P or R), the two chains of two slices; the second
+// warp of a slice finds A in L1. A row's sum is one chain of dependent FMAs,
+// 64 cycles each on GB300, so a long row costs its length in latency however
+// idle the GPU is: the two chains on two warps halve that, and small CTAs
+// spread a small system over more SMs. row_chain keeps two groups of A and one
+// of gathers in flight. Otherwise: 128 rows, both chains in one thread.
+// 8 CTAs per SM (64 registers) beat 7 (72) by 4 % and 10 (48, spilling) by
+// 18 %. FP64-bound: 1.71M warp FMAs (10 systems, two banded of 117 and 129
+// entries a row) take 111 us, 0.79 of the FP64 pipe. 32 systems of 1e3..1e5
+// rows, targets 1e-8 and 1e-12: 236.4 -> 195.1 ms a batch with the exponents
+// folded in below (one thread per row with both chains in 256-row CTAs, and a
+// pass over the bases for the exponents before).
+__global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __restrict__ descs,
+                                                           const RowItem* __restrict__ items,
+                                                           const int* __restrict__ sys_steps, int j,
+                                                           int* __restrict__ emax_all) {
+  const RowItem it = items[blockIdx.x];
   const SysDesc d = descs[it.sys];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ch = it.by_chain ? warp & 1 : 0;
+  const int first = kSlice * (it.by_chain ? warp >> 1 : warp);
+  const bool any = first < it.nrows, on = first + lane < it.nrows;
   const int64_t row = (int64_t)it.row0 + first + lane;
-  const bool on = first + lane < it.nrows;
-  const int64_t sl = row >> 5;
-  const int64_t b = d.o_ptr[sl];
-  const int width = (int)((d.o_ptr[sl + 1] - b) >> 5);
-  const double dg = on ? d.diag[row] : 0.0;
-  const double* x = d.Y + (int64_t)(2 * j + ch) * d.ldY;
+  int64_t b = 0;
+  int width = 0;
+  double dg = 0.0;
+  if (any) {
+    const int64_t sl = row >> 5;
+    b = d.o_ptr[sl];
+    width = (int)((d.o_ptr[sl + 1] - b) >> 5);
+    if (on) dg = d.diag[row];
+  }
   pdl_wait();  // the step before (its column of Y) and the lanes' tables
   pdl_release();
   const int steps = sys_steps[it.sys];
-  if (j + ch >= steps) return;  // no step j, or no R chain in the last one; uniform over the warp
+  if (!any || j + ch >= steps) return;  // uniform over the warp: no step j, or no R chain in the last one
+  const double* x = d.Y + (int64_t)(2 * j + ch) * d.ldY;
+  double* y = d.Y + (int64_t)(2 * j + 2 + ch) * d.ldY;
+  const double* v = d.o_val + b + lane;
+  const int32_t* c = d.o_col + b + lane;
+  const bool both = !it.by_chain && j + 1 < steps;
   const double xi = on ? x[row] : 0.0;
-  const double t = row_chain(d.o_val + b + lane, d.o_col + b + lane, width, x, dg * xi);
-  if (on) d.Y[(int64_t)(2 * j + 2 + ch) * d.ldY + row] = t;
+  double t = dg * xi, xr = 0.0, tr = 0.0;
+  if (!both) {
+    t = row_chain(v, c, width, x, t);
+  } else {
+    const double* r = x + d.ldY;
+    xr = on ? r[row] : 0.0;
+    tr = dg * xr;
+    int k = 0;
+    for (; k + 2 <= width; k += 2) {
+      const int c0 = __ldg(c + kSlice * k), c1 = __ldg(c + kSlice * (k + 1));
+      const double a0 = __ldg(v + kSlice * k), a1 = __ldg(v + kSlice * (k + 1));
+      const double p0 = __ldg(x + c0), p1 = __ldg(x + c1);
+      const double r0 = __ldg(r + c0), r1 = __ldg(r + c1);
+      t = fma(a0, p0, t);
+      tr = fma(a0, r0, tr);
+      t = fma(a1, p1, t);
+      tr = fma(a1, r1, tr);
+    }
+    if (k < width) {
+      const double a = __ldg(v + kSlice * k);
+      const int cc = __ldg(c + kSlice * k);
+      t = fma(a, __ldg(x + cc), t);
+      tr = fma(a, __ldg(r + cc), tr);
+    }
+    if (on) y[d.ldY + row] = tr;
+  }
+  if (on) y[row] = t;
   if (!emax_all) return;
-  // the largest biased exponent of the column written (and, at step 0, of the
+  // the largest biased exponent of the columns written (and, at step 0, of the
   // input columns) for the tensor-core Gram: one reduction without return per
-  // warp, in place of another pass over the basis
-  int* em = emax_all + (int64_t)it.sys * kMaxW;
-  const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(t) : 0u);
-  if (lane == 0) atomicMax(em + 2 * j + 2 + ch, (int)e);
+  // warp and column, in place of another pass over the basis
+  int* em = emax_all + (int64_t)it.sys * kMaxW + ch;
+  const auto record = [&](int col, double val) {
+    const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(val) : 0u);
+    if (lane == 0) atomicMax(em + col, (int)e);
+  };
+  record(2 * j + 2, t);
+  if (both) record(2 * j + 3, tr);
   if (j == 0) {
-    const unsigned e0 = __reduce_max_sync(0xffffffffu, biased_exp(xi));
-    if (lane == 0) atomicMax(em + ch, (int)e0);
+    record(0, xi);
+    if (both) record(1, xr);
   }
 }
 
@@ -178,7 +215,7 @@ cudaError_t launch_fill_uniform(double* v, int64_t count, uint64_t seed, cudaStr
 cudaError_t launch_mpk_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
                              int* emax_all, cudaStream_t s) {
   if (nitems < 1) return cudaSuccess;
-  return launch_pdl(mpk_items_kernel, nitems * kMpkSplit, 2 * kMpkRows, s, descs, items, sys_steps, j, emax_all);
+  return launch_pdl(mpk_items_kernel, nitems, 128, s, descs, items, sys_steps, j, emax_all);
 }
 
 cudaError_t launch_residual_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sel,

@@ -128,6 +128,60 @@ __global__ void __launch_bounds__(kSpmvRows, 6)
   }
 }
 
+// The same step, one warp per slice and chain: 128 threads take the two chains
+// of two slices, or (R = false) the P chain of four. The same sums in the same
+// order, so the same bits.
+template <int SIG, bool R>
+__global__ void __launch_bounds__(128, 8)
+    mpk_chain_step_kernel(DevSell O, const double* __restrict__ oval, const double* __restrict__ dtil, double sig,
+                          double* __restrict__ Y, int64_t ldY, int j, int* emax_part, int64_t emax_ld,
+                          const int* __restrict__ gate) {
+  constexpr int kSlices = R ? 2 : 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ch = R ? warp & 1 : 0;
+  const int64_t sl = (int64_t)blockIdx.x * kSlices + (R ? warp >> 1 : warp);
+  const int64_t row = sl * kSlice + lane;
+  const bool on = row < O.n, any = sl * kSlice < O.n;
+  // The operator is constant during a block: its row is looked up before the
+  // wait on the previous step. (Before step 0 the operator itself may have
+  // been written by the kernel just before, the folding of the coefficients.)
+  if (j == 0) pdl_wait();
+  int64_t b = 0;
+  int width = 0;
+  double dt = 0.0;
+  if (any) {
+    b = O.ptr[sl];
+    width = (int)((O.ptr[sl + 1] - b) >> 5);
+    if (on) dt = dtil[row];
+  }
+  if (j > 0) pdl_wait();
+  pdl_release();
+  if (!any || (gate && !*gate)) return;  // uniform over the warp
+  const double* x = Y + (int64_t)(2 * j + ch) * ldY;
+  const double xi = on ? x[row] : 0.0;
+  double t;
+  if (SIG == 0) {
+    t = dt * xi;
+  } else {
+    const double z = on ? Y[(int64_t)(2 * j - 2 + ch) * ldY + row] : 0.0;
+    t = fma(dt, xi, SIG == 1 ? -z : -sig * z);
+  }
+  t = row_chain(oval + b + lane, O.col + b + lane, width, x, t);
+  if (on) Y[(int64_t)(2 * j + 2 + ch) * ldY + row] = t;
+  if (!emax_part) return;
+  const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(t) : 0u);
+  if (lane == 0) emax_part[(int64_t)(2 * j + 2 + ch) * emax_ld + sl] = (int)e;
+  if (j == 0) {
+    // columns 0 and 1; with one step (no R chain) the P warps record both
+    const unsigned e0 = __reduce_max_sync(0xffffffffu, on ? biased_exp(xi) : 0u);
+    if (lane == 0) emax_part[(int64_t)ch * emax_ld + sl] = (int)e0;
+    if (!R) {
+      const unsigned e1 = __reduce_max_sync(0xffffffffu, on ? biased_exp(Y[ldY + row]) : 0u);
+      if (lane == 0) emax_part[emax_ld + sl] = (int)e1;
+    }
+  }
+}
+
 // col_emax[c] = max over the warp entries of column c: one CTA of 1024 threads
 // per column, 16-byte loads, four in flight per thread. emax_ld is a multiple
 // of 4 and entries past the warp count are zero.
@@ -309,11 +363,15 @@ cudaError_t recover_split_w(int64_t n, const double* Y, int64_t ldY, const doubl
 cudaError_t launch_mpk_split_step(const DevSplit& O, const StepOp& op, double* Y, int64_t ldY, int j, int do_p,
                                   int do_r, int* emax_part, int64_t emax_ld, cudaStream_t s, const int* gate) {
   if (!do_p) return cudaErrorInvalidValue;  // every step forms the P column
-  const int g = (int)((O.O.n + kSpmvRows - 1) / kSpmvRows);
   const int sig_mode = (op.sig == 0.0 || j < 1) ? 0 : (op.sig == 1.0 ? 1 : 2);
-#define ASCG_MPK(S, R)                                                                                        \
-  return launch_pdl(mpk_split_step_kernel<S, R>, g, kSpmvRows, s, O.O, op.oval, op.dtil, op.sig, Y, ldY, j, emax_part, \
-                    emax_ld, gate)
+  const bool chains = mpk_by_chain(O.O.n, (double)O.o_len / (double)O.O.n);
+  const int64_t rows = chains ? (do_r ? 64 : 128) : kSpmvRows;
+  const int g = (int)((O.O.n + rows - 1) / rows);
+#define ASCG_MPK(S, R)                                                                                              \
+  return chains ? launch_pdl(mpk_chain_step_kernel<S, R>, g, 128, s, O.O, op.oval, op.dtil, op.sig, Y, ldY, j,      \
+                             emax_part, emax_ld, gate)                                                              \
+                : launch_pdl(mpk_split_step_kernel<S, R>, g, kSpmvRows, s, O.O, op.oval, op.dtil, op.sig, Y, ldY, j, \
+                             emax_part, emax_ld, gate)
   if (do_r) {
     if (sig_mode == 0) ASCG_MPK(0, true);
     else if (sig_mode == 1) ASCG_MPK(1, true);
@@ -324,7 +382,6 @@ cudaError_t launch_mpk_split_step(const DevSplit& O, const StepOp& op, double* Y
     else ASCG_MPK(2, false);
   }
 #undef ASCG_MPK
-  return cudaGetLastError();
 }
 
 cudaError_t launch_emax_reduce(const int* emax_part, int64_t emax_ld, int64_t n, int w, int* col_emax,

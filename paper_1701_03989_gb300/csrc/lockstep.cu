@@ -600,7 +600,7 @@ class Lockstep {
     // the steps record the column exponents that the tensor-core Gram needs
     if (tc_gram) LS_CUDA(cudaMemsetAsync(d_emax_, 0, sizeof(int) * kMaxW * hi_, s_));
     for (int j = 0; j < max_sbar; ++j)
-      LS_CUDA(launch_mpk_items(d_desc_, d_ritems_, nr, d_steps, j, tc_gram ? d_emax_ : nullptr, s_));
+      LS_CUDA(launch_mpk_items(d_desc_, d_mitems_, (int)mitems_.size(), d_steps, j, tc_gram ? d_emax_ : nullptr, s_));
     if (item_gram) {
       // pair groups: enough CTAs to cover the SMs twice
       const int groups = std::max(1, std::min(16, (2 * gram_grid() + ng - 1) / std::max(ng, 1)));
@@ -904,6 +904,16 @@ class Lockstep {
     return ASCG_OK;
   }
 
+  ascg_status grow_mitems(int64_t mitems) {
+    if (mitems > mcap_items_) {
+      LS_CUDA(cudaStreamSynchronize(s_));
+      dfree(d_mitems_);
+      mcap_items_ = std::max<int64_t>(mitems, 2 * mcap_items_);
+      LS_TRY(dalloc(&d_mitems_, (size_t)mcap_items_));
+    }
+    return ASCG_OK;
+  }
+
   ascg_status grow_items(int64_t ritems, int64_t gitems) {
     if (ritems > rcap_items_) {
       LS_CUDA(cudaStreamSynchronize(s_));
@@ -928,6 +938,7 @@ class Lockstep {
   // before it changes the lanes again).
   ascg_status rebuild_tables() {
     ritems_.clear();
+    mitems_.clear();
     gitems_.clear();
     titems_.clear();
     int* h_item0 = h_int_ + kItem0 * lanes_;
@@ -961,13 +972,20 @@ class Lockstep {
       const int64_t n = lane_[q].d.n;
       for (int64_t r = 0; r < n; r += kRowItem)
         ritems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(kRowItem, n - r), 0});
+      const bool by_chain = mpk_by_chain(n, lane_[q].row_len);
+      const int64_t mr = by_chain ? kMpkChainRows : kMpkBothRows;
+      for (int64_t r = 0; r < n; r += mr)
+        mitems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(mr, n - r), by_chain ? 1 : 0});
     }
     LS_TRY(grow_items((int64_t)ritems_.size(), (int64_t)gitems_.size()));
+    LS_TRY(grow_mitems((int64_t)mitems_.size()));
     LS_TRY(grow_titems((int64_t)titems_.size()));
     if (!titems_.empty())
       LS_CUDA(cudaMemcpyAsync(d_titems_, titems_.data(), sizeof(GramItem) * titems_.size(), cudaMemcpyHostToDevice, s_));
     if (!ritems_.empty())
       LS_CUDA(cudaMemcpyAsync(d_ritems_, ritems_.data(), sizeof(RowItem) * ritems_.size(), cudaMemcpyHostToDevice, s_));
+    if (!mitems_.empty())
+      LS_CUDA(cudaMemcpyAsync(d_mitems_, mitems_.data(), sizeof(RowItem) * mitems_.size(), cudaMemcpyHostToDevice, s_));
     if (!gitems_.empty())
       LS_CUDA(cudaMemcpyAsync(d_gitems_, gitems_.data(), sizeof(GramItem) * gitems_.size(), cudaMemcpyHostToDevice, s_));
     if (hi_ > 0) {
@@ -992,7 +1010,7 @@ class Lockstep {
   void release() {
     drop_graphs();
     dfree(d_desc_); dfree(d_bst_); dfree(d_G_); dfree(d_coords_); dfree(d_int_); dfree(d_sums_); dfree(d_params_);
-    dfree(d_res_hist_); dfree(d_ab_hist_); dfree(d_ritems_); dfree(d_gitems_); dfree(d_partials_);
+    dfree(d_res_hist_); dfree(d_ab_hist_); dfree(d_ritems_); dfree(d_mitems_); dfree(d_gitems_); dfree(d_partials_);
     dfree(d_titems_); dfree(d_tpart_); dfree(d_emax_); dfree(d_spec_); dfree(d_tickets_);
     dfree(d_run_); dfree(d_iter_); dfree(d_seq_);
     hfree(h_desc_); hfree(h_bst_); hfree(h_int_); hfree(h_sums_);
@@ -1014,7 +1032,8 @@ class Lockstep {
   std::vector<RowItem> ritems_;
   std::vector<GramItem> gitems_;
   std::vector<GramItem> titems_;
-  int64_t rcap_items_ = 0, gcap_items_ = 0;
+  std::vector<RowItem> mitems_;  // matrix powers items
+  int64_t rcap_items_ = 0, gcap_items_ = 0, mcap_items_ = 0;
   SysDesc* d_desc_ = nullptr;
   BlockState* d_bst_ = nullptr;
   double* d_G_ = nullptr;
@@ -1025,6 +1044,7 @@ class Lockstep {
   double* d_res_hist_ = nullptr;
   double* d_ab_hist_ = nullptr;
   RowItem* d_ritems_ = nullptr;
+  RowItem* d_mitems_ = nullptr;
   GramItem* d_gitems_ = nullptr;
   double* d_partials_ = nullptr;
   double* ybase_ = nullptr;  // the shared basis matrix (leading dimension yld_)
