@@ -16,9 +16,12 @@
  *  - "device" pointers are CUDA device memory of the current device. "host"
  *    pointers are ordinary (pageable or pinned) host memory.
  *  - Calls are ordered on the given CUDA stream (NULL = the legacy default
- *    stream). Calls that report results on the host or free temporaries
- *    (ascg_solve*, ascg_block_step, ascg_newton_shifts, ascg_matrix_powers,
- *    ascg_gram) synchronise that stream before they return. The others return
+ *    stream). Calls that report results on the host or use scratch of the
+ *    library's (ascg_solve*, ascg_block_step, ascg_newton_shifts,
+ *    ascg_matrix_powers, ascg_gram*, ascg_recover_tc; not ascg_gram_noalloc)
+ *    synchronise that stream before they return. Scratch blocks (1 MB of
+ *    device memory) are kept between calls, at most four idle ones per
+ *    process, until the last operator is destroyed. The others return
  *    as soon as their work is enqueued.
  *  - Sizes are int64_t. Matrices have n >= 1 rows and nnz < 2^31 nonzeros.
  *  - All arithmetic is IEEE double. eps = 2^-53.
@@ -353,7 +356,7 @@ ascg_status ascg_recover(int64_t n, int w, const double* Y, int64_t ldY, const d
  *  - n, w, Y, ldY, coords, x, r, p: as for ascg_recover, with
  *    9 <= w <= 33, Y 16-byte aligned and ldY even (else ASCG_ERR_INVALID),
  *    n <= 2^31 - 1. r and p may alias columns 1 and 0 of Y.
- *  - Allocates 136 bytes of device memory for the column exponents and
+ *  - Takes 136 bytes of the library's scratch for the column exponents and
  *    synchronises the stream. ASCG_ERR_TIMEOUT: a bounded wait of the kernel
  *    ran out (the outputs are then incomplete). */
 ascg_status ascg_recover_tc(int64_t n, int w, const double* Y, int64_t ldY, const double* coords,

@@ -9,7 +9,9 @@
 // next block's basis size sbar_k = min(s_{k-1} + f, s_max) depends on it.
 #include <cmath>
 #include <cstdio>
+#include <cstddef>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -59,6 +61,107 @@ void dev_free(T*& p) {
   p = nullptr;
 }
 
+// Scratch of the single-step calls (ascg_gram, ascg_block_step, ...), which
+// used to allocate and free on each call: 130 of the 162 us of a 1024-row Gram
+// went to cudaMalloc and cudaFree. A call takes a block (device memory, and a
+// page of pinned host memory) for itself and gives it back after it has
+// synchronised its stream, so a block is never shared between threads or
+// streams. At most kKeepBlocks idle blocks are kept per process; they are
+// freed when the last operator is destroyed.
+constexpr size_t kScratchBytes = (size_t)1 << 20, kScratchHost = 4096;
+constexpr size_t kKeepBlocks = 4;
+struct ScratchBlock {
+  int dev = -1;
+  size_t bytes = 0;
+  unsigned char* d = nullptr;
+  unsigned char* h = nullptr;
+};
+struct ScratchPool {
+  std::mutex mu;
+  std::vector<ScratchBlock> idle;
+  int ops = 0;  // operators alive
+};
+ScratchPool& scratch_pool() {
+  static ScratchPool* p = new ScratchPool();  // never destroyed: calls may outlive static destruction
+  return *p;
+}
+void scratch_free(ScratchBlock& b) {
+  if (b.d) cudaFree(b.d);
+  if (b.h) cudaFreeHost(b.h);
+  b = ScratchBlock();
+}
+void scratch_op_created() {
+  ScratchPool& p = scratch_pool();
+  std::lock_guard<std::mutex> lock(p.mu);
+  ++p.ops;
+}
+void scratch_op_destroyed() {
+  ScratchPool& p = scratch_pool();
+  std::vector<ScratchBlock> drop;
+  {
+    std::lock_guard<std::mutex> lock(p.mu);
+    if (--p.ops == 0) drop.swap(p.idle);
+  }
+  for (ScratchBlock& b : drop) scratch_free(b);
+}
+
+// One call's scratch, carved front to back in 256-byte steps.
+class Scratch {
+ public:
+  ~Scratch() {
+    if (!b_.d) return;
+    ScratchPool& p = scratch_pool();
+    if (clean_) {
+      std::lock_guard<std::mutex> lock(p.mu);
+      if (p.idle.size() < kKeepBlocks) {
+        p.idle.push_back(b_);
+        b_ = ScratchBlock();
+      }
+    }
+    scratch_free(b_);  // waits for the device where the call could not
+  }
+  ascg_status open(size_t bytes) {
+    int dev = 0;
+    ASCG_CUDA(cudaGetDevice(&dev));
+    ScratchPool& p = scratch_pool();
+    {
+      std::lock_guard<std::mutex> lock(p.mu);
+      for (size_t i = p.idle.size(); i-- > 0;)
+        if (p.idle[i].dev == dev && p.idle[i].bytes >= bytes) {
+          b_ = p.idle[i];
+          p.idle.erase(p.idle.begin() + (std::ptrdiff_t)i);
+          return ASCG_OK;
+        }
+    }
+    b_.dev = dev;
+    b_.bytes = bytes > kScratchBytes ? bytes : kScratchBytes;
+    cudaError_t e = cudaMalloc((void**)&b_.d, b_.bytes);
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&b_.h, kScratchHost);
+    if (e != cudaSuccess) {
+      scratch_free(b_);
+      cudaGetLastError();
+      return fail(ASCG_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
+    return ASCG_OK;
+  }
+  static size_t round(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
+  template <class T>
+  T* take(size_t count) {
+    T* r = reinterpret_cast<T*>(b_.d + used_);
+    used_ += round(count * sizeof(T));
+    return r;
+  }
+  template <class T>
+  T* host() const { return reinterpret_cast<T*>(b_.h); }
+  // Nothing enqueued by the call is still running: the block can be reused.
+  void synced() { clean_ = true; }
+
+ private:
+  ScratchBlock b_;
+  size_t used_ = 0;
+  bool clean_ = false;
+};
+
 // Records of the blocks in flight: block j uses slot j % kRing.
 constexpr int kRing = 4;
 
@@ -90,7 +193,8 @@ struct Workspace {
   int res_cap = 0;
   double* ab_hist = nullptr;  // alpha[ab_cap], beta[ab_cap]
   int ab_cap = 0;
-  double* dtils = nullptr;      // folded diagonals Dt_j, kMaxS x n
+  double* dtils = nullptr;      // folded diagonals Dt_j, dt_rows x n
+  int dt_rows = 0;
   double* oscaled[2] = {};      // O / gamma for up to two gamma != 1
   bool steps_ready = false;
   // pinned host mirrors
@@ -127,7 +231,7 @@ struct Workspace {
     side = nullptr;
     ev_gram = nullptr;
     ev_x[0] = ev_x[1] = nullptr;
-    n = 0; wcols = 0; ldY = 0; partials_cap = 0; res_cap = 0; ab_cap = 0; emax_ld = 0;
+    n = 0; wcols = 0; ldY = 0; partials_cap = 0; res_cap = 0; ab_cap = 0; emax_ld = 0; dt_rows = 0;
   }
 };
 
@@ -277,11 +381,6 @@ ascg_status ensure(ascg_op op, int wcols, int res_cap) {
     ASCG_TRY(dev_alloc(&w.emax_part, (size_t)kMaxW * w.emax_ld));
     ASCG_CUDA(cudaMemset(w.emax_part, 0, sizeof(int) * kMaxW * w.emax_ld));
   }
-  if (wcols > 2 && !w.dtils) {
-    ASCG_TRY(dev_alloc(&w.dtils, (size_t)kMaxS * n));
-    ASCG_TRY(dev_alloc(&w.oscaled[0], (size_t)op->o_len));
-    ASCG_TRY(dev_alloc(&w.oscaled[1], (size_t)op->o_len));
-  }
   if (w.res_cap < res_cap) {
     dev_free(w.res_hist); dev_free(w.ab_hist);
     ASCG_TRY(dev_alloc(&w.res_hist, (size_t)res_cap));
@@ -398,51 +497,64 @@ void basis_params(const ascg_options& o, double* th, double* sg, double* gm) {
   }
 }
 
-// Runs classical CG iterations (Alg. 1) on the device until the CG state says
-// done. x, r, p, q are device vectors. Returns the iterations done by this call.
 // Per-step operators of the matrix powers recurrence with theta, sigma and gamma
-// folded in (see StepOp). dtils: n x s doubles; oscaled: two arrays of o_len
-// doubles (used when gamma != 1; at most two distinct gamma values, which covers
-// the monomial, Chebyshev and Newton bases).
-ascg_status prepare_steps(ascg_op op, const double* th, const double* sg, const double* gm, int s, double* dtils,
-                          double* const oscaled[2], StepOp* out, cudaStream_t st, int* launches) {
+// folded in (see StepOp), in the operator's workspace: one vector Dt per
+// distinct (theta, gamma) and one scaled O per distinct gamma != 1 (at most
+// two, which covers the monomial, Chebyshev and Newton bases).
+ascg_status prepare_steps(ascg_op op, const double* th, const double* sg, const double* gm, int s, StepOp* out,
+                          cudaStream_t st, int* launches) {
+  Workspace& w = op->ws;
   double gam_of[2] = {0.0, 0.0};
-  int ng = 0;
+  int ng = 0, nd = 0;
+  int o_slot[kMaxS], d_row[kMaxS];  // -1: O and D themselves
   for (int j = 0; j < s; ++j) {
     if (!(gm[j] != 0.0) || !std::isfinite(gm[j]) || !std::isfinite(th[j]))
       return fail(ASCG_ERR_INVALID, "basis coefficients must be finite with gamma != 0");
-    const double inv = 1.0 / gm[j];
-    const double* ov = op->o_val;
+    o_slot[j] = -1;
     if (gm[j] != 1.0) {
-      int slot = -1;
       for (int q = 0; q < ng; ++q)
-        if (gam_of[q] == gm[j]) slot = q;
-      if (slot < 0) {
+        if (gam_of[q] == gm[j]) o_slot[j] = q;
+      if (o_slot[j] < 0) {
         if (ng == 2) return fail(ASCG_ERR_INVALID, "at most two distinct gamma != 1 are supported");
-        slot = ng++;
-        gam_of[slot] = gm[j];
-        ASCG_CUDA(launch_shift_scale(op->o_val, op->o_len, 0.0, inv, oscaled[slot], st));
-        ++*launches;
+        o_slot[j] = ng;
+        gam_of[ng++] = gm[j];
       }
-      ov = oscaled[slot];
     }
-    const double* dt = nullptr;
-    if (th[j] == 0.0 && gm[j] == 1.0) dt = op->diag;
-    for (int q = 0; q < j && !dt; ++q)
-      if (th[q] == th[j] && gm[q] == gm[j]) dt = out[q].dtil;
-    if (!dt) {
-      double* dst = dtils + (int64_t)j * op->n;
-      ASCG_CUDA(launch_shift_scale(op->diag, op->n, th[j], inv, dst, st));
+    d_row[j] = -2;
+    if (th[j] == 0.0 && gm[j] == 1.0) d_row[j] = -1;
+    for (int q = 0; q < j && d_row[j] == -2; ++q)
+      if (th[q] == th[j] && gm[q] == gm[j]) d_row[j] = d_row[q];
+    if (d_row[j] == -2) d_row[j] = nd++;
+  }
+  if (nd > w.dt_rows) {
+    dev_free(w.dtils);
+    w.dt_rows = 0;
+    ASCG_TRY(dev_alloc(&w.dtils, (size_t)nd * op->n));
+    w.dt_rows = nd;
+  }
+  for (int q = 0; q < ng; ++q) {
+    if (!w.oscaled[q]) ASCG_TRY(dev_alloc(&w.oscaled[q], (size_t)op->o_len));
+    ASCG_CUDA(launch_shift_scale(op->o_val, op->o_len, 0.0, 1.0 / gam_of[q], w.oscaled[q], st));
+    ++*launches;
+  }
+  int made = 0;
+  for (int j = 0; j < s; ++j) {
+    const double inv = 1.0 / gm[j];
+    const double* dt = d_row[j] < 0 ? op->diag : w.dtils + (int64_t)d_row[j] * op->n;
+    if (d_row[j] == made) {
+      ASCG_CUDA(launch_shift_scale(op->diag, op->n, th[j], inv, w.dtils + (int64_t)made * op->n, st));
+      ++made;
       ++*launches;
-      dt = dst;
     }
     // sig_j = sigma_{j-1} / gamma_j, exactly 1 when the two are equal (Chebyshev)
     const double sj = j < 1 ? 0.0 : (sg[j - 1] == gm[j] ? 1.0 : sg[j - 1] * inv);
-    out[j] = StepOp{ov, dt, sj};
+    out[j] = StepOp{o_slot[j] < 0 ? op->o_val : w.oscaled[o_slot[j]], dt, sj};
   }
   return ASCG_OK;
 }
 
+// Runs classical CG iterations (Alg. 1) on the device until the CG state says
+// done. x, r, p, q are device vectors. Returns the iterations done by this call.
 ascg_status run_classical(ascg_op op, double* x, double* r, double* p, double eps_star, double bnorm,
                           int max_iters, int iter0, cudaStream_t s, ascg_result* res, bool timing) {
   Workspace& w = op->ws;
@@ -581,7 +693,7 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
     StepOp steps[kMaxS];
     if (!done) {
       int nl = 0;
-      ASCG_TRY(prepare_steps(op, th, sg, gm, o.s_max, w.dtils, w.oscaled, steps, s, &nl));
+      ASCG_TRY(prepare_steps(op, th, sg, gm, o.s_max, steps, s, &nl));
       res->launches += nl;
     }
     const DevSplit Asplit = op->split();
@@ -943,6 +1055,7 @@ ascg_status ascg_op_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, co
     delete op;
     return st;
   }
+  scratch_op_created();
   *out = op;
   return ASCG_OK;
 }
@@ -952,6 +1065,7 @@ ascg_status ascg_op_destroy(ascg_op op) {
   op->ws.release();
   op->free_device();
   delete op;
+  scratch_op_destroyed();
   return ASCG_OK;
 }
 
@@ -1051,22 +1165,13 @@ ascg_status ascg_matrix_powers(ascg_op op, int s, const double* theta, const dou
   if (s < 1 || s > ASCG_MAX_S) return fail(ASCG_ERR_INVALID, "s must be in 1..16");
   if (ldY < op->n) return fail(ASCG_ERR_INVALID, "ldY < n");
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  double* dtils = nullptr;
-  double* osc[2] = {nullptr, nullptr};
-  ascg_status rs = dev_alloc(&dtils, (size_t)s * op->n);
-  if (rs == ASCG_OK) rs = dev_alloc(&osc[0], (size_t)op->o_len);
-  if (rs == ASCG_OK) rs = dev_alloc(&osc[1], (size_t)op->o_len);
   StepOp steps[kMaxS];
   int nl = 0;
-  if (rs == ASCG_OK) rs = prepare_steps(op, theta, sigma, gamma, s, dtils, osc, steps, st, &nl);
+  ASCG_TRY(prepare_steps(op, theta, sigma, gamma, s, steps, st, &nl));
   cudaError_t e = cudaSuccess;
-  for (int j = 0; rs == ASCG_OK && j < s && e == cudaSuccess; ++j)
+  for (int j = 0; j < s && e == cudaSuccess; ++j)
     e = launch_mpk_split_step(op->split(), steps[j], Y, ldY, j, 1, j < s - 1, nullptr, 0, st);
-  if (e == cudaSuccess && rs == ASCG_OK) e = cudaStreamSynchronize(st);
-  cudaFree(dtils);
-  cudaFree(osc[0]);
-  cudaFree(osc[1]);
-  if (rs != ASCG_OK) return rs;
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("matrix powers: ") + cudaGetErrorString(e));
   return ASCG_OK;
 }
@@ -1075,27 +1180,22 @@ ascg_status ascg_gram(int64_t n, int w, const double* Y, int64_t ldY, double* G,
   g_err.clear();
   if (!Y || !G || n < 1 || w < 1 || w > ASCG_MAX_W || ldY < n) return fail(ASCG_ERR_INVALID, "bad argument");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  double* partials = nullptr;
-  int* expp = nullptr;
+  Scratch sc;
+  const size_t np = (size_t)gram_grid() * kMaxPairs;
+  ASCG_TRY(sc.open(Scratch::round(np * sizeof(double)) + Scratch::round((kMaxW + 1) * sizeof(int))));
+  double* partials = sc.take<double>(np);
+  int* expp = sc.take<int>(kMaxW + 1);  // column exponents, then one error word of the tensor-core kernel
+  int* herr = sc.host<int>();
   int parts = 0;
-  ASCG_TRY(dev_alloc(&partials, (size_t)gram_grid() * kMaxPairs));
-  // column exponents, then one error word of the tensor-core kernel
-  const size_t nexp = (size_t)gram_grid() * kMaxW;
-  ascg_status rs = dev_alloc(&expp, nexp + 1);
-  if (rs != ASCG_OK) {
-    cudaFree(partials);
-    return rs;
-  }
-  int herr = 0;
-  cudaError_t e = cudaMemsetAsync(expp + nexp, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = launch_gram_any(n, w, Y, ldY, false, expp, false, partials, &parts, s, expp + nexp);
+  cudaError_t e = cudaMemsetAsync(expp, 0, (kMaxW + 1) * sizeof(int), s);
+  if (e == cudaSuccess) e = launch_gram_any(n, w, Y, ldY, false, expp, false, partials, &parts, s, expp + kMaxW);
   if (e == cudaSuccess) e = launch_gram_finalize(w, partials, parts, G, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, expp + nexp, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(herr, expp + kMaxW, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(partials);
-  cudaFree(expp);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("gram: ") + cudaGetErrorString(e));
-  if (herr == ASCG_ERR_TIMEOUT) return fail(ASCG_ERR_TIMEOUT, "gram: a bounded wait of the tensor-core kernel ran out");
+  sc.synced();
+  if (*herr == ASCG_ERR_TIMEOUT)
+    return fail(ASCG_ERR_TIMEOUT, "gram: a bounded wait of the tensor-core kernel ran out");
   return ASCG_OK;
 }
 
@@ -1103,15 +1203,17 @@ ascg_status ascg_gram_moments(int64_t n, int s_, const double* Y, int64_t ldY, d
   g_err.clear();
   if (!Y || !G || n < 1 || s_ < 1 || s_ > ASCG_MAX_S || ldY < n) return fail(ASCG_ERR_INVALID, "bad argument");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  double* partials = nullptr;
-  ASCG_TRY(dev_alloc(&partials, (size_t)gram_grid() * kMomSlots));
+  Scratch sc;
+  const size_t np = (size_t)gram_grid() * kMomSlots;
+  ASCG_TRY(sc.open(Scratch::round(np * sizeof(double))));
+  double* partials = sc.take<double>(np);
   int parts = 0;
   const int w = 2 * s_ + 1;
   cudaError_t e = launch_gram_moments(n, w, Y, ldY, partials, &parts, s);
   if (e == cudaSuccess) e = launch_gram_moment_finalize(w, partials, parts, G, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(partials);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("gram moments: ") + cudaGetErrorString(e));
+  sc.synced();
   return ASCG_OK;
 }
 
@@ -1125,25 +1227,21 @@ ascg_status ascg_block_step(int sbar, const double* G, int method, const double*
   if (method != ASCG_ADAPTIVE && method != ASCG_FIXED_S) return fail(ASCG_ERR_INVALID, "method");
   if (!(bnorm > 0.0) || !(c > 0.0) || nrows < 1 || max_steps < 0) return fail(ASCG_ERR_INVALID, "bad scalar");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  BlockState* bst = nullptr;
-  double* dpar = nullptr;
-  double* dhist = nullptr;
-  double* dspec = nullptr;
-  unsigned* dcnt = nullptr;
-  ASCG_TRY(dev_alloc(&bst, 1));
-  ascg_status st = dev_alloc(&dpar, 3 * kMaxS);
-  if (st == ASCG_OK) st = dev_alloc(&dhist, 3 * kMaxS);
-  if (st == ASCG_OK) st = dev_alloc(&dspec, kSpecDoubles);
-  if (st == ASCG_OK) st = dev_alloc(&dcnt, 1);
-  if (st != ASCG_OK) {
-    cudaFree(bst);
-    cudaFree(dpar);
-    cudaFree(dhist);
-    cudaFree(dspec);
-    return st;
-  }
-  BlockState hb;
-  std::memset(&hb, 0, sizeof(hb));
+  // one copy in (state, coefficients, the controller's ticket), one out (state, histories)
+  struct In {
+    BlockState st;
+    double hist[3 * kMaxS];
+    double par[3 * kMaxS];
+    unsigned ticket;
+  };
+  static_assert(sizeof(In) <= kScratchHost, "staging");
+  Scratch sc;
+  ASCG_TRY(sc.open(Scratch::round(sizeof(In)) + Scratch::round(kSpecDoubles * sizeof(double))));
+  In* din = sc.take<In>(1);
+  double* dspec = sc.take<double>(kSpecDoubles);
+  In& h = *sc.host<In>();
+  std::memset(&h, 0, sizeof(h));
+  BlockState& hb = h.st;
   hb.sbar = sbar;
   hb.method = method;
   hb.check_in_loop = check_in_loop;
@@ -1153,28 +1251,19 @@ ascg_status ascg_block_step(int sbar, const double* G, int method, const double*
   hb.bnorm = bnorm;
   hb.sqrt_n = std::sqrt((double)nrows);
   hb.active = 1;
-  double hp[3 * kMaxS];
   for (int j = 0; j < kMaxS; ++j) {
-    hp[j] = j < sbar ? theta[j] : 0.0;
-    hp[kMaxS + j] = j < sbar ? sigma[j] : 0.0;
-    hp[2 * kMaxS + j] = j < sbar ? gamma[j] : 1.0;
+    h.par[j] = j < sbar ? theta[j] : 0.0;
+    h.par[kMaxS + j] = j < sbar ? sigma[j] : 0.0;
+    h.par[2 * kMaxS + j] = j < sbar ? gamma[j] : 1.0;
   }
-  double hh[3 * kMaxS];
-  cudaError_t e = cudaMemcpyAsync(bst, &hb, sizeof(hb), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dpar, hp, sizeof(hp), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dcnt, 0, sizeof(unsigned), s);
+  cudaError_t e = cudaMemcpyAsync(din, &h, sizeof(In), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = launch_block_ctrl(G, dpar, dpar + kMaxS, dpar + 2 * kMaxS, bst, sbar, method == ASCG_ADAPTIVE, coords, dhist,
-                          nullptr, 0, nullptr, 0, dspec, dcnt, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hb, bst, sizeof(hb), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(hh, dhist, sizeof(hh), cudaMemcpyDeviceToHost, s);
+    e = launch_block_ctrl(G, din->par, din->par + kMaxS, din->par + 2 * kMaxS, &din->st, sbar, method == ASCG_ADAPTIVE,
+                          coords, din->hist, nullptr, 0, nullptr, 0, dspec, &din->ticket, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, din, offsetof(In, par), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(bst);
-  cudaFree(dpar);
-  cudaFree(dhist);
-  cudaFree(dspec);
-  cudaFree(dcnt);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("block step: ") + cudaGetErrorString(e));
+  sc.synced();
   std::memset(info, 0, sizeof(*info));
   info->sbar = sbar;
   info->stilde = hb.stilde;
@@ -1184,7 +1273,7 @@ ascg_status ascg_block_step(int sbar, const double* G, int method, const double*
   info->threshold = hb.threshold;
   info->gamma = hb.gamma;
   for (int i = 0; i < sbar; ++i) info->sqrt_kappa[i] = method == ASCG_ADAPTIVE ? hb.sqrt_kappa[i] : 0.0;
-  if (hist) std::memcpy(hist, hh, sizeof(double) * 3 * std::max(hb.s_k, 0));
+  if (hist) std::memcpy(hist, h.hist, sizeof(double) * 3 * std::max(hb.s_k, 0));
   return ASCG_OK;
 }
 
@@ -1204,17 +1293,18 @@ ascg_status ascg_recover_tc(int64_t n, int w, const double* Y, int64_t ldY, cons
     return fail(ASCG_ERR_INVALID, "bad argument");
   if (!gram_tc_aligned(Y, ldY)) return fail(ASCG_ERR_INVALID, "Y must be 16-byte aligned with an even ldY");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  int* expp = nullptr;  // column exponents, then the kernel's error word
-  ASCG_TRY(dev_alloc(&expp, (size_t)kMaxW + 1));
-  int herr = 0;
+  Scratch sc;
+  ASCG_TRY(sc.open(Scratch::round((kMaxW + 1) * sizeof(int))));
+  int* expp = sc.take<int>(kMaxW + 1);  // column exponents, then the kernel's error word
+  int* herr = sc.host<int>();
   cudaError_t e = cudaMemsetAsync(expp + kMaxW, 0, sizeof(int), s);
   if (e == cudaSuccess) e = launch_col_exponents(n, w, Y, ldY, expp, s);
   if (e == cudaSuccess) e = launch_recover_tc(n, w, Y, ldY, expp, coords, x, r, p, s, expp + kMaxW);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, expp + kMaxW, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(herr, expp + kMaxW, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(expp);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("recover_tc: ") + cudaGetErrorString(e));
-  if (herr == ASCG_ERR_TIMEOUT) return fail(ASCG_ERR_TIMEOUT, "recover_tc: a bounded wait of the kernel ran out");
+  sc.synced();
+  if (*herr == ASCG_ERR_TIMEOUT) return fail(ASCG_ERR_TIMEOUT, "recover_tc: a bounded wait of the kernel ran out");
   return ASCG_OK;
 }
 
@@ -1224,17 +1314,19 @@ ascg_status ascg_newton_shifts(const double* alphas, const double* betas, int k,
   if (!alphas || (k > 1 && !betas) || !shifts || k < 1 || k > 32 || s < 1 || s > k)
     return fail(ASCG_ERR_INVALID, "bad argument");
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  double* d = nullptr;
-  ASCG_TRY(dev_alloc(&d, 96));
-  double h[96] = {0};
+  Scratch sc;
+  ASCG_TRY(sc.open(96 * sizeof(double)));
+  double* d = sc.take<double>(96);
+  double* h = sc.host<double>();
+  std::memset(h, 0, 96 * sizeof(double));
   for (int j = 0; j < k; ++j) h[j] = alphas[j];
   for (int j = 0; j + 1 < k; ++j) h[32 + j] = betas[j];
-  cudaError_t e = cudaMemcpyAsync(d, h, sizeof(h), cudaMemcpyHostToDevice, st);
+  cudaError_t e = cudaMemcpyAsync(d, h, 96 * sizeof(double), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = launch_newton_shifts(d, d + 32, k, d + 64, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h, d + 64, sizeof(double) * 32, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(d);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("newton shifts: ") + cudaGetErrorString(e));
+  sc.synced();
   for (int j = 0; j < s; ++j) shifts[j] = h[j];
   return ASCG_OK;
 }

@@ -1,7 +1,8 @@
 // ascg_gram_noalloc: the Gram matrix G = Y^T Y without any device allocation.
 //
-// ascg_gram obtains its per-CTA partial sums from cudaMalloc and releases them
-// with cudaFree on every call. Some callers cannot allow that. Examples are code
+// ascg_gram keeps its per-CTA partial sums in a scratch block that a call may
+// have to obtain from cudaMalloc or release with cudaFree. Some callers cannot
+// allow that. Examples are code
 // that runs under a fixed device-memory budget owned by a host framework, and
 // latency-sensitive loops where the implicit device synchronisation of
 // cudaFree would stall other streams. This variant keeps its partial sums in

@@ -44,3 +44,88 @@ def test_batch_row_lengths(n):
     for (a, *_), b, x in zip(sys, bs, xd):
         ref = np.linalg.solve(a, b)
         assert np.linalg.norm(x.cpu().numpy() - ref) <= 1.6e-10 * np.linalg.norm(ref)
+
+
+def _diagonals(n, h, rng):
+    """Integer band matrix as diagonals: main[n] in 1..4, off[k-1][n-k] in -2..2 without 0, k = 1..h."""
+    main = rng.integers(1, 5, n).astype(np.float64)
+    off = [rng.choice([-2.0, -1.0, 1.0, 2.0], max(n - k, 0)) for k in range(1, h + 1)]
+    return main, off
+
+
+def _apply(main, off, v):
+    y = main * v
+    for k, u in enumerate(off, 1):
+        if len(u):
+            y[: -k] += u * v[k:]
+            y[k:] += u * v[: -k]
+    return y
+
+
+@pytest.mark.parametrize("h", [0, 1, 2, 3, 6, 9])
+@pytest.mark.parametrize("n", [1, 31, 33, 127, 129, 65536, 65537])
+def test_matrix_powers_exact_integers(n, h):
+    """Small integers and powers of two: every result is an exact integer, so both kernels (a warp per chain up to 65536
+    rows or for long rows, both chains in a thread otherwise) must give numpy's values bit for bit, whatever the order."""
+    import paper_1701_03989_gb300 as P
+
+    rng = np.random.default_rng(1000 * h + n)
+    h = min(h, n - 1)
+    main, off = _diagonals(n, h, rng)
+    cols = np.arange(n)[:, None] + np.arange(-h, h + 1)[None, :]
+    vals = np.zeros((n, 2 * h + 1))
+    vals[:, h] = main
+    for k, u in enumerate(off, 1):
+        vals[: n - k, h + k] = u
+        vals[k:, h - k] = u
+    keep = (cols >= 0) & (cols < n)
+    rowptr = np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int64)
+    op = P.ascg_op_create_csr(n, int(rowptr[-1]), rowptr, cols[keep].astype(np.int32), vals[keep], 0)
+    for s, th, sg, gm in ((1, [1.0], [0.0], [1.0]), (4, [0.0] * 4, [0.0] * 4, [1.0] * 4),
+                          (4, [1.0, 2.0, 1.0, 3.0], [0.5, 0.5, 0.5, 0.5], [1.0, 0.5, 0.5, 0.5]),
+                          (3, [1.0, 0.0, 2.0], [2.0, 4.0, 1.0], [0.5, 0.5, 0.5])):
+        Y = np.zeros((2 * s + 1, n))
+        Y[0], Y[1] = rng.integers(-3, 4, n), rng.integers(-3, 4, n)
+        Yd = torch.from_numpy(Y.copy()).cuda()
+        P.ascg_matrix_powers(op, s, np.array(th), np.array(sg), np.array(gm), Yd, n)
+        for k in range(2, 2 * s + 1):
+            j = k // 2 - 1
+            v = _apply(main, off, Y[k - 2]) - th[j] * Y[k - 2]
+            if j:
+                v = v - sg[j - 1] * Y[k - 4]
+            Y[k] = v / gm[j]
+        assert np.array_equal(Yd.cpu().numpy(), Y), (s, th)
+    P.ascg_op_destroy(op)
+
+
+def test_scratch_of_concurrent_calls():
+    """Single-step calls from several threads on streams of their own: each gives the bits it gives alone."""
+    import threading
+
+    import paper_1701_03989_gb300 as P
+
+    g = torch.Generator(device="cuda").manual_seed(5)
+    Ys = [torch.rand((w, 2048), dtype=torch.float64, device="cuda", generator=g) for w in (5, 9, 17, 33)]
+    Gs = [torch.empty((len(Y), len(Y)), dtype=torch.float64, device="cuda") for Y in Ys]
+    alone = []
+    for Y, G in zip(Ys, Gs):
+        P.ascg_gram(2048, len(Y), Y, 2048, G)
+        alone.append(G.cpu())
+    bad = []
+
+    def work(k):
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            G = torch.empty_like(Gs[k])
+            for _ in range(50):
+                P.ascg_gram(2048, len(Ys[k]), Ys[k], 2048, G, stream=s)
+                if not torch.equal(G.cpu(), alone[k]):
+                    bad.append(k)
+
+    threads = [threading.Thread(target=work, args=(k % 4,)) for k in range(8)]
+    torch.cuda.synchronize()
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
