@@ -432,7 +432,7 @@ struct BlockState {
 // capacity res_cap (entries m+1 .. m+s_k written), or nullptr. spec: device
 // scratch of kSpecDoubles; counter: device unsigned, zero on entry and left
 // zero. adaptive: st->method == ASCG_ADAPTIVE.
-constexpr int kSpecDoubles = kMaxS * (3 * kMaxW + 3) + 1;
+constexpr int kSpecDoubles = kMaxS * (3 * kMaxW + 3) + 1 + (2 * kMaxS + 3);
 cudaError_t launch_block_ctrl(const double* G, const double* theta, const double* sigma, const double* gamma,
                               BlockState* st, int sbar, int adaptive, double* coords, double* hist, double* res_hist,
                               int res_cap, double* ab_hist, int ab_cap, double* spec, unsigned* counter,

@@ -4,8 +4,9 @@
 // shifts.
 //
 // All of this is tiny dense work on matrices of order <= 33. On GB300 an FP64
-// warp instruction costs ~20 SM cycles whether 1 or 32 lanes are active, and
-// a dependent DFMA takes 64 cycles. So this code keeps the lanes busy on
+// warp instruction takes 64 cycles of its SM sub-partition (77 with all four
+// busy) whether 0, 1 or 32 lanes are active, a comparison 110 to 220, a
+// reciprocal 325, a square root 550, a shuffle and add 110. So this code keeps the lanes busy on
 // independent work: one lane per row for the Householder steps, and 64
 // evaluation points per Sturm multisection round.
 #include <math_constants.h>
@@ -56,40 +57,66 @@ __device__ void gershgorin(const double* d, const double* e, int m, double* lo, 
 // rescalings do not change signs), the backward error of the pivot form.
 // The loop is unrolled with d and e2 in registers. Each step costs three FP64
 // instructions (d_k - x, the product with e2 and the FMA); on GB300 an SM
-// sub-partition issues about one FP64 warp instruction per 64 cycles, and
-// that rate, not latency, sets the time of a multisection round. The leading
-// minors grow at most like (1 + sqrt 2)^k <= 2^43 for M <= 33, so they cannot
-// overflow. One integer test of the exponent per step catches, on a rarely
-// taken branch, both a minor below 2^-256 (rescaled exactly by 2^256, with
-// its predecessor) and a zero minor (replaced by a tiny value of the sign
-// opposite to its predecessor).
-template <int M>
-__device__ __forceinline__ int sturm_unrolled(const double (&d)[M], const double (&e2)[M], double x) {
+// sub-partition issues about one FP64 warp instruction per 64 cycles (77 with
+// all four busy), and that rate sets the time of a multisection round, so a
+// minor is looked at only once the next step's instructions are on their way
+// (244 cycles a step against 260 before and 231 for the three alone). The
+// leading minors grow at most like (1 + sqrt 2)^k <= 2^43 for M <= 33, so they
+// cannot overflow. One integer test of the exponent per step catches, on a
+// rarely taken branch, both a minor below 2^-256 (rescaled exactly by 2^256,
+// with its predecessor) and a zero minor (replaced by a tiny value of the sign
+// opposite to its predecessor). The vote keeps it a branch of the whole warp:
+// a predicated-off FP64 instruction takes its 64 cycles too.
+__device__ __forceinline__ bool minor_small(double p) { return ((__double2hiint(p) >> 20) & 0x7ff) < 767; }
+__device__ __forceinline__ void minor_rescale(double& p, double& before) {
   const double kUp = 1.157920892373162e77;     // 2^256
   const double kTiny = 8.636168555094445e-78;  // 2^-256
-  double pm2 = 1.0;
-  double pm1 = d[0] - x;
-  if (pm1 == 0.0) pm1 = -kTiny * kTiny;
-  int hprev = __double2hiint(pm1);
+  if (((__double2hiint(p) & 0x7fffffff) | __double2loint(p)) == 0) {
+    p = -copysign(fabs(before) * kTiny, before);
+  } else {
+    p *= kUp;
+    before *= kUp;
+  }
+}
+template <int M>
+__device__ __forceinline__ int sturm_unrolled(const double (&d)[M], const double (&e2)[M], double x) {
+  const double kTiny = 8.636168555094445e-78;  // 2^-256
+  double q2 = 1.0, q1 = d[0] - x;              // p_{k-2}, p_{k-1}
+  if (((__double2hiint(q1) & 0x7fffffff) | __double2loint(q1)) == 0) q1 = -kTiny * kTiny;
+  double t = e2[0], dx = d[M > 1 ? 1 : 0] - x;  // of step k: e2_{k-1} p_{k-2} and d_k - x
+  int hprev = __double2hiint(q1);
   int cnt = (int)((unsigned)hprev >> 31);
 #pragma unroll
   for (int k = 1; k < M; ++k) {
-    const double t = e2[k - 1] * pm2;
-    double p = fma(d[k] - x, pm1, -t);
-    int hp = __double2hiint(p);
-    if (((hp >> 20) & 0x7ff) < 767) {  // |p| < 2^-256 or p == 0 (rare)
-      if (((hp & 0x7fffffff) | __double2loint(p)) == 0) {
-        p = -copysign(fabs(pm1) * kTiny, pm1);
-      } else {  // exact rescaling of p_k and p_{k-1}
-        p *= kUp;
-        pm1 *= kUp;
-      }
-      hp = __double2hiint(p);
+    double p = fma(dx, q1, -t), tn = 0.0, dxn = 0.0;
+    if (k + 1 < M) {
+      tn = e2[k] * q1;
+      dxn = d[k + 1 < M ? k + 1 : k] - x;
     }
-    cnt += (int)((unsigned)(hp ^ hprev) >> 31);
-    pm2 = pm1;
-    pm1 = p;
-    hprev = hp;
+    if (k >= 2) {  // p_{k-1}, now that this step is on its way
+      if (__any_sync(kFull, minor_small(q1))) {
+        asm volatile("" ::: "memory");
+        if (minor_small(q1)) {
+          minor_rescale(q1, q2);
+          p = fma(dx, q1, -(e2[k - 1] * q2));
+          if (k + 1 < M) tn = e2[k] * q1;
+        }
+      }
+      const int h = __double2hiint(q1);
+      cnt += (int)((unsigned)(h ^ hprev) >> 31);
+      hprev = h;
+    }
+    q2 = q1;
+    q1 = p;
+    t = tn;
+    dx = dxn;
+  }
+  if (M > 1) {
+    if (__any_sync(kFull, minor_small(q1))) {
+      asm volatile("" ::: "memory");
+      if (minor_small(q1)) minor_rescale(q1, q2);
+    }
+    cnt += (int)((unsigned)(__double2hiint(q1) ^ hprev) >> 31);
   }
   return cnt;
 }
@@ -99,11 +126,12 @@ __device__ __forceinline__ int sturm_unrolled(const double (&d)[M], const double
 // for the smallest x with count(x) >= target on [lo, hi]. half: the warp's
 // place in the pair. geo0: the first round uses the points hi * 2^(k - 64),
 // k = 0..63. stop_below: if the first geometric bracket lies at or below this
-// value, sets *below and stops. Both warps compute the same brackets.
+// value, sets *below and stops. frac: shared, frac[k] = (k + 1) / 65. Both
+// warps compute the same brackets.
 template <int M>
 __device__ void multisect_pair(const double* ds, const double* e2s, int target, int rounds, bool geo0,
                                double stop_below, double* lo_io, double* hi_io, int* below, int half, int bar_id,
-                               unsigned* s_mask) {
+                               unsigned* s_mask, const double* frac) {
   const int lane = threadIdx.x & 31;
   const int k = lane + 32 * half;
   double d[M], e2[M];
@@ -112,11 +140,11 @@ __device__ void multisect_pair(const double* ds, const double* e2s, int target, 
     d[q] = ds[q];
     e2[q] = q + 1 < M ? e2s[q] : 0.0;
   }
-  const double kStep = 1.0 / 65.0;
+  const double fk = frac[k];
   double lo = *lo_io, hi = *hi_io;
   for (int round = 0; round < rounds; ++round) {
     const bool geo = geo0 && round == 0;
-    const double x = geo ? ldexp(hi, k - 64) : lo + (hi - lo) * ((double)(k + 1) * kStep);
+    const double x = geo ? ldexp(hi, k - 64) : lo + (hi - lo) * fk;
     const unsigned mk = __ballot_sync(kFull, sturm_unrolled<M>(d, e2, x) >= target);
     if (lane == 0) s_mask[half] = mk;
     asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
@@ -124,7 +152,7 @@ __device__ void multisect_pair(const double* ds, const double* e2s, int target, 
     asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");  // both masks read before the next round
     // the point k' of either warp, recomputed from the shared bracket
     auto point = [&](int kk) {
-      return geo ? ldexp(hi, kk - 64) : lo + (hi - lo) * ((double)(kk + 1) * kStep);
+      return geo ? ldexp(hi, kk - 64) : lo + (hi - lo) * frac[kk];
     };
     double nlo = lo, nhi = hi;
     if (both == 0ull) {
@@ -147,11 +175,11 @@ __device__ void multisect_pair(const double* ds, const double* e2s, int target, 
 
 __device__ void multisect_pair_dispatch(int m, const double* ds, const double* e2s, int target, int rounds,
                                         bool geo0, double stop_below, double* lo, double* hi, int* below, int half,
-                                        int bar_id, unsigned* s_mask) {
+                                        int bar_id, unsigned* s_mask, const double* frac) {
   switch (m) {
 #define ASCG_MP(M)                                                                                          \
   case M:                                                                                                   \
-    multisect_pair<M>(ds, e2s, target, rounds, geo0, stop_below, lo, hi, below, half, bar_id, s_mask); \
+    multisect_pair<M>(ds, e2s, target, rounds, geo0, stop_below, lo, hi, below, half, bar_id, s_mask, frac); \
     break;
     ASCG_MP(3) ASCG_MP(5) ASCG_MP(7) ASCG_MP(9) ASCG_MP(11) ASCG_MP(13) ASCG_MP(15) ASCG_MP(17)
     ASCG_MP(19) ASCG_MP(21) ASCG_MP(23) ASCG_MP(25) ASCG_MP(27) ASCG_MP(29) ASCG_MP(31) ASCG_MP(33)
@@ -161,16 +189,67 @@ __device__ void multisect_pair_dispatch(int m, const double* ds, const double* e
   }
 }
 
-// Warp-wide min and max (identical in all lanes).
-__device__ __forceinline__ double warp_min(double v) {
+// Sum over the lanes 0 .. len - 1 (the others hold zeros) in warp_sum's order,
+// valid in those lanes: the levels of the tree that would only add zeros are
+// left out (each level is a shuffle and an add, 110 cycles).
+template <int LEVELS>
+__device__ __forceinline__ double warp_sum_levels(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(kFull, v, o));
+  for (int o = 1 << (LEVELS - 1); o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_max(double v) {
+__device__ __forceinline__ double warp_sum_len(double v, int len) {
+  if (len > 16) return warp_sum_levels<5>(v);
+  if (len > 8) return warp_sum_levels<4>(v);
+  if (len > 4) return warp_sum_levels<3>(v);
+  return warp_sum_levels<2>(v);
+}
+
+// sum_c a[c] v[c], c < NC: even and odd c in two chains, then their sum.
+template <int NC>
+__device__ __forceinline__ double dot_even_odd(const double* a, const double* v) {
+  double ac[NC], vc[NC];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
-  return v;
+  for (int q = 0; q < NC; ++q) {
+    ac[q] = a[q];
+    vc[q] = v[q];
+  }
+  double p0 = 0.0, p1 = 0.0;
+#pragma unroll
+  for (int q = 0; q < NC; q += 2) {
+    p0 = fma(ac[q], vc[q], p0);
+    if (q + 1 < NC) p1 = fma(ac[q + 1], vc[q + 1], p1);
+  }
+  return p0 + p1;
+}
+
+// Warp-wide min and max (identical in all lanes; a NaN counts as absent, as in
+// fmin and fmax), by integer comparisons: an FP64 fmin takes 220 cycles.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);  // its own inverse; increasing in v
+}
+__device__ __forceinline__ double key_value(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+__device__ __forceinline__ bool is_nan(double v) {
+  return (__double_as_longlong(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ double warp_min(long long k) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long u = __shfl_xor_sync(kFull, k, o);
+    k = u < k ? u : k;
+  }
+  return key_value(k);
+}
+__device__ __forceinline__ double warp_max(long long k) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long u = __shfl_xor_sync(kFull, k, o);
+    k = u > k ? u : k;
+  }
+  return key_value(k);
 }
 
 // kappa(G_{k,i}). G_{k,i} is the leading (2i+1) block of G
@@ -190,6 +269,15 @@ __device__ __forceinline__ double warp_max(double v) {
 // most 2 lambda_max wide, and six rounds leave < 2e-10 of it. kappa is thus
 // known to about 1e-9, far inside the 1e-6 to which rounding in G already
 // makes decisions near a threshold uncertain.
+//
+// Cycles at m = 33 / 17 (one SM, measured with its clock): load 2300 / 1800
+// (4300 / 1800 before every load was in flight at once), Householder 136400 /
+// 62300 (147900 / 70700 before predicated-off FMAs, FP64 comparisons and the
+// sums' empty levels were taken out), scaling 4800 / 3900 (7900 / 6200 with
+// FP64 minima), multisection 57000 / 32000 (58800 / 34000), end and
+// selection 13000 / 12700 before the selection's scalars moved to the CTA of
+// the coordinate steps. ascg_block_step at s = 16: 138.2 -> 125.7 us, the same
+// bits. What bounds it is the latency of one warp's FP64 chain.
 constexpr int kKappaRounds = 6;
 
 // Run by a whole CTA of 128 threads: sqrt(kappa(G_{k,i})) into st->sqrt_kappa[i-1]
@@ -205,20 +293,39 @@ __device__ void kappa_body(const double* __restrict__ G, BlockState* st, int i, 
   __shared__ double den_s[2], floor_s;
   __shared__ int go_s[2], uncert_s;
   __shared__ unsigned s_mask[2][2];
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) A[idx / m][idx % m] = G[(idx / m) * w + (idx % m)];
-  __syncthreads();
+  __shared__ double frac_s[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // The reflection that zeroes column kk below its subdiagonal (run by warp 0):
-  // v = x - alpha e_1 over rows kk+1 .. m-1, alpha = -sign(x_0) ||x||, and
-  // beta = 2 / v^T v = 1 / (s2 + |x_0| ||x||) (v^T v = 2 (s2 + |x_0| ||x||));
-  // warp 0 publishes the denominator and every warp divides for itself.
-  auto reflector = [&](int kk, int slot) {
+  // warp q takes rows q, q + 4, ...; every load is in flight before the first store
+  {
+    double g[9], g32[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      const int r = warp + 4 * q;
+      g[q] = r < m && lane < m ? G[r * w + lane] : 0.0;
+      g32[q] = r < m && m > 32 && lane == 0 ? G[r * w + 32] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      const int r = warp + 4 * q;
+      if (r < m && lane < m) A[r][lane] = g[q];
+      if (r < m && m > 32 && lane == 0) A[r][32] = g32[q];
+    }
+  }
+  if (threadIdx.x < 64) frac_s[threadIdx.x] = (double)(threadIdx.x + 1) * (1.0 / 65.0);
+  __syncthreads();
+  // The reflection that zeroes column kk below its subdiagonal (run by warp 0;
+  // xi: the column's entry in row kk + 1 + lane): v = x - alpha e_1 over rows
+  // kk+1 .. m-1, alpha = -sign(x_0) ||x||, and beta = 2 / v^T v = 1 / (s2 +
+  // |x_0| ||x||) (v^T v = 2 (s2 + |x_0| ||x||)); warp 0 publishes the
+  // denominator and every warp divides for itself.
+  auto reflector = [&](int kk, int slot, double xi) {
     const int len_ = m - kk - 1;
     const bool on_ = lane < len_;
-    const double xi = on_ ? A[kk + 1 + lane][kk] : 0.0;
-    const double s2 = warp_sum(xi * xi);
+    if (!on_) xi = 0.0;
+    const double s2 = warp_sum_len(xi * xi, len_);
     const double x0 = __shfl_sync(kFull, xi, 0);
-    const int go = s2 > 0.0;
+    const unsigned long long sb = (unsigned long long)__double_as_longlong(s2);
+    const int go = sb - 1 < 0x7ff0000000000000ull;  // s2 > 0 (s2 >= 0 or NaN), without an FP64 comparison
     double alpha = 0.0, vv = 0.0;
     if (go) {
       const double r = sqrt(s2);
@@ -236,45 +343,67 @@ __device__ void kappa_body(const double* __restrict__ G, BlockState* st, int i, 
   // forms the product p = A22 v (columns split evenly), then, redundantly in
   // each warp, w = beta p - (beta^2 v^T p / 2) v, and applies the rank-2
   // update to its columns. Warp 0 owns only the first trailing column (column
-  // k+1), so it can form the next step's reflection while warps 1..3 update
-  // the rest. Two barriers per step; the arithmetic, and so every bit, is the
-  // same as updating in turn.
-  if (warp == 0 && m >= 3) reflector(0, 0);
+  // k+1), so it can form the next step's reflection, from registers, while
+  // warps 1..3 update the rest. Two barriers per step; the arithmetic, and so
+  // every bit, is the same as updating in turn. What bounds a step is the FP64
+  // pipe of warp 0's sub-partition (about 47 instructions of 64 cycles, half
+  // of them the two sums, the square root and the division), so every operand
+  // is loaded ahead of the FMAs that use it.
+  if (warp == 0 && m >= 3) reflector(0, 0, lane + 1 < m ? A[1 + lane][0] : 0.0);
   __syncthreads();
   for (int k = 0; k + 2 < m; ++k) {
     const int len = m - k - 1;  // rows k+1 .. m-1, at most 32
     const int row = k + 1 + lane;
     const bool on = lane < len;
     const int sl = k & 1;
+    double next = 0.0;  // warp 0: column k + 1 after the update, row k + 1 + lane
     if (go_s[sl]) {  // uniform
       const double vi = on ? vb[sl][lane] : 0.0;
-      const double beta = 1.0 / den_s[sl];  // off warp 0's path: it overlaps this warp's product below
-      const int c0 = (len * warp) >> 2, c1 = (len * (warp + 1)) >> 2;
-      double p0 = 0.0, p1 = 0.0;
-      if (on) {
-        int c = c0;
-        for (; c + 1 < c1; c += 2) {
-          p0 = fma(A[row][k + 1 + c], vb[sl][c], p0);
-          p1 = fma(A[row][k + 2 + c], vb[sl][c + 1], p1);
-        }
-        if (c < c1) p0 = fma(A[row][k + 1 + c], vb[sl][c], p0);
+      const double den = den_s[sl];
+      const int c0 = (len * warp) >> 2, c1 = (len * (warp + 1)) >> 2;  // at most 8 columns
+      const double beta = 1.0 / den, hbeta = 0.5 * beta;
+      const double* ar = &A[on ? row : m - 1][k + 1 + c0];
+      const double* vr = &vb[sl][c0];
+      double pp = 0.0;
+      switch (c1 - c0) {  // straight-line code per length: a predicated-off FMA costs its 64 cycles too
+        case 1: pp = dot_even_odd<1>(ar, vr); break;
+        case 2: pp = dot_even_odd<2>(ar, vr); break;
+        case 3: pp = dot_even_odd<3>(ar, vr); break;
+        case 4: pp = dot_even_odd<4>(ar, vr); break;
+        case 5: pp = dot_even_odd<5>(ar, vr); break;
+        case 6: pp = dot_even_odd<6>(ar, vr); break;
+        case 7: pp = dot_even_odd<7>(ar, vr); break;
+        case 8: pp = dot_even_odd<8>(ar, vr); break;
+        default: break;
       }
-      part[warp][lane] = p0 + p1;
+      part[warp][lane] = on ? pp : 0.0;
+      next = warp == 0 && on ? A[row][k + 1] : 0.0;
       __syncthreads();
       const double pi = beta * ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]));
-      const double K = 0.5 * beta * warp_sum(vi * pi);
+      const double K = hbeta * warp_sum_len(vi * pi, len);
       const double wi = pi - K * vi;
       // rank-2 update of this warp's columns: warp 0 column 0, warps 1..3 the rest
-      const int g0 = warp == 0 ? 0 : 1 + (((len - 1) * (warp - 1)) / 3);
-      const int g1 = warp == 0 ? 1 : 1 + (((len - 1) * warp) / 3);
-      for (int c = g0; c < g1; ++c) {
-        const double vc = __shfl_sync(kFull, vi, c), wc = __shfl_sync(kFull, wi, c);
-        if (on) A[row][k + 1 + c] = fma(-vi, wc, fma(-wi, vc, A[row][k + 1 + c]));
+      if (warp == 0) {
+        const double v0 = __shfl_sync(kFull, vi, 0), w0 = __shfl_sync(kFull, wi, 0);
+        if (on) {
+          next = fma(-vi, w0, fma(-wi, v0, next));
+          A[row][k + 1] = next;
+        }
+      } else {
+        const int g0 = 1 + (((len - 1) * (warp - 1)) / 3), g1 = 1 + (((len - 1) * warp) / 3);
+#pragma unroll 4
+        for (int c = g0; c < g1; ++c) {
+          const double vc_ = __shfl_sync(kFull, vi, c), wc_ = __shfl_sync(kFull, wi, c);
+          if (on) A[row][k + 1 + c] = fma(-vi, wc_, fma(-wi, vc_, A[row][k + 1 + c]));
+        }
       }
+    } else if (warp == 0 && on) {
+      next = A[row][k + 1];
     }
     if (warp == 0 && k + 3 < m) {
-      __syncwarp();
-      reflector(k + 1, sl ^ 1);
+      // row k + 2 + lane of the column sits one lane up
+      const double xi = __shfl_down_sync(kFull, next, 1);
+      reflector(k + 1, sl ^ 1, lane < 31 ? xi : 0.0);
     }
     __syncthreads();
   }
@@ -284,18 +413,19 @@ __device__ void kappa_body(const double* __restrict__ G, BlockState* st, int i, 
     for (int r = lane; r < m; r += 32) d[r] = A[r][r];
     if (lane == 0) e[m - 2] = A[m - 1][m - 2];
     __syncwarp();
-    double gl = CUDART_INF, gh = -CUDART_INF, dmin = CUDART_INF, dmax = -CUDART_INF;
+    long long kgl = order_key(CUDART_INF), kgh = order_key(-CUDART_INF), kdmin = kgl, kdmax = kgh;
     for (int r = lane; r < m; r += 32) {
       const double off = (r > 0 ? fabs(e[r - 1]) : 0.0) + (r + 1 < m ? fabs(e[r]) : 0.0);
-      gl = fmin(gl, d[r] - off);
-      gh = fmax(gh, d[r] + off);
-      dmin = fmin(dmin, d[r]);
-      dmax = fmax(dmax, d[r]);
+      const double lo = d[r] - off, hi = d[r] + off, dr = d[r];
+      if (!is_nan(lo)) kgl = min(kgl, order_key(lo));
+      if (!is_nan(hi)) kgh = max(kgh, order_key(hi));
+      if (!is_nan(dr)) {
+        kdmin = min(kdmin, order_key(dr));
+        kdmax = max(kdmax, order_key(dr));
+      }
     }
-    gl = warp_min(gl);
-    gh = warp_max(gh);
-    dmin = warp_min(dmin);
-    dmax = warp_max(dmax);
+    const double gl = warp_min(kgl), gh = warp_max(kgh);
+    double dmin = warp_min(kdmin), dmax = warp_max(kdmax);
     const double S = fmax(fabs(gl), fabs(gh));
     const double inv = S > 0.0 ? 1.0 / S : 1.0;
     for (int r = lane; r < m; r += 32) {
@@ -328,7 +458,7 @@ __device__ void kappa_body(const double* __restrict__ G, BlockState* st, int i, 
     int below = 0;
     if (!(pair == 0 && uncert_s))  // uniform over the pair
       multisect_pair_dispatch(m, d, e2, pair == 0 ? 1 : m, kKappaRounds, pair == 0, pair == 0 ? floor_s : -1.0, &lo,
-                              &hi, &below, half, 1 + pair, s_mask[pair]);
+                              &hi, &below, half, 1 + pair, s_mask[pair], frac_s);
     __syncthreads();  // every warp has read lo_s, hi_s and uncert_s
     if (lane == 0 && half == 0) {
       lo_s[pair] = lo;
@@ -388,7 +518,7 @@ __device__ __forceinline__ void gmatvec4(const double (*Gs)[kMaxW], const double
   __syncthreads();
 }
 
-// sum_r a[r] b[r] over the first w rows, by warp 0 (valid in all its lanes).
+// sum_r a[r] b[r] over the first w rows, by one warp (valid in all its lanes).
 __device__ __forceinline__ double dot_rows(const double* a, const double* b, int w) {
   const int lane = threadIdx.x & 31;
   double t = warp_sum(lane < w ? a[lane] * b[lane] : 0.0);
@@ -398,10 +528,14 @@ __device__ __forceinline__ double dot_rows(const double* a, const double* b, int
 
 // Records of the speculative coordinate steps, per system: for step j =
 // 1..kMaxS, x', r', p' after the step (3 kMaxW) and alpha_j, beta_j,
-// sqrt(max(r'^T G r', 0)); then the number of steps taken.
+// sqrt(max(r'^T G r', 0)); then the number of steps taken, and what the
+// selection needs that does not depend on the condition estimates: ||r_{m+1}||,
+// the threshold of eq. (condy), ||r_{m+1}|| / ||b||, and for step j the
+// threshold of eq. (check) and the relative residual.
 constexpr int kSpecRow = 3 * kMaxW + 3;
 constexpr int kSpecDone = kMaxS * kSpecRow;
-static_assert(kSpecDone + 1 == kSpecDoubles, "spec record layout");
+constexpr int kSpecNorm = kSpecDone + 1, kSpecTj = kSpecNorm + 3, kSpecRel = kSpecTj + kMaxS;
+static_assert(kSpecRel + kMaxS == kSpecDoubles, "spec record layout");
 
 // The coordinate CG steps (Alg. 4 inner loop, Sec. 2.1) on the whole basis of
 // size sbar, before s~_k is known. Because p' and r' after j steps have no
@@ -419,7 +553,7 @@ __device__ void spec_steps(const double* __restrict__ G, const double* __restric
   __shared__ double part[4][32];
   __shared__ double th[kMaxS], sg[kMaxS], gm[kMaxS];
   __shared__ int s_flag;
-  __shared__ double s_alpha, s_beta;
+  __shared__ double s_alpha, s_beta, s_rnn[kMaxS];
   const int t = threadIdx.x;
   const int sbar = st->sbar;
   const int w = 2 * sbar + 1;
@@ -472,17 +606,21 @@ __device__ void spec_steps(const double* __restrict__ G, const double* __restric
     __syncthreads();
     gmatvec4(Gs, rn, w, g, part);
     double* r = rec + (int64_t)(j - 1) * kSpecRow;
-    if (t < 32) {
+    if (t < 64) {
+      // warps 0 and 1 form the same dot product; then one divides while the
+      // other takes the square root
       const double rGr_new = dot_rows(rn, g, w);
       if (t == 0) {
         const double beta = rGr_new / rGr;
-        const double rnn = sqrt(fmax(rGr_new, 0.0));
         r[3 * kMaxW] = alpha;
         r[3 * kMaxW + 1] = beta;
-        r[3 * kMaxW + 2] = rnn;
         s_beta = beta;
-        s_flag = rnn <= eps_star;  // converged: no later step can be taken
         s_alpha = rGr_new;
+      } else if (t == 32) {
+        const double rnn = sqrt(fmax(rGr_new, 0.0));
+        r[3 * kMaxW + 2] = rnn;
+        s_rnn[j - 1] = rnn;
+        s_flag = rnn <= eps_star;  // converged: no later step can be taken
       }
     }
     __syncthreads();
@@ -501,6 +639,21 @@ __device__ void spec_steps(const double* __restrict__ G, const double* __restric
     if (conv) break;
   }
   if (t == 0) rec[kSpecDone] = (double)done;
+  // the selection's own scalars, formed here, beside the condition estimates
+  const double bnorm = st->bnorm;
+  if (t < done) {
+    const double rnn = s_rnn[t];
+    const double cj = st->c_step > 0.0 ? st->c_step * (t + 1) : st->c;
+    rec[kSpecTj + t] = rnn > 0.0 ? eps_star / (cj * kEps * rnn) : CUDART_INF;
+    rec[kSpecRel + t] = rnn / bnorm;
+  } else if (t == 32) {
+    // ||r_{m+1}|| from G: column 1 is rho_0(A) r = r; eq. (condy) takes c_{k,s_max}
+    const double rnorm = sqrt(fmax(Gs[1][1], 0.0));
+    const double c_condy = st->c_step > 0.0 ? st->c_step * st->c_smax : st->c;
+    rec[kSpecNorm] = rnorm;
+    rec[kSpecNorm + 1] = rnorm > 0.0 ? eps_star / (c_condy * kEps * rnorm) : CUDART_INF;
+    rec[kSpecNorm + 2] = rnorm / bnorm;
+  }
 }
 
 // Applies eq. (condy) and eq. (check) to the kappa values and the step
@@ -509,31 +662,31 @@ __device__ void spec_steps(const double* __restrict__ G, const double* __restric
 // coordinates. All loads are issued at once by the CTA's threads into shared
 // memory; thread 0 then decides on shared values only, so the decision does
 // not wait on a chain of dependent global loads.
-__device__ void select_steps(const double* __restrict__ G, BlockState* st, const double* __restrict__ rec,
-                             double* __restrict__ coords, double* __restrict__ hist, double* __restrict__ res_hist,
-                             int res_cap, double* __restrict__ ab_hist, int ab_cap) {
+__device__ void select_steps(BlockState* st, const double* __restrict__ rec, double* __restrict__ coords,
+                             double* __restrict__ hist, double* __restrict__ res_hist, int res_cap,
+                             double* __restrict__ ab_hist, int ab_cap) {
   __shared__ int s_steps;
-  __shared__ double s_sk[kMaxS], s_step[kMaxS][3], s_g11, s_done;
+  __shared__ double s_sk[kMaxS], s_step[kMaxS][3], s_done, s_norm[3], s_tj[kMaxS], s_rel[kMaxS];
   const int t = threadIdx.x;
   const int sbar = st->sbar;
   const int w = 2 * sbar + 1;
   if (t < 3 * sbar) s_step[t / 3][t % 3] = __ldcg(rec + (int64_t)(t / 3) * kSpecRow + 3 * kMaxW + t % 3);
-  if (t >= 64 && t < 64 + sbar) s_sk[t - 64] = __ldcg(&st->sqrt_kappa[t - 64]);
-  if (t == 96) s_g11 = __ldcg(G + 1 * w + 1);
-  if (t == 97) s_done = __ldcg(rec + kSpecDone);
+  if (t >= 64 && t < 64 + sbar) {
+    s_sk[t - 64] = __ldcg(&st->sqrt_kappa[t - 64]);
+    s_tj[t - 64] = __ldcg(rec + kSpecTj + t - 64);
+    s_rel[t - 64] = __ldcg(rec + kSpecRel + t - 64);
+  }
+  if (t >= 96 && t < 99) s_norm[t - 96] = __ldcg(rec + kSpecNorm + t - 96);
+  if (t == 99) s_done = __ldcg(rec + kSpecDone);
   __syncthreads();
   if (t < 32) {
-    // warp 0, lane j - 1 for step j and submatrix i = j: the same scalar
-    // formulas as a serial scan, evaluated for all j at once (an FP64
-    // instruction costs the same for 1 or 32 lanes), then ballots
+    // warp 0, lane j - 1 for step j and submatrix i = j: the decisions of a
+    // serial scan, taken for all j at once (an FP64 instruction costs the same
+    // for 1 or 32 lanes), then ballots
     const int lane = t;
     const int adaptive = st->method == ASCG_ADAPTIVE;
-    const double eps_star = st->eps_star, cc = st->c, bnorm = st->bnorm;
-    // ||r_{m+1}|| from G: column 1 is rho_0(A) r = r
-    const double rnorm = sqrt(fmax(s_g11, 0.0));
-    // eq. (condy) takes c_{k,s_max}
-    const double c_condy = st->c_step > 0.0 ? st->c_step * st->c_smax : cc;
-    const double T = rnorm > 0.0 ? eps_star / (c_condy * kEps * rnorm) : CUDART_INF;
+    const double eps_star = st->eps_star;
+    const double rnorm = s_norm[0], T = s_norm[1];
     int stilde;
     double gamma;
     if (adaptive) {
@@ -556,9 +709,7 @@ __device__ void select_steps(const double* __restrict__ G, BlockState* st, const
     const bool conv = !bd && rnn <= eps_star;
     bool brk = false;
     if (!bd && !conv && adaptive && st->check_in_loop) {
-      const double cj = st->c_step > 0.0 ? st->c_step * j : cc;
-      const double Tj = rnn > 0.0 ? eps_star / (cj * kEps * rnn) : CUDART_INF;
-      brk = gamma >= Tj;
+      brk = gamma >= s_tj[lane < kMaxS ? lane : 0];
     }
     const unsigned ev = __ballot_sync(kFull, j <= nmax && (bd || conv || brk));
     const unsigned cv = __ballot_sync(kFull, conv);
@@ -585,7 +736,7 @@ __device__ void select_steps(const double* __restrict__ G, BlockState* st, const
       st->s_k = steps;
       st->stop = stop;
       st->converged = stop == ASCG_STOP_CONVERGED;
-      st->rel_res = steps > 0 ? s_step[steps - 1][2] / bnorm : rnorm / bnorm;
+      st->rel_res = steps > 0 ? s_rel[steps - 1] : s_norm[2];
       s_steps = steps;
     }
   }
@@ -594,7 +745,7 @@ __device__ void select_steps(const double* __restrict__ G, BlockState* st, const
   // histories of the steps taken: step j (1-based) is iteration m + j
   if (t < steps) {
     const int j = t + 1;
-    const double alpha = s_step[t][0], beta = s_step[t][1], relres = s_step[t][2] / st->bnorm;
+    const double alpha = s_step[t][0], beta = s_step[t][1], relres = s_rel[t];
     const int it = st->m + j;
     if (res_hist && it < res_cap) res_hist[it] = relres;
     if (ab_hist && it - 1 < ab_cap) {
@@ -627,7 +778,7 @@ __device__ void select_steps(const double* __restrict__ G, BlockState* st, const
 // last CTA to finish (a ticket counter per system, reset afterwards; nothing
 // waits) selects s~_k and s_k and writes the outputs. The condition
 // estimates and the steps thus overlap instead of following each other.
-__global__ void __launch_bounds__(128) block_ctrl_kernel(const double* __restrict__ G,
+__global__ void __launch_bounds__(128, 1) block_ctrl_kernel(const double* __restrict__ G,
                                                          const double* __restrict__ th_g,
                                                          const double* __restrict__ sg_g,
                                                          const double* __restrict__ gm_g, BlockState* st,
@@ -642,7 +793,7 @@ __global__ void __launch_bounds__(128) block_ctrl_kernel(const double* __restric
   G += (int64_t)q * g_stride;
   st += q;
   coords += (int64_t)q * c_stride;
-  spec += (int64_t)q * (kSpecDone + 1);
+  spec += (int64_t)q * kSpecDoubles;
   counters += q;
   if (res_hist) res_hist += (int64_t)q * res_cap;
   if (ab_hist) ab_hist += (int64_t)q * 2 * ab_cap;
@@ -663,7 +814,7 @@ __global__ void __launch_bounds__(128) block_ctrl_kernel(const double* __restric
   __syncthreads();
   if (s_ticket != (unsigned)(parts - 1)) return;
   __threadfence();
-  select_steps(G, st, spec, coords, hist, res_hist, res_cap, ab_hist, ab_cap);
+  select_steps(st, spec, coords, hist, res_hist, res_cap, ab_hist, ab_cap);
   if (threadIdx.x == 0) *counters = 0u;
 }
 

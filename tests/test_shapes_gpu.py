@@ -129,3 +129,34 @@ def test_scratch_of_concurrent_calls():
     for t in threads:
         t.join()
     assert not bad
+
+
+@pytest.mark.parametrize("s", range(1, 17))
+@pytest.mark.parametrize("kind", ["dense", "diagonal"])
+def test_condition_estimates_every_order(s, kind):
+    """sqrt(kappa(G_{k,i})) for every order 3 .. 33 against numpy's eigenvalues.
+
+    dense: random Gram matrices of condition below 1e8; diagonal: zero off-diagonals (every minor a product, the small ones
+    rescaled, exact condition numbers). Tolerance: the multisection leaves relative brackets below 1e-9 for both ends, and
+    rounding moves an eigenvalue by at most 64 w eps ||G||, so sqrt(kappa) is within 1e-9 + 32 w eps kappa relatively.
+    """
+    import paper_1701_03989_gb300 as P
+
+    w, eps = 2 * s + 1, 2.0 ** -53
+    rng = np.random.default_rng(s)
+    if kind == "dense":
+        Y = rng.standard_normal((200, w)) * 10.0 ** rng.uniform(-1.5, 0, w)
+        G = Y.T @ Y
+    else:
+        G = np.diag(10.0 ** rng.uniform(-6, 0, w))
+    G = (G + G.T) / 2
+    Gd = torch.from_numpy(G.copy()).cuda()
+    coords = torch.zeros(3 * w, dtype=torch.float64, device="cuda")
+    info, _ = P.ascg_block_step(s, Gd, P.ASCG_ADAPTIVE, np.zeros(s), np.zeros(s), np.ones(s), 200, 1e-8, 1.0, 1, 100, 1.0,
+                                coords)
+    for i in range(1, s + 1):
+        ev = np.linalg.eigvalsh(G[: 2 * i + 1, : 2 * i + 1])
+        kappa = ev[-1] / ev[0]
+        assert kappa < 1e8
+        got = info.sqrt_kappa[i - 1]
+        assert abs(got - np.sqrt(kappa)) <= (1e-9 + 32 * w * eps * kappa) * np.sqrt(kappa), (i, got, kappa)
