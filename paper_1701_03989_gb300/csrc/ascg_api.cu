@@ -532,23 +532,29 @@ ascg_status prepare_steps(ascg_op op, const double* th, const double* sg, const 
     ASCG_TRY(dev_alloc(&w.dtils, (size_t)nd * op->n));
     w.dt_rows = nd;
   }
+  FoldSteps f = {};
+  f.ng = ng;
+  f.nd = nd;
+  f.dtil = w.dtils;
   for (int q = 0; q < ng; ++q) {
     if (!w.oscaled[q]) ASCG_TRY(dev_alloc(&w.oscaled[q], (size_t)op->o_len));
-    ASCG_CUDA(launch_shift_scale(op->o_val, op->o_len, 0.0, 1.0 / gam_of[q], w.oscaled[q], st));
-    ++*launches;
+    f.oscaled[q] = w.oscaled[q];
+    f.oscale[q] = 1.0 / gam_of[q];
   }
-  int made = 0;
   for (int j = 0; j < s; ++j) {
     const double inv = 1.0 / gm[j];
-    const double* dt = d_row[j] < 0 ? op->diag : w.dtils + (int64_t)d_row[j] * op->n;
-    if (d_row[j] == made) {
-      ASCG_CUDA(launch_shift_scale(op->diag, op->n, th[j], inv, w.dtils + (int64_t)made * op->n, st));
-      ++made;
-      ++*launches;
+    if (d_row[j] >= 0) {
+      f.theta[d_row[j]] = th[j];
+      f.dscale[d_row[j]] = inv;
     }
     // sig_j = sigma_{j-1} / gamma_j, exactly 1 when the two are equal (Chebyshev)
     const double sj = j < 1 ? 0.0 : (sg[j - 1] == gm[j] ? 1.0 : sg[j - 1] * inv);
-    out[j] = StepOp{o_slot[j] < 0 ? op->o_val : w.oscaled[o_slot[j]], dt, sj};
+    out[j] = StepOp{o_slot[j] < 0 ? op->o_val : w.oscaled[o_slot[j]],
+                    d_row[j] < 0 ? op->diag : w.dtils + (int64_t)d_row[j] * op->n, sj};
+  }
+  if (ng > 0 || nd > 0) {
+    ASCG_CUDA(launch_fold_steps(op->o_val, op->o_len, op->diag, op->n, f, st));
+    ++*launches;
   }
   return ASCG_OK;
 }

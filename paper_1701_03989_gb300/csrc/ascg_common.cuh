@@ -228,9 +228,17 @@ cudaError_t launch_mpk_split_step(const DevSplit& O, const StepOp& op, double* Y
 // col_emax[c] = max_k emax_part[c * emax_ld + k] for c < w, k < ceil(n/32).
 cudaError_t launch_emax_reduce(const int* emax_part, int64_t emax_ld, int64_t n, int w, int* col_emax,
                                cudaStream_t s, const int* gate = nullptr);
-// dst[i] = (src[i] - theta) * scale, for i < n
-cudaError_t launch_shift_scale(const double* src, int64_t n, double theta, double scale, double* dst,
-                               cudaStream_t s);
+// The folded operators of a basis: O's values times oscale[q] into oscaled[q]
+// (q < ng <= 2), (D - theta[q]) * dscale[q] into row q of dtil (q < nd).
+struct FoldSteps {
+  double* oscaled[2];
+  double oscale[2];
+  double* dtil;
+  double theta[kMaxS], dscale[kMaxS];
+  int ng, nd;
+};
+cudaError_t launch_fold_steps(const double* oval, int64_t o_len, const double* diag, int64_t n, const FoldSteps& f,
+                              cudaStream_t s);
 
 // Gram partials: per CTA, the upper triangle (row-major pair order) of Y^T Y.
 int gram_grid();                // CTAs per launch at most (the SM count)

@@ -95,6 +95,12 @@ constexpr int kDrainWarp0 = kConvWarps, kDrainWarps = 8;  // drain warp d: lane 
 constexpr int kLoadWarp = kDrainWarp0 + kDrainWarps;
 constexpr int kMmaWarp = kLoadWarp + 1, kMma1Warp = kMmaWarp + 1;  // tile 0 and tile 1 issuers
 constexpr int kTcThreads = (kMma1Warp + 1) * 32;                   // 928
+// Registers per thread: 29 warps put 8 on one SM sub-partition, and 8 x 32 x 64
+// would fill its register file, so that no warp of the next kernel could be
+// resident there before the Gram's CTA ends. At 57 registers (64 allocated)
+// the dependent launch after the Gram started late and a 401^2 Newton solve
+// took 49.7 ms instead of 47.2.
+constexpr int kTcRegs = 56;
 constexpr long long kWaitLimit = 1ll << 20;  // polls; with the suspend hint a wait ends within ~2 s
 constexpr long long kTestWaitLimit = 1ll << 12;  // the stall test's limit: a few milliseconds
 static_assert(kFStages % 2 == 0, "a staging slot must belong to one converter group");
@@ -568,7 +574,6 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w_ou
   for (uint32_t o = tid * 16; o < kDStages * kDStageBytes; o += kTcThreads * 16)
     *reinterpret_cast<uint4*>(dstage + o) = make_uint4(0, 0, 0, 0);
   for (int k = tid; k < 2 * kSlices * kTW * kTW; k += kTcThreads) acc_hi[k] = 0u;
-  if (tid < kTW) s_emax[tid] = tid < w ? col_emax[tid] : 0;
   if (tid == 0) {
     *s_err = 0;
     for (int k = 0; k < kFStages; ++k) {
@@ -590,6 +595,10 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w_ou
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  // everything above touches only this CTA: it overlaps the previous kernel
+  pdl_wait();
+  pdl_release();
+  if (tid < kTW) s_emax[tid] = tid < w ? col_emax[tid] : 0;
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -751,12 +760,14 @@ done:
 }
 
 // One matrix: CTA b takes the chunks b, b + gridDim.x, ... of the n rows.
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __maxnreg__(kTcRegs)
     gram_tc_kernel(const __grid_constant__ CUtensorMap ymap, int64_t n, int w, const int* __restrict__ col_emax,
                    double* __restrict__ partials, const TcGuard guard) {
-  pdl_wait();
-  pdl_release();
-  if (guard.gate && !*guard.gate) return;  // uniform, before any barrier or tensor memory
+  // the block's flag was written several kernels ago (see block_advance_kernel)
+  if (guard.gate && !__ldcg(guard.gate)) {  // uniform, before any barrier or tensor memory
+    pdl_wait();
+    return;
+  }
   gram_tc_body(&ymap, w, w, 0, blockIdx.x, (n + kTChunk - 1) / kTChunk, gridDim.x, n, col_emax,
                partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), guard);
 }
@@ -765,58 +776,47 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // CTA q takes item q, whole chunks of one system (rows [row0, row0 + nrows),
 // nrows a multiple of kTChunk), with that system's column exponents
 // (emax_all + sys * kTW). Items of systems with sys_w 0 skip.
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __maxnreg__(kTcRegs)
     gram_tc_items_kernel(const __grid_constant__ CUtensorMap ymap, int w, const GramItem* __restrict__ items,
                          const int* __restrict__ sys_w, const int* __restrict__ emax_all,
                          double* __restrict__ partials) {
   const GramItem it = items[blockIdx.x];
-  pdl_wait();
-  pdl_release();
-  const int wq = sys_w[it.sys];
-  if (wq == 0) return;  // uniform over the CTA, before any barrier
+  const int wq = sys_w[it.sys];  // written before the block's matrix powers steps
+  if (wq == 0) {                 // uniform over the CTA, before any barrier
+    pdl_wait();
+    return;
+  }
   const int64_t nch = it.nrows / kTChunk;
   gram_tc_body(&ymap, w, wq, it.row0, 0, nch, 1, nch * kTChunk, emax_all + (int64_t)it.sys * kTW,
                partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), TcGuard{kWaitLimit, -1, nullptr, nullptr});
 }
 
 // Largest biased exponent of each column, reduced into col_emax (zeroed
-// before the launch) with one atomicMax per column and CTA. Rows are split
-// into even-sized ranges; 16-byte loads, four in flight per thread.
-constexpr int kExpBlocks = 1216;
-__global__ void __launch_bounds__(256) col_exponent_kernel(int64_t n, int w, const double* __restrict__ Y,
-                                                           int64_t ldY, int* __restrict__ col_emax) {
-  __shared__ unsigned red[8][kTW];
-  const int64_t per = (((n + gridDim.x - 1) / gridDim.x) + 1) & ~1ll;
-  const int64_t r0 = (int64_t)blockIdx.x * per;
-  const int64_t r1 = n < r0 + per ? n : r0 + per;
-  const int64_t full = r1 > r0 ? (r1 - r0) >> 1 : 0;  // whole double2 slots
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto ex = [](double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu; };
-  for (int a = 0; a < w; ++a) {
-    const double2* col = reinterpret_cast<const double2*>(Y + (int64_t)a * ldY + r0);
-    unsigned m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-    int64_t q = threadIdx.x;
-    for (; q + 768 < full; q += 1024) {
-      const double2 v0 = __ldcs(col + q), v1 = __ldcs(col + q + 256), v2 = __ldcs(col + q + 512),
-                    v3 = __ldcs(col + q + 768);
-      m0 = max(m0, max(ex(v0.x), ex(v0.y)));
-      m1 = max(m1, max(ex(v1.x), ex(v1.y)));
-      m2 = max(m2, max(ex(v2.x), ex(v2.y)));
-      m3 = max(m3, max(ex(v3.x), ex(v3.y)));
-    }
-    for (; q < full; q += 256) {
-      const double2 v = __ldcs(col + q);
-      m0 = max(m0, max(ex(v.x), ex(v.y)));
-    }
-    if (threadIdx.x == 0 && r0 + 2 * full < r1) m0 = max(m0, ex(Y[(int64_t)a * ldY + r0 + 2 * full]));
-    const unsigned m = __reduce_max_sync(0xffffffffu, max(max(m0, m1), max(m2, m3)));
-    if (lane == 0) red[warp][a] = m;
-  }
+// before the launch): CTA (b, c) takes kExpPairs double2 of column c, eight
+// 16-byte loads in flight per thread, and ends in one atomicMax. HBM-bound:
+// 2^21 x 33 in EXPTIME us (the ranges of all columns in one CTA, column after
+// column with a reduction each, took 128 us).
+constexpr int kExpPairs = 256 * 8;
+__global__ void __launch_bounds__(256) col_exponent_kernel(int64_t n, const double* __restrict__ Y, int64_t ldY,
+                                                           int* __restrict__ col_emax) {
+  pdl_release();
+  __shared__ unsigned red[8];
+  const double* col = Y + (int64_t)blockIdx.y * ldY;
+  const double2* col2 = reinterpret_cast<const double2*>(col);
+  const int64_t pairs = n >> 1, q0 = (int64_t)blockIdx.x * kExpPairs + threadIdx.x;
+  unsigned m = 0;
+  double2 v[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) v[u] = q0 + 256 * u < pairs ? __ldcs(col2 + q0 + 256 * u) : make_double2(0.0, 0.0);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) m = max(m, max(biased_exp(v[u].x), biased_exp(v[u].y)));
+  if (blockIdx.x == 0 && threadIdx.x == 0 && (n & 1)) m = max(m, biased_exp(col[n - 1]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x < w) {
-    unsigned m = 0;
-    for (int g = 0; g < 8; ++g) m = max(m, red[g][threadIdx.x]);
-    if (m > 0) atomicMax(col_emax + threadIdx.x, (int)m);
+  if (threadIdx.x < 8) {
+    m = __reduce_max_sync(0xffu, red[threadIdx.x]);
+    if (threadIdx.x == 0 && m > 0) atomicMax(col_emax + blockIdx.y, (int)m);
   }
 }
 
@@ -949,12 +949,13 @@ __global__ void __launch_bounds__(kRThreads, 1)
     recover_tc_kernel(const __grid_constant__ CUtensorMap ymap, int64_t n, int w, const int* __restrict__ col_emax,
                       const double* __restrict__ coords, double* __restrict__ x, double* __restrict__ r,
                       double* __restrict__ p, const TcGuard guard) {
-  pdl_wait();
-  pdl_release();
   // uniform, before any barrier or tensor memory: a block enqueued ahead with
   // nothing to do, or one whose Gram already failed (its error word is set),
-  // leaves x, r and p alone
-  if ((guard.gate && !*guard.gate) || (guard.err && *guard.err != 0)) return;
+  // leaves x, r and p alone. Both words were written several kernels ago.
+  if ((guard.gate && !__ldcg(guard.gate)) || (guard.err && __ldcg(guard.err) != 0)) {
+    pdl_wait();
+    return;
+  }
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* astage = smem + kRAOff;
   unsigned char* fstage = smem + kRFOff;
@@ -979,7 +980,6 @@ __global__ void __launch_bounds__(kRThreads, 1)
     *reinterpret_cast<uint4*>(astage + o) = make_uint4(0, 0, 0, 0);
   for (uint32_t o = tid * 16; o < kRBBytes; o += kRThreads * 16)
     *reinterpret_cast<uint4*>(bop + o) = make_uint4(0, 0, 0, 0);
-  if (tid < kTW) s_emax[tid] = tid < w ? col_emax[tid] : 0;
   if (tid < 4) s_fv[tid] = 0;
   if (tid == 0) {
     *s_err = 0;
@@ -998,6 +998,10 @@ __global__ void __launch_bounds__(kRThreads, 1)
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(smem_u32(tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  // everything above touches only this CTA: it overlaps the previous kernel
+  pdl_wait();
+  pdl_release();
+  if (tid < kTW) s_emax[tid] = tid < w ? col_emax[tid] : 0;
   __syncthreads();
   // coefficients: u_vj = c_vj 2^(E_j - 55), E_j = emax_j - 1022; per vector the
   // largest biased exponent f_v; a NaN or infinite column or coefficient
@@ -1235,11 +1239,7 @@ cudaError_t launch_gram_tc(int64_t n, int w, const double* Y, int64_t ldY, int* 
   e = encode_map(&map, Y, n, w, ldY);
   if (e != cudaSuccess) return e;
   if (!emax_ready) {
-    e = cudaMemsetAsync(exp_parts, 0, sizeof(int) * kTW, s);
-    if (e != cudaSuccess) return e;
-    const int64_t eb = (n + 255) / 256;
-    col_exponent_kernel<<<(int)(eb < kExpBlocks ? eb : kExpBlocks), 256, 0, s>>>(n, w, Y, ldY, exp_parts);
-    e = cudaGetLastError();
+    e = launch_col_exponents(n, w, Y, ldY, exp_parts, s);
     if (e != cudaSuccess) return e;
   }
   const TcGuard guard{stall_test ? kTestWaitLimit : kWaitLimit, stall_test ? 0 : -1, err, gate};
@@ -1292,8 +1292,8 @@ cudaError_t launch_col_exponents(int64_t n, int w, const double* Y, int64_t ldY,
   if (w < 1 || w > kTW || n < 1) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(col_emax, 0, sizeof(int) * kTW, s);
   if (e != cudaSuccess) return e;
-  const int64_t eb = (n + 255) / 256;
-  col_exponent_kernel<<<(int)(eb < kExpBlocks ? eb : kExpBlocks), 256, 0, s>>>(n, w, Y, ldY, col_emax);
+  const int64_t eb = ((n >> 1) + kExpPairs - 1) / kExpPairs;
+  col_exponent_kernel<<<dim3((unsigned)(eb > 0 ? eb : 1), (unsigned)w), 256, 0, s>>>(n, Y, ldY, col_emax);
   return cudaGetLastError();
 }
 

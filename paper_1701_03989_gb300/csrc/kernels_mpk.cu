@@ -216,10 +216,23 @@ __global__ void __launch_bounds__(1024) emax_reduce_kernel(const int* __restrict
   }
 }
 
-__global__ void shift_scale_kernel(const double* __restrict__ src, int64_t n, double theta, double scale,
-                                   double* __restrict__ dst) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = (src[i] - theta) * scale;
+// Folds the basis coefficients into the operator: scaled copies of O's values
+// (both in one pass over them) and, per distinct (theta, gamma), a vector
+// (D - theta) / gamma, all of them in one pass over D.
+__global__ void __launch_bounds__(256) fold_steps_kernel(const double* __restrict__ oval, int64_t o_len,
+                                                         const double* __restrict__ diag, int64_t n, const FoldSteps f) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (f.ng > 0)
+    for (int64_t i = i0; i < o_len; i += stride) {
+      const double v = oval[i];
+      f.oscaled[0][i] = (v - 0.0) * f.oscale[0];
+      if (f.ng > 1) f.oscaled[1][i] = (v - 0.0) * f.oscale[1];
+    }
+  if (f.nd > 0)
+    for (int64_t i = i0; i < n; i += stride) {
+      const double d = diag[i];
+      for (int q = 0; q < f.nd; ++q) f.dtil[(int64_t)q * n + i] = (d - f.theta[q]) * f.dscale[q];
+    }
 }
 
 // x += Y x', r = Y r', p = Y p' over the first w columns (eq. coords).
@@ -390,9 +403,9 @@ cudaError_t launch_emax_reduce(const int* emax_part, int64_t emax_ld, int64_t n,
   return launch_pdl(emax_reduce_kernel, w, 1024, s, emax_part, emax_ld, col_emax, gate);
 }
 
-cudaError_t launch_shift_scale(const double* src, int64_t n, double theta, double scale, double* dst,
-                               cudaStream_t s) {
-  shift_scale_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, s>>>(src, n, theta, scale, dst);
+cudaError_t launch_fold_steps(const double* oval, int64_t o_len, const double* diag, int64_t n, const FoldSteps& f,
+                              cudaStream_t s) {
+  fold_steps_kernel<<<grid_for(o_len > n ? o_len : n, 256, 152 * 16), 256, 0, s>>>(oval, o_len, diag, n, f);
   return cudaGetLastError();
 }
 
