@@ -321,14 +321,23 @@ bool gram_tc_fits(int64_t n);
 // Tensor-core Gram of many systems whose bases are row ranges of one matrix
 // Y (rows x w used, leading dimension ldY, rows a multiple of 1024): items
 // are whole 1024-row chunks of one system each (GramItem rows in Y, nrows a
-// multiple of 1024, at most 8 chunks); items of systems with sys_w 0 skip.
-// Each item takes its system's column exponents (emax_all: 33 ints per
-// system, filled by launch_tc_items_exponents or the matrix powers steps) and
-// writes w(w+1)/2 partials, of which the pairs of its system's own sys_w
-// columns hold values.
-cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramItem* items,
-                                 int nitems, const int* sys_w, const int* emax_all, double* partials,
-                                 cudaStream_t s);
+// multiple of 1024, at most 8 chunks), each run as one or more pieces of whole
+// chunks; pieces of systems with sys_w 0 skip.
+// Each piece takes its system's column exponents (emax_all: 33 ints per
+// system, filled by launch_tc_items_exponents or the matrix powers steps).
+// Each item gets w(w+1)/2 partials, of which the pairs of its system's own
+// sys_w columns hold values. Where an item has several pieces: sums, w(w+1)
+// words per item, and tickets, one per item, zero on entry and left zero.
+struct GramPiece {
+  int64_t row0;
+  int nrows;
+  int sys;
+  int item;
+  int pieces;  // of this item
+};
+cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramPiece* pieces,
+                                 int npieces, const int* sys_w, const int* emax_all, double* partials,
+                                 unsigned long long* sums, unsigned* tickets, cudaStream_t s);
 // The column exponents of every item's system (emax_all zeroed here), by a pass over Y.
 cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramItem* items, int nitems,
                                       const int* sys_w, int nsys, int* emax_all, cudaStream_t s);

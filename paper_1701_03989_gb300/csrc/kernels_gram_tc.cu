@@ -541,17 +541,28 @@ __device__ __forceinline__ void drain_quarter(uint32_t tq, int a, int w, uint32_
   }
 }
 
+// A partial formed by several CTAs: each adds its exact integer sums to sums
+// (hi and lo of every pair, w_out (w_out + 1) / 2 each, zero before the first)
+// and counts itself in ticket (zero before the first; 2^16 marks one that gave
+// up); the last one forms the partial from the totals and leaves both zero.
+// Integer sums do not depend on the split, so neither does the partial.
+struct PieceSums {
+  unsigned long long* sums;
+  unsigned* ticket;
+  int pieces;  // 1: nothing to add up
+};
+
 // The Gram partial of the chunks ch = c_lo, c_lo + c_step, ... < c_hi of the
 // rows [row_base, row_base + n_local) of the tensor map's matrix (chunk ch
 // starts at row row_base + ch * kTChunk), over the first w columns (the others
 // count as zero) with the column exponents col_emax, written to out[w_out
 // (w_out + 1) / 2], w <= w_out. Run by a whole CTA of kTcThreads. guard: the
 // wait limit, where a wait that ran out is reported, and the stall test's
-// stage (see TcGuard).
+// stage (see TcGuard). ps: this CTA's part in a sum of several (see PieceSums).
 __device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w_out, int w, int64_t row_base, int64_t c_lo,
                                              int64_t c_hi, int64_t c_step, int64_t n_local,
                                              const int* __restrict__ col_emax, double* __restrict__ out,
-                                             const TcGuard guard) {
+                                             const TcGuard guard, const PieceSums ps) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* dstage = smem + kDOff;
   unsigned char* fstage = smem + kFOff;
@@ -734,23 +745,59 @@ done:
   const int ok = !*s_err;
   if (!ok && tid == 0 && guard.err) atomicExch(guard.err, (int)ASCG_ERR_TIMEOUT);
   const int np = w_out * (w_out + 1) / 2;
-  for (int p = tid; p < np; p += kTcThreads) {
-    int a = 0, rem = p;
-    while (rem >= w_out - a) {
-      rem -= w_out - a;
-      ++a;
+  // pair p of the triangle: its words in the CTA's sums
+  const auto pair_of = [&](int p, int* a, int* b) {
+    int ra = 0, rem = p;
+    while (rem >= w_out - ra) {
+      rem -= w_out - ra;
+      ++ra;
     }
-    const int b = a + rem;
-    double v;
-    if (!ok || s_emax[a] == 0x7ff || s_emax[b] == 0x7ff) {
-      v = CUDART_NAN;
-    } else {
+    *a = ra;
+    *b = ra + rem;
+  };
+  bool write = true, good = ok != 0;
+  if (ps.pieces > 1) {  // uniform
+    for (int p = tid; p < np; p += kTcThreads) {
+      int a, b;
+      pair_of(p, &a, &b);
       const long long hi = slice_value(acc_hi, a * kTW + b), lo = slice_value(acc_lo, a * kTW + b);
-      // G_ab = 2^(E_a + E_b - 14) (hi 2^-24 + lo 2^-56), E = emax - 1022
-      const double s = ldexp((double)hi, -24) + ldexp((double)lo, -56);
-      v = ldexp(s, s_emax[a] + s_emax[b] - 2058);
+      if (hi != 0) atomicAdd(ps.sums + p, (unsigned long long)hi);
+      if (lo != 0) atomicAdd(ps.sums + np + p, (unsigned long long)lo);
     }
-    out[p] = v;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) tslot[1] = atomicAdd(ps.ticket, ok ? 1u : 0x10001u);
+    __syncthreads();
+    const uint32_t tick = tslot[1];
+    write = (tick & 0xffffu) == (uint32_t)(ps.pieces - 1);
+    good = good && (tick >> 16) == 0;
+    if (write) {
+      __threadfence();
+      if (tid == 0) *ps.ticket = 0u;
+    }
+  }
+  if (write) {
+    for (int p = tid; p < np; p += kTcThreads) {
+      int a, b;
+      pair_of(p, &a, &b);
+      long long hi, lo;
+      if (ps.pieces > 1) {
+        hi = (long long)atomicExch(ps.sums + p, 0ull);
+        lo = (long long)atomicExch(ps.sums + np + p, 0ull);
+      } else {
+        hi = slice_value(acc_hi, a * kTW + b);
+        lo = slice_value(acc_lo, a * kTW + b);
+      }
+      double v;
+      if (!good || s_emax[a] == 0x7ff || s_emax[b] == 0x7ff) {
+        v = CUDART_NAN;
+      } else {
+        // G_ab = 2^(E_a + E_b - 14) (hi 2^-24 + lo 2^-56), E = emax - 1022
+        const double s = ldexp((double)hi, -24) + ldexp((double)lo, -56);
+        v = ldexp(s, s_emax[a] + s_emax[b] - 2058);
+      }
+      out[p] = v;
+    }
   }
   if (warp == kMmaWarp) {
     __syncwarp();
@@ -769,32 +816,35 @@ __global__ void __maxnreg__(kTcRegs)
     return;
   }
   gram_tc_body(&ymap, w, w, 0, blockIdx.x, (n + kTChunk - 1) / kTChunk, gridDim.x, n, col_emax,
-               partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), guard);
+               partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), guard, PieceSums{nullptr, nullptr, 1});
 }
 
 // Many systems whose bases are row ranges of one matrix (the tensor map's):
-// CTA q takes item q, whole chunks of one system (rows [row0, row0 + nrows),
-// nrows a multiple of kTChunk), with that system's column exponents
-// (emax_all + sys * kTW). Items of systems with sys_w 0 skip.
+// CTA q takes piece q, whole chunks of one item of one system (rows [row0,
+// row0 + nrows), nrows a multiple of kTChunk), with that system's column
+// exponents (emax_all + sys * kTW). Pieces of systems with sys_w 0 skip.
 __global__ void __maxnreg__(kTcRegs)
-    gram_tc_items_kernel(const __grid_constant__ CUtensorMap ymap, int w, const GramItem* __restrict__ items,
+    gram_tc_items_kernel(const __grid_constant__ CUtensorMap ymap, int w, const GramPiece* __restrict__ pieces,
                          const int* __restrict__ sys_w, const int* __restrict__ emax_all,
-                         double* __restrict__ partials) {
-  const GramItem it = items[blockIdx.x];
+                         double* __restrict__ partials, unsigned long long* __restrict__ sums,
+                         unsigned* __restrict__ tickets) {
+  const GramPiece it = pieces[blockIdx.x];
   const int wq = sys_w[it.sys];  // written before the block's matrix powers steps
   if (wq == 0) {                 // uniform over the CTA, before any barrier
     pdl_wait();
     return;
   }
   const int64_t nch = it.nrows / kTChunk;
+  const int np = w * (w + 1) / 2;
   gram_tc_body(&ymap, w, wq, it.row0, 0, nch, 1, nch * kTChunk, emax_all + (int64_t)it.sys * kTW,
-               partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), TcGuard{kWaitLimit, -1, nullptr, nullptr});
+               partials + (int64_t)it.item * np, TcGuard{kWaitLimit, -1, nullptr, nullptr},
+               PieceSums{sums + (int64_t)it.item * 2 * np, tickets + it.item, it.pieces});
 }
 
 // Largest biased exponent of each column, reduced into col_emax (zeroed
 // before the launch): CTA (b, c) takes kExpPairs double2 of column c, eight
 // 16-byte loads in flight per thread, and ends in one atomicMax. HBM-bound:
-// 2^21 x 33 in EXPTIME us (the ranges of all columns in one CTA, column after
+// 2^21 x 33 (554 MB) in about 90 us (the ranges of all columns in one CTA, column after
 // column with a reduction each, took 128 us).
 constexpr int kExpPairs = 256 * 8;
 __global__ void __launch_bounds__(256) col_exponent_kernel(int64_t n, const double* __restrict__ Y, int64_t ldY,
@@ -1247,10 +1297,10 @@ cudaError_t launch_gram_tc(int64_t n, int w, const double* Y, int64_t ldY, int* 
                        guard);
 }
 
-cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramItem* items,
-                                 int nitems, const int* sys_w, const int* emax_all, double* partials,
-                                 cudaStream_t s) {
-  if (nitems < 1) return cudaSuccess;
+cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramPiece* pieces,
+                                 int npieces, const int* sys_w, const int* emax_all, double* partials,
+                                 unsigned long long* sums, unsigned* tickets, cudaStream_t s) {
+  if (npieces < 1) return cudaSuccess;
   if (!gram_tc_applies(w) || !gram_tc_aligned(Y, ldY) || rows < 1 || rows > 0x7fffffffll || rows > ldY ||
       (rows % kTChunk) != 0)
     return cudaErrorInvalidValue;
@@ -1259,8 +1309,8 @@ cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t ro
   CUtensorMap map;
   e = encode_map(&map, Y, rows, w, ldY);
   if (e != cudaSuccess) return e;
-  return launch_pdl_ex(gram_tc_items_kernel, dim3(nitems), dim3(kTcThreads), kTcSmem, s, map, w, items, sys_w, emax_all,
-                       partials);
+  return launch_pdl_ex(gram_tc_items_kernel, dim3(npieces), dim3(kTcThreads), kTcSmem, s, map, w, pieces, sys_w,
+                       emax_all, partials, sums, tickets);
 }
 
 cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramItem* items, int nitems,

@@ -361,6 +361,30 @@ class Lockstep {
   static int64_t row_items_of(int64_t n) { return (n + kRowItem - 1) / kRowItem; }
   // Tensor-core Gram items: up to kTcItemRows rows (whole 1024-row chunks) each.
   static constexpr int64_t kTcItemRows = 8192;
+  // Pieces of the items (GramPiece), one CTA each. With few items (at most
+  // kSplitItems) an item is cut into pieces of about a third of the chunks per
+  // SM, so that a handful of systems still covers the SMs: a CTA takes about 5
+  // us for the launch, pipeline fill and epilogue and 9 us per chunk, and with
+  // whole items a 93057-row system alone had 12 CTAs of 78 us. 32 systems of
+  // 1e3..1e5 rows: 190.4 -> 182.2 ms a batch; 16 served requests: 334 -> 330.
+  static constexpr int kSplitItems = 256;
+  static std::vector<GramPiece> pieces_of(const std::vector<GramItem>& items) {
+    std::vector<GramPiece> out;
+    int64_t chunks = 0;
+    for (const GramItem& it : items) chunks += it.nrows / Arena::kRowAlign;
+    const int64_t most = kTcItemRows / Arena::kRowAlign;
+    const int64_t per = (int)items.size() > kSplitItems
+                            ? most
+                            : std::max<int64_t>(1, std::min<int64_t>(most, chunks / (3 * gram_grid())));
+    const int64_t rows = per * Arena::kRowAlign;
+    for (size_t i = 0; i < items.size(); ++i) {
+      const int np = (int)((items[i].nrows + rows - 1) / rows);
+      for (int64_t r = 0; r < items[i].nrows; r += rows)
+        out.push_back(GramPiece{items[i].row0 + r, (int)std::min<int64_t>(rows, items[i].nrows - r), items[i].sys,
+                                (int)i, np});
+    }
+    return out;
+  }
   static int64_t tc_items_of(int64_t n) { return (Arena::rounded(n) + kTcItemRows - 1) / kTcItemRows; }
   // Basis bytes of a system of n rows: 2 s_max + 1 columns of round_up(n, 1024).
   static size_t basis_bytes(int s_max, int64_t n) {
@@ -527,7 +551,7 @@ class Lockstep {
     int* d_wtc = d_int_ + kWTc * lanes_;
     int* d_tc0 = d_int_ + kTcItem0 * lanes_;
     int* d_tcn = d_int_ + kTcNItems * lanes_;
-    const int nr = (int)ritems_.size(), ng = (int)gitems_.size(), nt = (int)titems_.size();
+    const int nr = (int)ritems_.size(), ng = (int)gitems_.size();
     const bool item_gram = n_tc < count_active();
     const bool tc_gram = n_tc > 0;
     const int Wb = 2 * max_sbar + 1;
@@ -595,7 +619,7 @@ class Lockstep {
     int* d_wtc = d_int_ + kWTc * lanes_;
     int* d_tc0 = d_int_ + kTcItem0 * lanes_;
     int* d_tcn = d_int_ + kTcNItems * lanes_;
-    const int nr = (int)ritems_.size(), ng = (int)gitems_.size(), nt = (int)titems_.size();
+    const int nr = (int)ritems_.size(), ng = (int)gitems_.size();
     const int Wb = 2 * max_sbar + 1;
     // the steps record the column exponents that the tensor-core Gram needs
     if (tc_gram) LS_CUDA(cudaMemsetAsync(d_emax_, 0, sizeof(int) * kMaxW * hi_, s_));
@@ -608,7 +632,8 @@ class Lockstep {
       LS_CUDA(launch_gram_items_finalize(Wb, d_partials_, d_item0, d_nitems, d_wi, hi_, d_G_, kGStride, moments_, s_));
     }
     if (tc_gram) {  // every tensor-core lane in one launch over the shared basis matrix
-      LS_CUDA(launch_gram_tc_items(Wb, ybase_, yld_, yld_, d_titems_, nt, d_wtc, d_emax_, d_tpart_, s_));
+      LS_CUDA(launch_gram_tc_items(Wb, ybase_, yld_, yld_, d_pieces_, (int)pieces_.size(), d_wtc, d_emax_, d_tpart_,
+                                   d_psums_, d_ptick_, s_));
       LS_CUDA(launch_gram_items_finalize(Wb, d_tpart_, d_tc0, d_tcn, d_wtc, hi_, d_G_, kGStride, false, s_));
     }
     LS_CUDA(launch_block_ctrl_batch(d_G_, kGStride, d_params_, d_params_ + kMaxS, d_params_ + 2 * kMaxS, d_bst_,
@@ -892,14 +917,24 @@ class Lockstep {
     return c;
   }
 
-  ascg_status grow_titems(int64_t titems) {
+  ascg_status grow_titems(int64_t titems, int64_t pieces) {
     if (titems > tcap_items_) {
       LS_CUDA(cudaStreamSynchronize(s_));
-      dfree(d_titems_);
       dfree(d_tpart_);
       tcap_items_ = std::max<int64_t>(titems, 2 * tcap_items_);
-      LS_TRY(dalloc(&d_titems_, (size_t)tcap_items_));
       LS_TRY(dalloc(&d_tpart_, (size_t)tcap_items_ * tcnp_));
+    }
+    if (pieces > pcap_) {
+      LS_CUDA(cudaStreamSynchronize(s_));
+      dfree(d_pieces_);
+      pcap_ = std::max<int64_t>(pieces, 2 * pcap_);
+      LS_TRY(dalloc(&d_pieces_, (size_t)pcap_));
+    }
+    if (!d_psums_) {  // the sums of split items, left zero by every block
+      LS_TRY(dalloc(&d_psums_, (size_t)kSplitItems * 2 * tcnp_));
+      LS_TRY(dalloc(&d_ptick_, (size_t)kSplitItems));
+      LS_CUDA(cudaMemsetAsync(d_psums_, 0, sizeof(unsigned long long) * kSplitItems * 2 * tcnp_, s_));
+      LS_CUDA(cudaMemsetAsync(d_ptick_, 0, sizeof(unsigned) * kSplitItems, s_));
     }
     return ASCG_OK;
   }
@@ -979,9 +1014,11 @@ class Lockstep {
     }
     LS_TRY(grow_items((int64_t)ritems_.size(), (int64_t)gitems_.size()));
     LS_TRY(grow_mitems((int64_t)mitems_.size()));
-    LS_TRY(grow_titems((int64_t)titems_.size()));
-    if (!titems_.empty())
-      LS_CUDA(cudaMemcpyAsync(d_titems_, titems_.data(), sizeof(GramItem) * titems_.size(), cudaMemcpyHostToDevice, s_));
+    pieces_ = pieces_of(titems_);
+    LS_TRY(grow_titems((int64_t)titems_.size(), (int64_t)pieces_.size()));
+    if (!pieces_.empty())
+      LS_CUDA(cudaMemcpyAsync(d_pieces_, pieces_.data(), sizeof(GramPiece) * pieces_.size(), cudaMemcpyHostToDevice,
+                              s_));
     if (!ritems_.empty())
       LS_CUDA(cudaMemcpyAsync(d_ritems_, ritems_.data(), sizeof(RowItem) * ritems_.size(), cudaMemcpyHostToDevice, s_));
     if (!mitems_.empty())
@@ -1011,7 +1048,7 @@ class Lockstep {
     drop_graphs();
     dfree(d_desc_); dfree(d_bst_); dfree(d_G_); dfree(d_coords_); dfree(d_int_); dfree(d_sums_); dfree(d_params_);
     dfree(d_res_hist_); dfree(d_ab_hist_); dfree(d_ritems_); dfree(d_mitems_); dfree(d_gitems_); dfree(d_partials_);
-    dfree(d_titems_); dfree(d_tpart_); dfree(d_emax_); dfree(d_spec_); dfree(d_tickets_);
+    dfree(d_pieces_); dfree(d_psums_); dfree(d_ptick_); dfree(d_tpart_); dfree(d_emax_); dfree(d_spec_); dfree(d_tickets_);
     dfree(d_run_); dfree(d_iter_); dfree(d_seq_);
     hfree(h_desc_); hfree(h_bst_); hfree(h_int_); hfree(h_sums_);
   }
@@ -1049,7 +1086,11 @@ class Lockstep {
   double* d_partials_ = nullptr;
   double* ybase_ = nullptr;  // the shared basis matrix (leading dimension yld_)
   int64_t yld_ = 0;
-  GramItem* d_titems_ = nullptr;  // tensor-core Gram items (row ranges in the shared matrix)
+  std::vector<GramPiece> pieces_;
+  GramPiece* d_pieces_ = nullptr;  // tensor-core Gram items (row ranges in the shared matrix) in pieces
+  unsigned long long* d_psums_ = nullptr;  // integer sums of split items
+  unsigned* d_ptick_ = nullptr;            // and their tickets
+  int64_t pcap_ = 0;
   double* d_tpart_ = nullptr;     // their partials, tcnp_ each
   int* d_emax_ = nullptr;         // per-lane column exponents, kMaxW each
   int64_t tcap_items_ = 0;
@@ -1488,10 +1529,13 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
     int *ints = nullptr, *emax = nullptr;
     SysDesc* desc = nullptr;
     GramItem *items = nullptr, *titems = nullptr;
+    GramPiece* pieces = nullptr;
+    unsigned long long* psums = nullptr;
+    unsigned* ptick = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     ~Bufs() {
       dfree(Y); dfree(G); dfree(part); dfree(tpart); dfree(ints); dfree(emax); dfree(desc); dfree(items);
-      dfree(titems);
+      dfree(titems); dfree(pieces); dfree(psums); dfree(ptick);
       if (e0) cudaEventDestroy(e0);
       if (e1) cudaEventDestroy(e1);
     }
@@ -1507,6 +1551,11 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
   LS_TRY(dalloc(&B.desc, 1));
   LS_TRY(dalloc(&B.items, (size_t)max_items));
   LS_TRY(dalloc(&B.titems, (size_t)max_titems));
+  LS_TRY(dalloc(&B.pieces, (size_t)(ld / Arena::kRowAlign + 1)));
+  LS_TRY(dalloc(&B.psums, (size_t)Lockstep::kSplitItems * 2 * np));
+  LS_TRY(dalloc(&B.ptick, (size_t)Lockstep::kSplitItems));
+  LS_CUDA(cudaMemsetAsync(B.psums, 0, sizeof(unsigned long long) * Lockstep::kSplitItems * 2 * np, s));
+  LS_CUDA(cudaMemsetAsync(B.ptick, 0, sizeof(unsigned) * Lockstep::kSplitItems, s));
   LS_CUDA(cudaEventCreate(&B.e0));
   LS_CUDA(cudaEventCreate(&B.e1));
   LS_CUDA(launch_fill_uniform(B.Y, (int64_t)w * ld, 0x5eed5eedull, s));
@@ -1529,6 +1578,8 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
     LS_CUDA(cudaMemcpyAsync(B.desc, &d, sizeof(d), cudaMemcpyHostToDevice, s));
     LS_CUDA(cudaMemcpyAsync(B.items, items.data(), sizeof(GramItem) * ng, cudaMemcpyHostToDevice, s));
     LS_CUDA(cudaMemcpyAsync(B.titems, titems.data(), sizeof(GramItem) * nt, cudaMemcpyHostToDevice, s));
+    const std::vector<GramPiece> pieces = Lockstep::pieces_of(titems);
+    LS_CUDA(cudaMemcpyAsync(B.pieces, pieces.data(), sizeof(GramPiece) * pieces.size(), cudaMemcpyHostToDevice, s));
     LS_CUDA(cudaMemcpyAsync(B.ints, ints, sizeof(ints), cudaMemcpyHostToDevice, s));
     // a solve's exponents come from its matrix powers steps: not timed
     LS_CUDA(launch_tc_items_exponents(w, B.Y, ld, B.titems, nt, B.ints, 1, B.emax, s));
@@ -1545,7 +1596,8 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
       LS_CUDA(cudaEventElapsedTime(&ms, B.e0, B.e1));
       if (rep > 0) a[rep - 1] = ms;
       LS_CUDA(cudaEventRecord(B.e0, s));
-      LS_CUDA(launch_gram_tc_items(w, B.Y, ld, ld, B.titems, nt, B.ints, B.emax, B.tpart, s));
+      LS_CUDA(launch_gram_tc_items(w, B.Y, ld, ld, B.pieces, (int)pieces.size(), B.ints, B.emax, B.tpart, B.psums,
+                                   B.ptick, s));
       LS_CUDA(launch_gram_items_finalize(w, B.tpart, B.ints + 3, B.ints + 4, B.ints, 1, B.G, kMaxW * kMaxW, false, s));
       LS_CUDA(cudaEventRecord(B.e1, s));
       LS_CUDA(cudaEventSynchronize(B.e1));

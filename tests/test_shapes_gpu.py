@@ -160,3 +160,41 @@ def test_condition_estimates_every_order(s, kind):
         assert kappa < 1e8
         got = info.sqrt_kappa[i - 1]
         assert abs(got - np.sqrt(kappa)) <= (1e-9 + 32 * w * eps * kappa) * np.sqrt(kappa), (i, got, kappa)
+
+
+def test_gram_pieces_do_not_change_a_bit():
+    """A system's tensor-core Gram alone (its items cut into one-chunk pieces) and beside enough rows that no item is cut:
+    the integer sums do not depend on the cut, so x and the iteration count are the same bit for bit."""
+    import paper_1701_03989_gb300 as P
+
+    def system(m, seed):
+        n = m ** 3
+        i = np.arange(n)
+        cols, keep = [], []
+        for s in (m * m, m, 1, 0, -1, -m, -m * m):
+            cols.append(i - s)
+            keep.append(np.ones(n, bool) if s == 0 else
+                        (((i // abs(s)) % m > 0) if s > 0 else ((i // abs(s)) % m < m - 1)))
+        cols, keep = np.stack(cols, 1), np.stack(keep, 1)
+        vals = np.full((n, 7), -1.0 / 6)
+        vals[:, 3] = 1.0
+        rowptr = np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int64)
+        op = P.ascg_op_create_csr(n, int(rowptr[-1]), rowptr, cols[keep].astype(np.int32), vals[keep], 0)
+        b = np.random.default_rng(seed).uniform(-1, 1, n)
+        return op, torch.from_numpy(b).cuda()
+
+    small = [system(m, m) for m in (10, 13, 27, 33)]  # 1, 3, 20 and 36 chunks
+    big = [system(103, 7), system(104, 8)]            # 2166 chunks: more than 256 items
+    o = P.make_options(s_max=8, eps_target=1e-8, max_iters=60)
+
+    def run(members):
+        xs = [torch.zeros_like(b) for _, b in members]
+        res, _ = P.ascg_solve_batch([op for op, _ in members], [b for _, b in members], xs, o)
+        return [(x.cpu().numpy(), r.iters, r.blocks) for x, r in zip(xs, res)]
+
+    mixed = run(small + big)
+    for k, m in enumerate(small):
+        x, it, bl = run([m])[0]
+        assert (it, bl) == mixed[k][1:] and np.array_equal(x, mixed[k][0])
+    for op, _ in small + big:
+        P.ascg_op_destroy(op)
