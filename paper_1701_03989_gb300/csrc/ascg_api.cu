@@ -198,12 +198,12 @@ struct Workspace {
   double* oscaled[2] = {};      // O / gamma for up to two gamma != 1
   bool steps_ready = false;
   // pinned host mirrors
-  BlockState* h_bst = nullptr;
+  BlockState* h_bst = nullptr;  // the blocks' records, written by the device
+  unsigned* h_seq = nullptr;    // per record slot: the number of the block whose record is in place, + 1
   CGState* h_cgs = nullptr;
   double* h_scal = nullptr;
   cudaEvent_t ev[8] = {};
   cudaEvent_t ev_blk[kRing][5] = {};  // per record slot: the phase boundaries of a block (timing)
-  cudaEvent_t ev_rec[kRing] = {};     // per record slot: the block's record is on the host
   bool events = false;
   cudaStream_t side = nullptr;  // x += Y x' of the previous block
   cudaEvent_t ev_gram = nullptr, ev_x[2] = {};
@@ -215,14 +215,14 @@ struct Workspace {
     dev_free(dtils); dev_free(oscaled[0]); dev_free(oscaled[1]);
     steps_ready = false;
     if (h_bst) cudaFreeHost(h_bst);
+    if (h_seq) cudaFreeHost(h_seq);
     if (h_cgs) cudaFreeHost(h_cgs);
     if (h_scal) cudaFreeHost(h_scal);
-    h_bst = nullptr; h_cgs = nullptr; h_scal = nullptr;
+    h_bst = nullptr; h_seq = nullptr; h_cgs = nullptr; h_scal = nullptr;
     if (events) {
       for (auto& e : ev) cudaEventDestroy(e);
       for (auto& row : ev_blk)
         for (auto& e : row) cudaEventDestroy(e);
-      for (auto& e : ev_rec) cudaEventDestroy(e);
       cudaEventDestroy(ev_gram);
       for (auto& e : ev_x) cudaEventDestroy(e);
       if (side) cudaStreamDestroy(side);
@@ -326,6 +326,8 @@ int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 // cores by default (measured on GB300: the tensor-core kernel costs about
 // 40 us at n = 1024, w = 17, where the FP64 kernel takes a few).
 constexpr double kTcSolveProducts = 33554432.0;  // 2^25
+// Rows up to which an FP64 recovery is one launch (x, r and p).
+constexpr int64_t kOnePassRows = 131072;
 
 // Ensures the workspace can hold n rows, wcols basis columns and histories of
 // res_cap entries.
@@ -343,13 +345,13 @@ ascg_status ensure(ascg_op op, int wcols, int res_cap) {
     ASCG_TRY(dev_alloc(&w.shifts, 32));
     ASCG_TRY(dev_alloc(&w.bst, kRing));
     ASCG_TRY(dev_alloc(&w.cgs, 1));
-    ASCG_CUDA(cudaMallocHost((void**)&w.h_bst, 2 * kRing * sizeof(BlockState)));
+    ASCG_CUDA(cudaMallocHost((void**)&w.h_bst, kRing * sizeof(BlockState)));
+    ASCG_CUDA(cudaMallocHost((void**)&w.h_seq, kRing * sizeof(unsigned)));
     ASCG_CUDA(cudaMallocHost((void**)&w.h_cgs, sizeof(CGState)));
     ASCG_CUDA(cudaMallocHost((void**)&w.h_scal, 4 * sizeof(double)));
     for (auto& e : w.ev) ASCG_CUDA(cudaEventCreate(&e));
     for (auto& row : w.ev_blk)
       for (auto& e : row) ASCG_CUDA(cudaEventCreate(&e));
-    for (auto& e : w.ev_rec) ASCG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     ASCG_CUDA(cudaEventCreateWithFlags(&w.ev_gram, cudaEventDisableTiming));
     for (auto& e : w.ev_x) ASCG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     ASCG_CUDA(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
@@ -559,6 +561,20 @@ ascg_status prepare_steps(ascg_op op, const double* th, const double* sg, const 
   return ASCG_OK;
 }
 
+// Waits until the device has put block `seq` - 1's record in the host's slot.
+// The work that writes it is already on the stream, so a stream that is idle
+// (or has failed) without it is an error and not a longer wait.
+ascg_status wait_record(const unsigned* slot, unsigned seq, cudaStream_t s) {
+  for (;;) {
+    for (int i = 0; i < 4096; ++i)
+      if (__atomic_load_n(slot, __ATOMIC_ACQUIRE) == seq) return ASCG_OK;
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e == cudaErrorNotReady) continue;
+    if (e == cudaSuccess && __atomic_load_n(slot, __ATOMIC_ACQUIRE) == seq) return ASCG_OK;
+    return fail(ASCG_ERR_CUDA, std::string("block record: ") + cudaGetErrorString(e));
+  }
+}
+
 // Runs classical CG iterations (Alg. 1) on the device until the CG state says
 // done. x, r, p, q are device vectors. Returns the iterations done by this call.
 ascg_status run_classical(ascg_op op, double* x, double* r, double* p, double eps_star, double bnorm,
@@ -618,9 +634,10 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
   double* r = w.Y + w.ldY;
   ASCG_CUDA(launch_dot(b, b, n, &w.scal[0], w.partials, w.counter, s));
   ASCG_CUDA(launch_residual(A, b, x, r, p, s));
-  res->launches += 2;
-  res->grid_reductions += 1;
-  ASCG_CUDA(cudaMemcpyAsync(w.h_scal, w.scal, sizeof(double), cudaMemcpyDeviceToHost, s));
+  if (sstep) ASCG_CUDA(launch_dot(r, r, n, &w.scal[1], w.partials, w.counter, s));  // ||r_1||, on the same trip
+  res->launches += sstep ? 3 : 2;
+  res->grid_reductions += sstep ? 2 : 1;
+  ASCG_CUDA(cudaMemcpyAsync(w.h_scal, w.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
   ASCG_CUDA(cudaStreamSynchronize(s));
   const double bnorm = std::sqrt(w.h_scal[0]);
   res->bnorm = bnorm;
@@ -651,11 +668,6 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
     basis_params(o, th, sg, gm);
     bool done = false;
     // the residual history entry for i = 1 (m = 0)
-    ASCG_CUDA(launch_dot(r, r, n, &w.scal[1], w.partials, w.counter, s));
-    ASCG_CUDA(cudaMemcpyAsync(w.h_scal + 1, w.scal + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
-    ASCG_CUDA(cudaStreamSynchronize(s));
-    res->launches += 1;
-    res->grid_reductions += 1;
     double r0 = std::sqrt(std::max(w.h_scal[1], 0.0));
     {
       const double rel = r0 / bnorm;
@@ -725,26 +737,28 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
     // x update takes every other SM, one CTA each
     const int x_ctas = std::max(1, gram_grid() - (o.method == ASCG_ADAPTIVE ? o.s_max + 1 : 1));
     // Block j uses basis buffer j & 1, coordinates cbuf[j & 1] and record slot
-    // j % kRing (device w.bst[slot], pinned host w.h_bst[slot] going in and
-    // w.h_bst[kRing + slot] coming back). When block j+1's basis size does not
-    // depend on block j's outcome (Alg. 2, Alg. 3, and Alg. 4 with f >= s_max - 1,
-    // where sbar_k = s_max for every k >= 1), block j+1 is enqueued before the
-    // host reads block j's record: the GPU never waits for the host between
-    // blocks. A device kernel carries m, k and the iteration budget from
-    // block to block and clears block j+1's flag when block j ended the solve;
-    // every kernel of a block then returns at once.
+    // j % kRing (device w.bst[slot], pinned host w.h_bst[slot]). When block
+    // j+1's basis size does not depend on block j's outcome (Alg. 2, Alg. 3, and
+    // Alg. 4 with f >= s_max - 1, where sbar_k = s_max for every k >= 1), block
+    // j+1 is enqueued before the host reads block j's record: the GPU never
+    // waits for the host between blocks. block_handover_kernel carries m, k and
+    // the iteration budget from block to block and clears block j+1's flag when
+    // block j ended the solve; every kernel of a block then returns at once.
     const bool ahead = o.method == ASCG_FIXED_S || o.method == ASCG_VARIABLE_S ||
                        (o.method == ASCG_ADAPTIVE && o.f >= o.s_max - 1);
     int wb_of[kRing] = {};
-    bool rec_tc_of[kRing] = {};  // the block's recovery ran on the tensor cores (x included)
+    bool rec_tc_of[kRing] = {};  // the block's recovery ran on the tensor cores
+    bool rec_x_of[kRing] = {};   // the block's recovery updated x too
+    for (int q = 0; q < kRing; ++q) __atomic_store_n(w.h_seq + q, 0u, __ATOMIC_RELEASE);
     int sbar_of[kRing] = {};
+    int recorded = 0;  // blocks whose record is on its way to the host
     auto enqueue = [&](int j, int sbar) -> ascg_status {
       const int slot = j % kRing, cur = j & 1;
       const int wb = 2 * sbar + 1;
       double* const Yc = Ybuf[cur];
       BlockState* const dst = w.bst + slot;
       const int* const gate = &dst->active;
-      BlockState& hb = w.h_bst[slot];
+      BlockState hb;
       std::memset(&hb, 0, sizeof(hb));
       hb.sbar = sbar;
       hb.method = o.method;
@@ -759,11 +773,11 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
       hb.bnorm = bnorm;
       hb.sqrt_n = sqrt_n;
       hb.active = 1;
-      ASCG_CUDA(cudaMemcpyAsync(dst, &hb, sizeof(BlockState), cudaMemcpyHostToDevice, s));
-      if (j > 0) {
-        ASCG_CUDA(launch_block_advance(w.bst + (j - 1) % kRing, dst, o.max_iters, s));
-        res->launches += 1;
-      }
+      const int ps = (j + kRing - 1) % kRing;  // block j - 1's slot
+      ASCG_CUDA(launch_block_handover(j > 0 ? w.bst + ps : nullptr, j > 0 && recorded < j ? w.h_bst + ps : nullptr,
+                                      w.h_seq + ps, (unsigned)j, dst, hb, o.max_iters, s));
+      recorded = j;
+      res->launches += 1;
       wb_of[slot] = wb;
       sbar_of[slot] = sbar;
       cudaEvent_t* ev = w.ev_blk[slot];
@@ -800,8 +814,7 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
       else
         ASCG_CUDA(launch_gram_finalize(wb, w.partials, nparts, w.G, s, gate));
       res->launches += 2;
-      if (j > 0 && !rec_tc_of[(j - 1) % kRing]) {  // block j-1's x += Y x', beside this block's controller
-        const int ps = (j - 1) % kRing;
+      if (j > 0 && !rec_x_of[ps]) {  // block j-1's x += Y x', beside this block's controller
         ASCG_CUDA(cudaEventRecord(w.ev_gram, s));
         ASCG_CUDA(cudaStreamWaitEvent(w.side, w.ev_gram, 0));
         ASCG_CUDA(launch_recover_x(n, wb_of[ps], Ybuf[cur ^ 1], w.ldY, cbuf[cur ^ 1], x, x_ctas, w.side,
@@ -820,19 +833,24 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
         x_out[cur ^ 1] = false;
       }
       // A block whose Gram took the tensor cores recovers x, r and p on them in
-      // one pass (its column exponents are in w.expp); otherwise r and p here
-      // and x during the next block.
+      // one pass (its column exponents are in w.expp). In FP64, short vectors go
+      // in one pass too (below kOnePassRows the x update, 3 us of FP64 at 131072
+      // rows and 17 columns, costs less than a launch and the two waits between
+      // the streams); otherwise r and p here and x during the next block. The
+      // same sums either way.
       const bool tc_rec = tc_gram && !rec_fp64;
+      const bool one_pass = !tc_rec && n <= kOnePassRows;
       rec_tc_of[slot] = tc_rec;
+      rec_x_of[slot] = tc_rec || one_pass;
       if (tc_rec)
         ASCG_CUDA(launch_recover_tc(n, wb, Yc, w.ldY, w.expp, cbuf[cur], x, Ybuf[cur ^ 1] + w.ldY, Ybuf[cur ^ 1], s,
                                     &dst->status, gate));
+      else if (one_pass)
+        ASCG_CUDA(launch_recover_xrp(n, wb, Yc, w.ldY, cbuf[cur], x, Ybuf[cur ^ 1] + w.ldY, Ybuf[cur ^ 1], s, gate));
       else
         ASCG_CUDA(launch_recover_rp(n, wb, Yc, w.ldY, cbuf[cur], Ybuf[cur ^ 1] + w.ldY, Ybuf[cur ^ 1], s, gate));
       res->launches += 2;
       if (timing) ASCG_CUDA(cudaEventRecord(ev[4], s));
-      ASCG_CUDA(cudaMemcpyAsync(w.h_bst + kRing + slot, dst, sizeof(BlockState), cudaMemcpyDeviceToHost, s));
-      ASCG_CUDA(cudaEventRecord(w.ev_rec[slot], s));
       return ASCG_OK;
     };
     // block sizes known without the previous block's outcome
@@ -855,9 +873,16 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
       const int slot = k % kRing;
       const int sbar = sbar_of[slot];
       const int wb = wb_of[slot];
-      ASCG_CUDA(cudaEventSynchronize(w.ev_rec[slot]));
+      if (recorded == k) {  // no block enqueued behind this one carries its record
+        ASCG_CUDA(launch_block_handover(w.bst + slot, w.h_bst + slot, w.h_seq + slot, (unsigned)(k + 1), nullptr,
+                                        BlockState(), o.max_iters, s));
+        recorded = k + 1;
+        res->launches += 1;
+      }
+      ASCG_TRY(wait_record(w.h_seq + slot, (unsigned)(k + 1), s));
       if (timing) {
         cudaEvent_t* ev = w.ev_blk[slot];
+        ASCG_CUDA(cudaEventSynchronize(ev[4]));
         float a = 0.f, b2 = 0.f, c2 = 0.f, d2 = 0.f;
         ASCG_CUDA(cudaEventElapsedTime(&a, ev[0], ev[1]));
         ASCG_CUDA(cudaEventElapsedTime(&b2, ev[1], ev[2]));
@@ -876,13 +901,13 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
         const double nchains = 2.0 * sbar - 1.0;
         res->mpk_flops += nchains * 2.0 * (double)op->nnz;
         res->mpk_bytes += (double)sbar * (12.0 * op->nnz + 4.0 * (n + 1)) + nchains * 16.0 * n + 8.0 * n;
-        // the timed part: r = Y r', p = Y p', and x += Y x' on the tensor-core
-        // path (the FP64 path's x update runs later, on the side stream)
-        const double nvec = rec_tc_of[slot] ? 3.0 : 2.0;
+        // the timed part: r = Y r', p = Y p', and x += Y x' where it is one pass
+        // (otherwise the x update runs later, on the side stream)
+        const double nvec = rec_x_of[slot] ? 3.0 : 2.0;
         res->recover_flops += 2.0 * nvec * wb * (double)n;
-        res->recover_bytes += 8.0 * wb * (double)n + (rec_tc_of[slot] ? 32.0 : 16.0) * n;
+        res->recover_bytes += 8.0 * wb * (double)n + (rec_x_of[slot] ? 32.0 : 16.0) * n;
       }
-      const BlockState& out = w.h_bst[kRing + slot];
+      const BlockState& out = w.h_bst[slot];
       res->grid_reductions += 1;
       if (o.block_hist && nb_info < o.block_hist_cap) {
         ascg_block_info& bi = o.block_hist[nb_info];
@@ -930,7 +955,7 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
     // on the side stream
     for (int bq = 0; bq < 2; ++bq)
       if (x_out[bq]) ASCG_CUDA(cudaStreamWaitEvent(s, w.ev_x[bq], 0));
-    if (enq > 0 && !rec_tc_of[(enq - 1) % kRing]) {
+    if (enq > 0 && !rec_x_of[(enq - 1) % kRing]) {
       const int last = enq - 1, ls = last % kRing;
       ASCG_CUDA(launch_recover_x(n, wb_of[ls], Ybuf[last & 1], w.ldY, cbuf[last & 1], x, x_ctas, s,
                                  &w.bst[ls].active));

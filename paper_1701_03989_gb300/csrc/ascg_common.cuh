@@ -149,6 +149,24 @@ inline cudaError_t smem_limit_once(std::atomic<uint64_t>& done, K* kernel, int b
 // predecessor finished would let its own successor overtake that predecessor.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A pointer to what the previous kernel wrote, for use after pdl_wait(): the
+// compiler may move loads it takes for invariant (__ldg, const __restrict__)
+// above the wait, but not above the point where it learns their address.
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+  asm volatile("" : "+l"(p));
+  return p;
+}
+// A word that the previous kernel may have written, read after pdl_wait() (not
+// moved above it) and through L1: every CTA reads the same one, and a trip to L2
+// in each cost 7 us per 128^3 step.
+__device__ __forceinline__ int load_after_wait(const int* p) {
+  int v;
+  asm volatile("ld.global.ca.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// A block's flag (see launch_mpk_split_step).
+__device__ __forceinline__ bool gate_closed(const int* gate) { return gate && load_after_wait(gate) == 0; }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                  Args... args) {
@@ -408,6 +426,10 @@ cudaError_t launch_recover_rp(int64_t n, int w, const double* Y, int64_t ldY, co
                               double* p, cudaStream_t s, const int* gate = nullptr);
 cudaError_t launch_recover_x(int64_t n, int w, const double* Y, int64_t ldY, const double* coords, double* x,
                              int ctas, cudaStream_t s, const int* gate = nullptr);
+// All three in one launch (r and p as for launch_recover_rp), a dependent
+// launch: for vectors so short that the launches cost more than the work.
+cudaError_t launch_recover_xrp(int64_t n, int w, const double* Y, int64_t ldY, const double* coords, double* x,
+                               double* r, double* p, cudaStream_t s, const int* gate);
 
 // Block controller state shared by the controller kernels and the host driver.
 struct BlockState {
@@ -463,9 +485,10 @@ cudaError_t launch_block_ctrl_batch(const double* G, int64_t g_stride, const dou
                                     double* coords, int64_t c_stride, double* res_hist, int res_cap, double* ab_hist,
                                     int ab_cap, double* spec, unsigned* counters, cudaStream_t s);
 
-// Block j+1 of a single solve from block j's record (m, k, iteration budget,
-// and the flag that gates every kernel of block j+1).
-cudaError_t launch_block_advance(const BlockState* prev, BlockState* cur, int max_iters, cudaStream_t s);
+// The hand-over between two blocks of a single solve (see the kernel): block
+// j's record to the host and block j+1's record from init and block j's.
+cudaError_t launch_block_handover(const BlockState* prev, BlockState* host_rec, unsigned* host_seq, unsigned seq,
+                                  BlockState* cur, const BlockState& init, int max_iters, cudaStream_t s);
 
 // Newton shifts: Ritz values of the CG tridiagonal, Leja order. alphas, betas:
 // device; shifts: device double[k].

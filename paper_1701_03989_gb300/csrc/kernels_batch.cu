@@ -57,9 +57,9 @@ __global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __rest
   }
   pdl_wait();  // the step before (its column of Y) and the lanes' tables
   pdl_release();
-  const int steps = sys_steps[it.sys];
+  const int steps = load_after_wait(sys_steps + it.sys);
   if (!any || j + ch >= steps) return;  // uniform over the warp: no step j, or no R chain in the last one
-  const double* x = d.Y + (int64_t)(2 * j + ch) * d.ldY;
+  const double* x = after_wait(d.Y + (int64_t)(2 * j + ch) * d.ldY);
   double* y = d.Y + (int64_t)(2 * j + 2 + ch) * d.ldY;
   const double* v = d.o_val + b + lane;
   const int32_t* c = d.o_col + b + lane;

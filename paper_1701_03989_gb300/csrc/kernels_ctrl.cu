@@ -818,21 +818,58 @@ __global__ void __launch_bounds__(128, 1) block_ctrl_kernel(const double* __rest
   if (threadIdx.x == 0) *counters = 0u;
 }
 
-// Carries a single solve from block j to block j+1 on the device: m, k and the
-// iteration budget of block j+1 from block j's outcome, and block j+1's flag,
-// cleared when block j ended the solve (converged, no step, a wait that ran
-// out, or the iteration cap reached), so that a block enqueued ahead does
-// nothing.
-__global__ void block_advance_kernel(const BlockState* __restrict__ prev, BlockState* __restrict__ cur,
-                                     int max_iters) {
+// Hands a single solve over from block j to block j+1 on the device, in one
+// launch: block j's record (prev, if host_rec is given) to the host's pinned
+// memory, then its sequence number to host_seq, which the host polls; and
+// block j+1's record (cur, if given): its constants, and m, k and the iteration
+// budget from block j's outcome. Block j+1's flag is cleared when block j ended
+// the solve (converged, no step, a wait that ran out, or the iteration cap
+// reached), so that a block enqueued ahead does nothing. prev may be null (the
+// first block). One warp. (A copy each way, an event and a launch before, which
+// cut the chain of dependent launches at every block: 2D Poisson 32^2 2117 ->
+// 1820 us a solve, with the FP64 Gram and recovery dependent launches too;
+// 401^2 Newton 46.8 -> 45.0 ms, 128^3 55.7 -> 55.3.)
+__global__ void __launch_bounds__(32) block_handover_kernel(const BlockState* prev, BlockState* host_rec,
+                                                            unsigned* host_seq, unsigned seq, BlockState* cur,
+                                                            const BlockState init, int max_iters) {
   pdl_wait();
   pdl_release();
-  if (threadIdx.x != 0) return;
-  const int m = prev->m + prev->s_k;
-  cur->m = m;
-  cur->k = prev->k + 1;
-  cur->max_steps = max_iters - m;
-  cur->active = prev->active && prev->s_k > 0 && !prev->converged && prev->status == ASCG_OK && m < max_iters;
+  constexpr int kWords = sizeof(BlockState) / 4;
+  static_assert(sizeof(BlockState) % 4 == 0, "word copy");
+  if (host_rec) {
+    for (int i = threadIdx.x; i < kWords; i += 32)
+      reinterpret_cast<unsigned*>(host_rec)[i] = __ldcg(reinterpret_cast<const unsigned*>(prev) + i);
+    __threadfence_system();
+    __syncwarp();
+    if (threadIdx.x == 0) *reinterpret_cast<volatile unsigned*>(host_seq) = seq;
+  }
+  if (cur && threadIdx.x == 0) {
+    int m = init.m, k = init.k, max_steps = init.max_steps, active = init.active;
+    if (prev) {
+      const int sk = __ldcg(&prev->s_k);
+      m = __ldcg(&prev->m) + sk;
+      k = __ldcg(&prev->k) + 1;
+      max_steps = max_iters - m;
+      active = __ldcg(&prev->active) && sk > 0 && !__ldcg(&prev->converged) && __ldcg(&prev->status) == ASCG_OK &&
+               m < max_iters;
+    }
+    cur->sbar = init.sbar;
+    cur->method = init.method;
+    cur->check_in_loop = init.check_in_loop;
+    cur->max_steps = max_steps;
+    cur->m = m;
+    cur->k = k;
+    cur->eps_star = init.eps_star;
+    cur->c = init.c;
+    cur->c_step = init.c_step;
+    cur->c_smax = init.c_smax;
+    cur->bnorm = init.bnorm;
+    cur->sqrt_n = init.sqrt_n;
+    cur->active = active;
+    cur->stilde = cur->s_k = cur->stop = cur->converged = cur->status = 0;
+    cur->rnorm = cur->threshold = cur->gamma = cur->rel_res = 0.0;
+    for (int i = 0; i < kMaxS; ++i) cur->sqrt_kappa[i] = 0.0;
+  }
 }
 
 // Ritz values of the CG tridiagonal (k <= 32), one lane per eigenvalue index by
@@ -921,8 +958,9 @@ cudaError_t launch_block_ctrl_batch(const double* G, int64_t g_stride, const dou
                        counters);
 }
 
-cudaError_t launch_block_advance(const BlockState* prev, BlockState* cur, int max_iters, cudaStream_t s) {
-  return launch_pdl(block_advance_kernel, 1, 32, s, prev, cur, max_iters);
+cudaError_t launch_block_handover(const BlockState* prev, BlockState* host_rec, unsigned* host_seq, unsigned seq,
+                                  BlockState* cur, const BlockState& init, int max_iters, cudaStream_t s) {
+  return launch_pdl(block_handover_kernel, 1, 32, s, prev, host_rec, host_seq, seq, cur, init, max_iters);
 }
 
 cudaError_t launch_newton_shifts(const double* alphas, const double* betas, int k, double* shifts,

@@ -155,7 +155,9 @@ template <int W, bool MOM = false>
 __global__ void __launch_bounds__(kGramThreads, 1) gram_partial_kernel(int64_t n, const double* __restrict__ Y,
                                                                         int64_t ldY, double* __restrict__ partials,
                                                                         const int* __restrict__ gate) {
-  if (gate && !*gate) return;  // uniform: a block enqueued ahead that has nothing to do
+  pdl_wait();
+  pdl_release();
+  if (gate_closed(gate)) return;  // uniform: a block enqueued ahead that has nothing to do
   constexpr int NP = MOM ? kMomSlots : W * (W + 1) / 2;
   const int64_t nchunks = (n + kChunk - 1) / kChunk;
   gram_chunks<W, MOM>(n, Y, ldY, nchunks * blockIdx.x / gridDim.x, nchunks * (blockIdx.x + 1) / gridDim.x,
@@ -196,7 +198,7 @@ __device__ __forceinline__ void moments_to_gram(const double* mu, int w, double*
 __global__ void __launch_bounds__(128) gram_moment_finalize_kernel(int w, const double* __restrict__ partials,
                                                                    int nparts, double* __restrict__ G,
                                                                    const int* __restrict__ gate) {
-  if (gate && !*gate) return;
+  if (gate_closed(gate)) return;
   __shared__ double mu[kMomSlots];
   const int S = (w - 1) / 2;
   for (int sl = threadIdx.x; sl < kMomSlots; sl += blockDim.x) {
@@ -245,7 +247,7 @@ __global__ void __launch_bounds__(128) gram_finalize_kernel(int w, const double*
                                                             double* __restrict__ G, const int* __restrict__ gate) {
   pdl_wait();
   pdl_release();
-  if (gate && !*gate) return;
+  if (gate_closed(gate)) return;
   const int np = w * (w + 1) / 2;
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
   const int p = gt >> 2, t = gt & 3;
@@ -310,8 +312,7 @@ __global__ void __launch_bounds__(256) gram_items_finalize_kernel(int W, const d
 template <int W>
 cudaError_t gram_w(int64_t n, const double* Y, int64_t ldY, double* partials, int grid, cudaStream_t s,
                    const int* gate) {
-  gram_partial_kernel<W><<<grid, kGramThreads, 0, s>>>(n, Y, ldY, partials, gate);
-  return cudaGetLastError();
+  return launch_pdl(gram_partial_kernel<W>, grid, kGramThreads, s, n, Y, ldY, partials, gate);
 }
 
 }  // namespace

@@ -609,7 +609,7 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w_ou
   // everything above touches only this CTA: it overlaps the previous kernel
   pdl_wait();
   pdl_release();
-  if (tid < kTW) s_emax[tid] = tid < w ? col_emax[tid] : 0;
+  if (tid < kTW) s_emax[tid] = tid < w ? __ldcg(col_emax + tid) : 0;
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -810,7 +810,7 @@ done:
 __global__ void __maxnreg__(kTcRegs)
     gram_tc_kernel(const __grid_constant__ CUtensorMap ymap, int64_t n, int w, const int* __restrict__ col_emax,
                    double* __restrict__ partials, const TcGuard guard) {
-  // the block's flag was written several kernels ago (see block_advance_kernel)
+  // the block's flag was written several kernels ago (see block_handover_kernel)
   if (guard.gate && !__ldcg(guard.gate)) {  // uniform, before any barrier or tensor memory
     pdl_wait();
     return;
@@ -1051,7 +1051,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
   // everything above touches only this CTA: it overlaps the previous kernel
   pdl_wait();
   pdl_release();
-  if (tid < kTW) s_emax[tid] = tid < w ? col_emax[tid] : 0;
+  if (tid < kTW) s_emax[tid] = tid < w ? __ldcg(col_emax + tid) : 0;
   __syncthreads();
   // coefficients: u_vj = c_vj 2^(E_j - 55), E_j = emax_j - 1022; per vector the
   // largest biased exponent f_v; a NaN or infinite column or coefficient
@@ -1061,7 +1061,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
   double u = 0.0;
   if (cthr) {
     // a zero column (emax 0) takes no part: its digits are all zero
-    u = s_emax[cj] == 0 ? 0.0 : ldexp(coords[cv * w + cj], s_emax[cj] - 1077);
+    u = s_emax[cj] == 0 ? 0.0 : ldexp(__ldcg(coords + cv * w + cj), s_emax[cj] - 1077);
     const int eu = (__double2hiint(u) >> 20) & 0x7ff;
     atomicMax(s_fv + cv, eu);
     if (eu == 0x7ff || s_emax[cj] == 0x7ff) atomicMax(s_fv + 3, 1);

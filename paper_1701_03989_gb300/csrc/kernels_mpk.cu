@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kSpmvRows, 6)
                           const int* __restrict__ gate) {
   pdl_wait();     // the previous step's columns (and the gate) are written by the kernel before
   pdl_release();  // the next step may be scheduled once every CTA of this one has started
-  if (gate && !*gate) return;  // uniform: a block enqueued ahead that has nothing to do
+  if (gate_closed(gate)) return;  // uniform: a block enqueued ahead that has nothing to do
   const int64_t row = (int64_t)blockIdx.x * kSpmvRows + threadIdx.x;
   unsigned e_op = 0, e_or = 0;
   if (row < O.n) {
@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(128, 8)
   }
   if (j > 0) pdl_wait();
   pdl_release();
-  if (!any || (gate && !*gate)) return;  // uniform over the warp
-  const double* x = Y + (int64_t)(2 * j + ch) * ldY;
+  if (!any || gate_closed(gate)) return;  // uniform over the warp
+  const double* x = after_wait(Y + (int64_t)(2 * j + ch) * ldY);
   const double xi = on ? x[row] : 0.0;
   double t;
   if (SIG == 0) {
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(1024) emax_reduce_kernel(const int* __restrict
                                                            int* __restrict__ col_emax, const int* __restrict__ gate) {
   pdl_wait();
   pdl_release();
-  if (gate && !*gate) return;
+  if (gate_closed(gate)) return;
   const int c = blockIdx.x;
   const int4* src = reinterpret_cast<const int4*>(emax_part + (int64_t)c * emax_ld);
   const int64_t n4 = emax_ld / 4;
@@ -250,12 +250,15 @@ constexpr int kRecGroup = 8;
 template <int W>
 __global__ void __launch_bounds__(256, 6) recover_kernel(int64_t n, const double* Y, int64_t ldY,
                                                          const double* __restrict__ coords, double* x, double* r,
-                                                         double* p) {
+                                                         double* p, const int* __restrict__ gate) {
+  pdl_wait();
+  pdl_release();
+  if (gate_closed(gate)) return;
   __shared__ double cx[W], cr[W], cp[W];
   if (threadIdx.x < W) {
-    cx[threadIdx.x] = coords[threadIdx.x];
-    cr[threadIdx.x] = coords[W + threadIdx.x];
-    cp[threadIdx.x] = coords[2 * W + threadIdx.x];
+    cx[threadIdx.x] = __ldcg(coords + threadIdx.x);
+    cr[threadIdx.x] = __ldcg(coords + W + threadIdx.x);
+    cp[threadIdx.x] = __ldcg(coords + 2 * W + threadIdx.x);
   }
   __syncthreads();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -286,9 +289,8 @@ inline int rec_grid(int64_t n) { return grid_for(n, 256, 152 * 64); }
 
 template <int W>
 cudaError_t recover_w(int64_t n, const double* Y, int64_t ldY, const double* coords, double* x, double* r,
-                      double* p, cudaStream_t s) {
-  recover_kernel<W><<<rec_grid(n), 256, 0, s>>>(n, Y, ldY, coords, x, r, p);
-  return cudaGetLastError();
+                      double* p, cudaStream_t s, const int* gate) {
+  return launch_pdl(recover_kernel<W>, rec_grid(n), 256, s, n, Y, ldY, coords, x, r, p, gate);
 }
 
 // The recovery split in two, with the same sums as recover_kernel (so the
@@ -300,7 +302,7 @@ __global__ void __launch_bounds__(256, 6) recover_rp_kernel(int64_t n, const dou
                                                             const double* __restrict__ coords,
                                                             double* __restrict__ r, double* __restrict__ p,
                                                             const int* __restrict__ gate) {
-  if (gate && !*gate) return;
+  if (gate_closed(gate)) return;
   __shared__ double cr[W], cp[W];
   if (threadIdx.x < W) {
     cr[threadIdx.x] = coords[W + threadIdx.x];
@@ -337,7 +339,7 @@ template <int W>
 __global__ void __launch_bounds__(kXThreads, 1) recover_x_kernel(int64_t n, const double* __restrict__ Y,
                                                                  int64_t ldY, const double* __restrict__ coords,
                                                                  double* __restrict__ x, const int* __restrict__ gate) {
-  if (gate && !*gate) return;
+  if (gate_closed(gate)) return;
   __shared__ double cx[W];
   if (threadIdx.x < W) cx[threadIdx.x] = coords[threadIdx.x];
   __syncthreads();
@@ -440,10 +442,15 @@ cudaError_t launch_recover_x(int64_t n, int w, const double* Y, int64_t ldY, con
 
 cudaError_t launch_recover(int64_t n, int w, const double* Y, int64_t ldY, const double* coords, double* x,
                            double* r, double* p, cudaStream_t s) {
+  return launch_recover_xrp(n, w, Y, ldY, coords, x, r, p, s, nullptr);
+}
+
+cudaError_t launch_recover_xrp(int64_t n, int w, const double* Y, int64_t ldY, const double* coords, double* x,
+                               double* r, double* p, cudaStream_t s, const int* gate) {
   switch (w) {
 #define ASCG_RW(W) \
   case W:          \
-    return recover_w<W>(n, Y, ldY, coords, x, r, p, s);
+    return recover_w<W>(n, Y, ldY, coords, x, r, p, s, gate);
     ASCG_RW(1) ASCG_RW(3) ASCG_RW(5) ASCG_RW(7) ASCG_RW(9) ASCG_RW(11) ASCG_RW(13) ASCG_RW(15) ASCG_RW(17)
     ASCG_RW(19) ASCG_RW(21) ASCG_RW(23) ASCG_RW(25) ASCG_RW(27) ASCG_RW(29) ASCG_RW(31) ASCG_RW(33)
 #undef ASCG_RW

@@ -198,3 +198,32 @@ def test_gram_pieces_do_not_change_a_bit():
         assert (it, bl) == mixed[k][1:] and np.array_equal(x, mixed[k][0])
     for op, _ in small + big:
         P.ascg_op_destroy(op)
+
+
+@pytest.mark.parametrize("method", ["fixed", "adaptive"])
+@pytest.mark.parametrize("n", [1, 33, 131072, 131073])
+def test_fp64_recovery_one_pass_and_split(n, method):
+    """The FP64 recovery in one launch (up to 131072 rows) and in two, over many short blocks: the solution's true residual.
+
+    Tolerance: the matrix is tridiagonal with diagonal 4 and off-diagonals -1 (condition below 3), so the updated residual,
+    below 1e-12 at convergence, and the true one differ by a few hundred rounding errors of the iterates: 4x the target.
+    """
+    import paper_1701_03989_gb300 as P
+
+    keep = np.ones((n, 3), bool)
+    keep[0, 0] = keep[-1, 2] = False
+    cols = np.arange(n)[:, None] + np.arange(-1, 2)[None, :]
+    vals = np.broadcast_to(np.array([-1.0, 4.0, -1.0]), (n, 3))
+    rowptr = np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int64)
+    op = P.ascg_op_create_csr(n, int(rowptr[-1]), rowptr, cols[keep].astype(np.int32), vals[keep], 0)
+    b = np.random.default_rng(n).uniform(-1, 1, n)
+    x = torch.zeros(n, dtype=torch.float64, device="cuda")
+    res = P.ascg_solve(op, torch.from_numpy(b).cuda(), x, P.make_options(method=method, s_max=3, eps_target=1e-12,
+                                                                          gram_fp64=True, max_iters=500))
+    P.ascg_op_destroy(op)
+    x = x.cpu().numpy()
+    r = b - 4.0 * x
+    r[1:] += x[:-1]
+    r[:-1] += x[1:]
+    assert res.status == P.ASCG_OK and res.blocks >= min(n, 3) / 3
+    assert np.linalg.norm(r) <= 4e-12 * np.linalg.norm(b)
