@@ -778,7 +778,9 @@ __device__ void select_steps(BlockState* st, const double* __restrict__ rec, dou
 // last CTA to finish (a ticket counter per system, reset afterwards; nothing
 // waits) selects s~_k and s_k and writes the outputs. The condition
 // estimates and the steps thus overlap instead of following each other.
-__global__ void __launch_bounds__(128, 1) block_ctrl_kernel(const double* __restrict__ G,
+// 3 CTAs per SM (166 registers): 192 systems in a batch 186.4 -> 185.5 ms against
+// 184 registers; 128 registers spill and take a single block from 126 to 137 us.
+__global__ void __launch_bounds__(128, 3) block_ctrl_kernel(const double* __restrict__ G,
                                                          const double* __restrict__ th_g,
                                                          const double* __restrict__ sg_g,
                                                          const double* __restrict__ gm_g, BlockState* st,
@@ -872,14 +874,19 @@ __global__ void __launch_bounds__(32) block_handover_kernel(const BlockState* pr
   }
 }
 
-// Ritz values of the CG tridiagonal (k <= 32), one lane per eigenvalue index by
-// bisection, then Leja order computed by the whole warp.
-__global__ void __launch_bounds__(32) newton_shifts_kernel(const double* __restrict__ al,
-                                                           const double* __restrict__ be, int k,
-                                                           double* __restrict__ shifts) {
-  __shared__ double d[32], e[32], e2[32], ritz[32];
-  __shared__ double gl, gh, pm;
-  const int lane = threadIdx.x;
+// Ritz values of the CG tridiagonal (k <= 32) by bisection, one CTA (one warp)
+// per eigenvalue: value i + 1 is the smallest x with count(x) >= i + 1. The warp
+// takes five bisection levels per round: lane L evaluates the midpoint of node
+// L of the tree of the next five intervals (root 1, lower half 2L, upper half
+// 2L + 1), and the warp then walks down the counts, testing the interval at each
+// level. The same midpoints and decisions, so the same bits, as one level at a
+// time; a round costs one Sturm sequence of FP64 latency (k divisions of 535
+// cycles). One warp with a lane per value, level by level, took 737 us at
+// k = 24; a 401^2 Newton solve, one such launch in it: 45.0 -> 43.5 ms.
+__global__ void __launch_bounds__(32) newton_ritz_kernel(const double* __restrict__ al, const double* __restrict__ be,
+                                                         int k, double* __restrict__ ritz) {
+  __shared__ double d[32], e[32], e2[32];
+  const int lane = threadIdx.x, want = blockIdx.x + 1;
   if (lane < k) {
     d[lane] = 1.0 / al[lane] + (lane > 0 ? be[lane - 1] / al[lane - 1] : 0.0);
     if (lane + 1 < k) {
@@ -888,33 +895,53 @@ __global__ void __launch_bounds__(32) newton_shifts_kernel(const double* __restr
     }
   }
   __syncwarp();
-  if (lane == 0) {
-    double lo, hi, piv;
-    gershgorin(d, e, k, &lo, &hi, &piv);
-    gl = lo;
-    gh = hi;
-    pm = piv;
-  }
-  __syncwarp();
-  if (lane < k) {
-    // the (lane+1)-th smallest eigenvalue: smallest x with count(x) >= lane + 1
-    double lo = gl, hi = gh;
-    for (int it = 0; it < 200; ++it) {
-      const double scale = fmax(fabs(lo), fabs(hi));
-      if (hi - lo <= 2.0 * kEps * scale || !(hi > lo)) break;
-      const double mid = 0.5 * (lo + hi);
-      if (mid <= lo || mid >= hi) break;
-      if (sturm_count(d, e2, k, mid, pm) >= lane + 1)
-        hi = mid;
+  double lo, hi, piv;
+  gershgorin(d, e, k, &lo, &hi, &piv);  // the same in every lane
+  bool open = true;
+  for (int it = 0; it < 200 && open; it += 5) {
+    // this lane's node: its interval, from the root down
+    double a = lo, b = hi;
+    const int depth = lane > 0 ? 31 - __clz(lane) : 0;
+    for (int q = depth - 1; q >= 0; --q) {
+      const double mid = 0.5 * (a + b);
+      if ((lane >> q) & 1)
+        a = mid;
       else
-        lo = mid;
+        b = mid;
     }
-    ritz[lane] = 0.5 * (lo + hi);
+    const bool low = lane > 0 && sturm_count(d, e2, k, 0.5 * (a + b), piv) >= want;
+    const unsigned down = __ballot_sync(kFull, low);  // bit L: the value lies in the lower half of node L
+    int node = 1;
+    for (int q = 0; q < 5; ++q) {
+      const double scale = fmax(fabs(lo), fabs(hi));
+      if (hi - lo <= 2.0 * kEps * scale || !(hi > lo)) {
+        open = false;
+        break;
+      }
+      const double mid = 0.5 * (lo + hi);
+      if (mid <= lo || mid >= hi) {
+        open = false;
+        break;
+      }
+      if ((down >> node) & 1u) {
+        hi = mid;
+        node = 2 * node;
+      } else {
+        lo = mid;
+        node = 2 * node + 1;
+      }
+    }
   }
-  __syncwarp();
+  if (lane == 0) ritz[blockIdx.x] = 0.5 * (lo + hi);
+}
+
+// Leja order of the k <= 32 values in shifts (in place), by one warp.
+__global__ void __launch_bounds__(32) newton_leja_kernel(int k, double* __restrict__ shifts) {
+  const int lane = threadIdx.x;
   // Leja order: first the largest |value|; then the largest product of distances
   // to the values chosen so far. Ties: larger value, then lower index.
-  const double val = lane < k ? ritz[lane] : 0.0;
+  const double val = lane < k ? shifts[lane] : 0.0;
+  __syncwarp();  // all read before the first is written
   double score = fabs(val);
   bool avail = lane < k;
   for (int step = 0; step < k; ++step) {
@@ -965,7 +992,8 @@ cudaError_t launch_block_handover(const BlockState* prev, BlockState* host_rec, 
 
 cudaError_t launch_newton_shifts(const double* alphas, const double* betas, int k, double* shifts,
                                  cudaStream_t s) {
-  newton_shifts_kernel<<<1, 32, 0, s>>>(alphas, betas, k, shifts);
+  newton_ritz_kernel<<<k, 32, 0, s>>>(alphas, betas, k, shifts);
+  newton_leja_kernel<<<1, 32, 0, s>>>(k, shifts);
   return cudaGetLastError();
 }
 

@@ -227,3 +227,23 @@ def test_fp64_recovery_one_pass_and_split(n, method):
     r[:-1] += x[1:]
     assert res.status == P.ASCG_OK and res.blocks >= min(n, 3) / 3
     assert np.linalg.norm(r) <= 4e-12 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 5, 6, 17, 31, 32])
+def test_newton_shifts_every_value(k):
+    """All k Ritz values (five bisection levels a round, one CTA a value) against numpy's eigenvalues of the tridiagonal.
+
+    Bisection ends at neighbouring doubles of the Sturm count's own tridiagonal, which is within a few eps ||T|| of the
+    exact one, as is numpy's: 32 k eps ||T|| covers both.
+    """
+    import paper_1701_03989_gb300 as P
+
+    rng = np.random.default_rng(k)
+    al, be = rng.uniform(0.3, 3.0, k), rng.uniform(0.01, 1.5, max(k - 1, 1))
+    d = 1 / al
+    d[1:] += be[: k - 1] / al[: k - 1]
+    e = np.sqrt(be[: k - 1]) / al[: k - 1]
+    ev = np.linalg.eigvalsh(np.diag(d) + np.diag(e, 1) + np.diag(e, -1))
+    got = P.ascg_newton_shifts(al, be, k, k)
+    assert abs(got[0]) == max(abs(got))
+    assert np.max(np.abs(np.sort(got) - ev)) <= 32 * k * 2.0 ** -53 * np.max(np.abs(ev))
