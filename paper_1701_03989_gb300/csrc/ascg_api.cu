@@ -696,7 +696,7 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
       if (!done) {
         if (m < o.s_max) return fail(ASCG_ERR_BREAKDOWN, "Newton warm-up ended early");
         ASCG_CUDA(launch_newton_shifts(w.ab_hist, w.ab_hist + w.ab_cap, m, w.shifts, s));
-        res->launches += 1;
+        res->launches += 2;
         double sh[32];
         ASCG_CUDA(cudaMemcpyAsync(sh, w.shifts, m * sizeof(double), cudaMemcpyDeviceToHost, s));
         ASCG_CUDA(cudaStreamSynchronize(s));
@@ -844,7 +844,7 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
       rec_x_of[slot] = tc_rec || one_pass;
       if (tc_rec)
         ASCG_CUDA(launch_recover_tc(n, wb, Yc, w.ldY, w.expp, cbuf[cur], x, Ybuf[cur ^ 1] + w.ldY, Ybuf[cur ^ 1], s,
-                                    &dst->status, gate));
+                                    &dst->status, &dst->status, gate));
       else if (one_pass)
         ASCG_CUDA(launch_recover_xrp(n, wb, Yc, w.ldY, cbuf[cur], x, Ybuf[cur ^ 1] + w.ldY, Ybuf[cur ^ 1], s, gate));
       else
@@ -1213,15 +1213,16 @@ ascg_status ascg_gram(int64_t n, int w, const double* Y, int64_t ldY, double* G,
   cudaStream_t s = (cudaStream_t)cuda_stream;
   Scratch sc;
   const size_t np = (size_t)gram_grid() * kMaxPairs;
-  ASCG_TRY(sc.open(Scratch::round(np * sizeof(double)) + Scratch::round((kMaxW + 1) * sizeof(int))));
+  ASCG_TRY(sc.open(Scratch::round(np * sizeof(double)) + Scratch::round(kMaxW * sizeof(int))));
   double* partials = sc.take<double>(np);
-  int* expp = sc.take<int>(kMaxW + 1);  // column exponents, then one error word of the tensor-core kernel
+  int* expp = sc.take<int>(kMaxW);  // column exponents
+  // the tensor-core kernel's error word, in the block's pinned page: written
+  // only when a wait runs out, so nothing is cleared or copied on the device
   int* herr = sc.host<int>();
+  *herr = 0;
   int parts = 0;
-  cudaError_t e = cudaMemsetAsync(expp, 0, (kMaxW + 1) * sizeof(int), s);
-  if (e == cudaSuccess) e = launch_gram_any(n, w, Y, ldY, false, expp, false, partials, &parts, s, expp + kMaxW);
+  cudaError_t e = launch_gram_any(n, w, Y, ldY, false, expp, false, partials, &parts, s, herr);
   if (e == cudaSuccess) e = launch_gram_finalize(w, partials, parts, G, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(herr, expp + kMaxW, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("gram: ") + cudaGetErrorString(e));
   sc.synced();
@@ -1325,13 +1326,12 @@ ascg_status ascg_recover_tc(int64_t n, int w, const double* Y, int64_t ldY, cons
   if (!gram_tc_aligned(Y, ldY)) return fail(ASCG_ERR_INVALID, "Y must be 16-byte aligned with an even ldY");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   Scratch sc;
-  ASCG_TRY(sc.open(Scratch::round((kMaxW + 1) * sizeof(int))));
-  int* expp = sc.take<int>(kMaxW + 1);  // column exponents, then the kernel's error word
-  int* herr = sc.host<int>();
-  cudaError_t e = cudaMemsetAsync(expp + kMaxW, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = launch_col_exponents(n, w, Y, ldY, expp, s);
-  if (e == cudaSuccess) e = launch_recover_tc(n, w, Y, ldY, expp, coords, x, r, p, s, expp + kMaxW);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(herr, expp + kMaxW, sizeof(int), cudaMemcpyDeviceToHost, s);
+  ASCG_TRY(sc.open(Scratch::round(kMaxW * sizeof(int))));
+  int* expp = sc.take<int>(kMaxW);  // column exponents
+  int* herr = sc.host<int>();       // the kernel's error word (pinned: see ascg_gram)
+  *herr = 0;
+  cudaError_t e = launch_col_exponents(n, w, Y, ldY, expp, s);
+  if (e == cudaSuccess) e = launch_recover_tc(n, w, Y, ldY, expp, coords, x, r, p, s, herr, nullptr, nullptr);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail(ASCG_ERR_CUDA, std::string("recover_tc: ") + cudaGetErrorString(e));
   sc.synced();

@@ -321,7 +321,7 @@ bool gram_tc_aligned(const double* Y, int64_t ldY);
 struct TcGuard {
   long long wait_limit;
   int stall_stage;
-  int* err;
+  int* err;         // device memory, or pinned host memory
   const int* gate;  // see launch_mpk_split_step
 };
 // col_emax: device int[kMaxW], the largest biased exponent of each column;
@@ -365,10 +365,11 @@ cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const
 // x', r', p'). Each result is the FP64 rounding of a fixed-point sum, within a
 // normwise bound (kernels_gram_tc.cu). kGramTcMinW <= w <= kMaxW, Y aligned
 // as for the tensor-core Gram; r and p may be columns 1 and 0 of Y. err and
-// gate: as in TcGuard.
+// gate: as in TcGuard. failed (device int, or nullptr): the Gram's error word;
+// when it is set, x, r and p are left alone.
 cudaError_t launch_recover_tc(int64_t n, int w, const double* Y, int64_t ldY, const int* col_emax,
-                              const double* coords, double* x, double* r, double* p, cudaStream_t s,
-                              int* err = nullptr, const int* gate = nullptr);
+                              const double* coords, double* x, double* r, double* p, cudaStream_t s, int* err,
+                              const int* failed, const int* gate);
 // The largest biased exponent of each column into col_emax (device int[kMaxW]).
 cudaError_t launch_col_exponents(int64_t n, int w, const double* Y, int64_t ldY, int* col_emax, cudaStream_t s);
 cudaError_t launch_gram_any(int64_t n, int w, const double* Y, int64_t ldY, bool force_fp64, int* col_emax,

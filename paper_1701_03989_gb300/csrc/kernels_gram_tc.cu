@@ -998,11 +998,11 @@ __device__ __forceinline__ double rec_value(const uint32_t (&e)[8], const uint32
 __global__ void __launch_bounds__(kRThreads, 1)
     recover_tc_kernel(const __grid_constant__ CUtensorMap ymap, int64_t n, int w, const int* __restrict__ col_emax,
                       const double* __restrict__ coords, double* __restrict__ x, double* __restrict__ r,
-                      double* __restrict__ p, const TcGuard guard) {
+                      double* __restrict__ p, const TcGuard guard, const int* failed) {
   // uniform, before any barrier or tensor memory: a block enqueued ahead with
   // nothing to do, or one whose Gram already failed (its error word is set),
   // leaves x, r and p alone. Both words were written several kernels ago.
-  if ((guard.gate && !__ldcg(guard.gate)) || (guard.err && __ldcg(guard.err) != 0)) {
+  if ((guard.gate && !__ldcg(guard.gate)) || (failed && __ldcg(failed) != 0)) {
     pdl_wait();
     return;
   }
@@ -1324,7 +1324,7 @@ cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const
 
 cudaError_t launch_recover_tc(int64_t n, int w, const double* Y, int64_t ldY, const int* col_emax,
                               const double* coords, double* x, double* r, double* p, cudaStream_t s, int* err,
-                              const int* gate) {
+                              const int* failed, const int* gate) {
   if (!gram_tc_applies(w) || !gram_tc_aligned(Y, ldY) || n < 1 || n > 0x7fffffffll) return cudaErrorInvalidValue;
   cudaError_t e = smem_limit_once(g_rec_smem_set, recover_tc_kernel, (int)kRSmem);
   if (e != cudaSuccess) return e;
@@ -1335,7 +1335,7 @@ cudaError_t launch_recover_tc(int64_t n, int w, const double* Y, int64_t ldY, co
   const int g = gram_grid();
   const TcGuard guard{kWaitLimit, -1, err, gate};
   return launch_pdl_ex(recover_tc_kernel, dim3((unsigned)(tiles < g ? tiles : g)), dim3(kRThreads), kRSmem, s, map, n,
-                       w, col_emax, coords, x, r, p, guard);
+                       w, col_emax, coords, x, r, p, guard, failed);
 }
 
 cudaError_t launch_col_exponents(int64_t n, int w, const double* Y, int64_t ldY, int* col_emax, cudaStream_t s) {
