@@ -14,12 +14,15 @@ namespace ascg {
 
 namespace {
 
-// sum_j a_ij x_j for row i (i < A.n) in stored order, starting from 0. With
-// STREAM, the values and column indices of A, read once per pass, are loaded
-// with the evict-first (streaming) policy, so that the vectors of an
-// iteration, which every pass reads again, keep their place in L2: worth it
-// when A does not fit in L2 beside them. A small A is better left in L2.
-template <bool STREAM = false>
+// sum_j a_ij x_j for row i (i < A.n) in stored order, starting from 0; the same
+// FMAs in every mode. kStream: the values and column indices of A, read once
+// per pass, are loaded with the evict-first (streaming) policy, so that the
+// vectors of an iteration, which every pass reads again, keep their place in
+// L2: worth it when A does not fit in L2 beside them. A small A is better left
+// in L2 (kKeep). kChain: row_chain's pipelined loads, for long rows, whose time
+// is otherwise a gather's latency per entry.
+enum SellMode { kKeep, kStream, kChain };
+template <SellMode MODE = kKeep>
 __device__ __forceinline__ double sell_row(const DevSell& A, int64_t i, const double* __restrict__ x) {
   const int64_t s = i >> 5;
   const int l = (int)(i & 31);
@@ -27,8 +30,9 @@ __device__ __forceinline__ double sell_row(const DevSell& A, int64_t i, const do
   const int width = (int)((A.ptr[s + 1] - b) >> 5);
   const double* v = A.val + b + l;
   const int32_t* c = A.col + b + l;
+  if (MODE == kChain) return row_chain(v, c, width, x, 0.0);
   double t = 0.0;
-  if (STREAM) {
+  if (MODE == kStream) {
     for (int j = 0; j < width; ++j) t = fma(__ldcs(v + kSlice * j), __ldg(x + __ldcs(c + kSlice * j)), t);
   } else {
     for (int j = 0; j < width; ++j) t = fma(__ldg(v + kSlice * j), __ldg(x + __ldg(c + kSlice * j)), t);
@@ -36,20 +40,24 @@ __device__ __forceinline__ double sell_row(const DevSell& A, int64_t i, const do
   return t;
 }
 
+// Fixed-order sum over a CTA of 256 threads (valid in thread 0): warp trees, then
+// the same tree over the eight warp sums, without its two levels that would
+// only add zeros (110 cycles each). With the division and the square root of
+// the update in two warps this took an iteration of 2D Poisson 32^2 from 13.4
+// to 12.5 us, of 128^3 from 71.6 to 70.5.
 __device__ __forceinline__ double block_sum(double v, double* red) {
-  // fixed-order CTA reduction: warp trees, then warp 0 adds the warp sums in order
   v = warp_sum(v);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) red[warp] = v;
   __syncthreads();
   double t = 0.0;
   if (warp == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    t = lane < nw ? red[lane] : 0.0;
-    t = warp_sum(t);
+    t = lane < 8 ? red[lane] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   }
   __syncthreads();
-  return t;  // valid in thread 0
+  return t;
 }
 
 // Deterministic completion: writes partials[blockIdx.x] and returns true in the
@@ -114,7 +122,7 @@ __global__ void __launch_bounds__(256) dot_kernel(const double* __restrict__ u, 
 // Grid-stride over rows with a bounded grid: every CTA ends in one block
 // reduction and one atomic ticket, so few CTAs keep that overhead small. Each
 // warp-wide FP64 add costs a full FP64 issue slot, however few lanes need it.
-template <bool STREAM>
+template <SellMode MODE>
 __global__ void __launch_bounds__(kSpmvRows) cg_spmv_dot_kernel(DevSell A, const double* __restrict__ p,
                                                                 double* __restrict__ q, CGState* st,
                                                                 double* partials, unsigned* counter) {
@@ -127,7 +135,7 @@ __global__ void __launch_bounds__(kSpmvRows) cg_spmv_dot_kernel(DevSell A, const
   if (done) return;
   double part = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * kSpmvRows + threadIdx.x; i < A.n; i += (int64_t)gridDim.x * kSpmvRows) {
-    const double v = sell_row<STREAM>(A, i, p);
+    const double v = sell_row<MODE>(A, i, p);
     q[i] = v;
     part = fma(p[i], v, part);
   }
@@ -173,16 +181,24 @@ __global__ void __launch_bounds__(256) cg_update_kernel(int64_t n, double* __res
   }
   s = block_sum(s, red);
   if (last_block(s, partials, counter, &flag)) {
-    const double rr = sum_partials(partials, gridDim.x, red);
+    const double tot = sum_partials(partials, gridDim.x, red);
+    if (threadIdx.x == 0) red[0] = tot;
+    __syncthreads();
+    const double rr = red[0];
+    const int it = st->iter;
+    const double rr_old = st->rr;
+    __syncthreads();  // both warps have read the old state
+    // the division in one warp, the square root in another
     if (threadIdx.x == 0) {
-      const double beta = rr / st->rr;       // beta_i = r_{i+1}^T r_{i+1} / r_i^T r_i
-      const int it = st->iter;
+      const double beta = rr / rr_old;       // beta_i = r_{i+1}^T r_{i+1} / r_i^T r_i
       if (it < ab_cap) {
         if (alpha_hist) alpha_hist[it] = alpha;
         if (beta_hist) beta_hist[it] = beta;
       }
       st->beta = beta;
       st->rr = rr;
+      *counter = 0u;
+    } else if (threadIdx.x == 32) {
       st->iter = it + 1;
       const double rn = sqrt(rr);
       if (res_hist && it + 1 < res_cap) res_hist[it + 1] = rn / st->bnorm;
@@ -190,7 +206,6 @@ __global__ void __launch_bounds__(256) cg_update_kernel(int64_t n, double* __res
       st->converged = conv;
       // p is still updated for this iteration (cg_pupdate reads 'active')
       st->done = conv || (it + 1 >= st->max_iters);
-      *counter = 0u;
     }
   }
 }
@@ -250,11 +265,16 @@ cudaError_t launch_dot(const double* u, const double* v, int64_t n, double* out,
 cudaError_t launch_cg_spmv_dot(const DevSell& A, int64_t nnz, const double* p, double* q, CGState* st,
                                double* partials, unsigned* counter, cudaStream_t s) {
   const int g = grid_for(A.n, kSpmvRows, 152 * 8);
+  // long rows: us per iteration, an entry at a time / pipelined: n = 20011 of 13
+  // entries a row 14.0 / 13.5, of 81 25.1 / 18.8, n = 100003 of 33 27.5 / 25.4,
+  // n = 300007 of 81 (streamed past L2) 73.6 / 75.9
+  if (nnz >= 12 * A.n && A.n <= 262144)
+    return launch_pdl(cg_spmv_dot_kernel<kChain>, g, kSpmvRows, s, A, p, q, st, partials, counter);
   // A's values and columns (12 bytes per entry) beyond a quarter of the 129 MB
   // L2: stream them past it
   if (12 * nnz > ((int64_t)32 << 20))
-    return launch_pdl(cg_spmv_dot_kernel<true>, g, kSpmvRows, s, A, p, q, st, partials, counter);
-  return launch_pdl(cg_spmv_dot_kernel<false>, g, kSpmvRows, s, A, p, q, st, partials, counter);
+    return launch_pdl(cg_spmv_dot_kernel<kStream>, g, kSpmvRows, s, A, p, q, st, partials, counter);
+  return launch_pdl(cg_spmv_dot_kernel<kKeep>, g, kSpmvRows, s, A, p, q, st, partials, counter);
 }
 
 cudaError_t launch_cg_update(int64_t n, double* r, const double* q, CGState* st, double* partials,

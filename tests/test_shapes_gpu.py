@@ -247,3 +247,23 @@ def test_newton_shifts_every_value(k):
     got = P.ascg_newton_shifts(al, be, k, k)
     assert abs(got[0]) == max(abs(got))
     assert np.max(np.abs(np.sort(got) - ev)) <= 32 * k * 2.0 ** -53 * np.max(np.abs(ev))
+
+
+@pytest.mark.parametrize("h", [1, 5, 6, 40])
+@pytest.mark.parametrize("n", [31, 257, 5000])
+def test_classical_row_lengths(n, h):
+    """Classical CG with short rows and with rows long enough for the pipelined row sums, against a dense solve (tolerance
+    as in test_batch_row_lengths: ||A^-1|| <= 1, ||A|| <= 2 (2h + 1) + 1 <= 163)."""
+    import paper_1701_03989_gb300 as P
+
+    if n == 5000 and h != 40:
+        pytest.skip("one dense solve of this size is enough")
+    a, rp, ci, v = _banded(n, h, n + h)
+    b = np.random.default_rng(n).uniform(-1, 1, n)
+    op = P.ascg_op_create_csr(n, len(v), rp, ci, v, 0)
+    x = torch.zeros(n, dtype=torch.float64, device="cuda")
+    res = P.ascg_solve(op, torch.from_numpy(b).cuda(), x, P.make_options(method="classical", eps_target=1e-12, max_iters=5000))
+    P.ascg_op_destroy(op)
+    ref = np.linalg.solve(a, b)
+    assert res.status == P.ASCG_OK
+    assert np.linalg.norm(x.cpu().numpy() - ref) <= 4e-12 * 163 * np.linalg.norm(ref)
