@@ -341,8 +341,8 @@ bool gram_tc_fits(int64_t n);
 // are whole 1024-row chunks of one system each (GramItem rows in Y, nrows a
 // multiple of 1024, at most 8 chunks), each run as one or more pieces of whole
 // chunks; pieces of systems with sys_w 0 skip.
-// Each piece takes its system's column exponents (emax_all: 33 ints per
-// system, filled by launch_tc_items_exponents or the matrix powers steps).
+// Each piece takes its system's column exponents (emax_all: kEmaxCopies x 33
+// ints per system, filled by launch_tc_items_exponents or the matrix powers steps).
 // Each item gets w(w+1)/2 partials, of which the pairs of its system's own
 // sys_w columns hold values. Where an item has several pieces: sums, w(w+1)
 // words per item, and tickets, one per item, zero on entry and left zero.
@@ -356,8 +356,8 @@ struct GramPiece {
 cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramPiece* pieces,
                                  int npieces, const int* sys_w, const int* emax_all, double* partials,
                                  unsigned long long* sums, unsigned* tickets, cudaStream_t s);
-// The column exponents of every item's system (emax_all zeroed here), by a pass over Y.
-cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramItem* items, int nitems,
+// The column exponents of every piece's system (emax_all zeroed here), by a pass over Y.
+cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramPiece* pieces, int npieces,
                                       const int* sys_w, int nsys, int* emax_all, cudaStream_t s);
 // Recovery (eq. coords) on the tensor cores: x += Y x', r = Y r', p = Y p' in
 // one pass, with the Gram's digit split of Y (col_emax: the Gram's column
@@ -395,15 +395,23 @@ struct RowItem {
   int sys;
   int row0;
   int nrows;
-  int by_chain;  // matrix powers items: see mpk_by_chain
+  int pad_;
 };
-// Rows of a matrix powers item: one CTA of 128 threads.
-constexpr int kMpkChainRows = 64, kMpkBothRows = 128;
+// Copies of a system's column exponents (kMaxW ints each) that its CTAs spread
+// their maxima over: atomics on one address take about 1 ns each, and with one
+// copy and one per warp a 140^3 system's steps took 41 ms instead of 28.
+constexpr int kEmaxCopies = 8;
+// Rows of a matrix powers item with a warp per chain.
+constexpr int kMpkChainRows = 64;
 // Matrix powers step j (monomial basis) of every system q with j < sys_steps[q].
-// emax_all (nsys x kMaxW ints, zeroed before step 0, or nullptr): the largest
-// biased exponent of every column formed, and of columns 0 and 1.
+// items: kMpkChainRows rows each, a warp per chain. emax_all (nsys x kEmaxCopies x kMaxW ints, zeroed before
+// step 0, or nullptr): the largest biased exponent of every column formed, and
+// of columns 0 and 1, is the maximum over the system's copies.
 cudaError_t launch_mpk_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
                              int* emax_all, cudaStream_t s);
+// The same with kRowItem rows per item and both chains in a thread, without exponents.
+cudaError_t launch_mpk_items_both(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
+                                  cudaStream_t s);
 // b - A x of the systems with sel[q] != 0: into Y columns 1 and 0, or into column 2.
 cudaError_t launch_residual_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sel,
                                   int into_col2, cudaStream_t s);

@@ -22,19 +22,29 @@ __device__ __forceinline__ bool item_row(const RowItem* items, int64_t* row, int
 // eq. (polybasiscg)) for every system q with j < sys_steps[q]: column 2j+2 =
 // A column 2j and, while j + 1 < sbar_q, column 2j+3 = A column 2j+1, A = D + O.
 //
-// An item is one CTA of 128 threads. by_chain (mpk_by_chain): one warp per
-// 32-row slice and chain (P or R), the two chains of two slices; the second
-// warp of a slice finds A in L1. A row's sum is one chain of dependent FMAs,
-// 64 cycles each on GB300, so a long row costs its length in latency however
-// idle the GPU is: the two chains on two warps halve that, and small CTAs
-// spread a small system over more SMs. row_chain keeps two groups of A and one
-// of gathers in flight. Otherwise: 128 rows, both chains in one thread.
-// 8 CTAs per SM (64 registers) beat 7 (72) by 4 % and 10 (48, spilling) by
-// 18 %. FP64-bound: 1.71M warp FMAs (10 systems, two banded of 117 and 129
-// entries a row) take 111 us, 0.79 of the FP64 pipe. 32 systems of 1e3..1e5
-// rows, targets 1e-8 and 1e-12: 236.4 -> 195.1 ms a batch with the exponents
-// folded in below (one thread per row with both chains in 256-row CTAs, and a
-// pass over the bases for the exponents before).
+// Two kernels. mpk_items_kernel: one warp per 32-row
+// slice and chain (P or R), an item of 64 rows per CTA of 128 threads; the
+// second warp of a slice finds A in L1. A row's sum is one chain of dependent
+// FMAs, 64 cycles each on GB300, so a long row costs its length in latency
+// however idle the GPU is: the two chains on two warps halve that, and small
+// CTAs spread a small system over more SMs. row_chain keeps two groups of A and
+// one of gathers in flight. 8 CTAs per SM (64 registers) beat 7 (72) by 4 % and
+// 10 (48, spilling) by 18 %. FP64-bound: 1.71M warp FMAs (10 systems, two banded
+// of 117 and 129 entries a row) take 111 us, 0.79 of the FP64 pipe. 32 systems of
+// 1e3..1e5 rows, targets 1e-8 and 1e-12: 236.4 -> 195.1 ms a batch with the
+// exponents folded in below (one thread per row with both chains in 256-row
+// CTAs, and a pass over the bases for the exponents before).
+// It records the largest biased exponent of the columns written (and, at step 0,
+// of the input columns) for the tensor-core Gram, in place of another pass over
+// the basis: one atomic without return per warp, into one of the system's
+// kEmaxCopies copies.
+//
+// mpk_items_both_kernel: 256 rows, both chains in one thread, for batches with so
+// many rows that the GPU is full anyway (Lockstep::rebuild_tables): A is read
+// once, the items stay in system order, which mixes FP64-bound long rows with
+// HBM-bound short ones, and the exponents take a pass of their own (recording
+// them here, even once per CTA, was slower: 140^3, 60 iterations, 29.7 ms
+// against 27.8).
 __global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __restrict__ descs,
                                                            const RowItem* __restrict__ items,
                                                            const int* __restrict__ sys_steps, int j,
@@ -42,8 +52,7 @@ __global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __rest
   const RowItem it = items[blockIdx.x];
   const SysDesc d = descs[it.sys];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ch = it.by_chain ? warp & 1 : 0;
-  const int first = kSlice * (it.by_chain ? warp >> 1 : warp);
+  const int ch = warp & 1, first = kSlice * (warp >> 1);
   const bool any = first < it.nrows, on = first + lane < it.nrows;
   const int64_t row = (int64_t)it.row0 + first + lane;
   int64_t b = 0;
@@ -60,53 +69,53 @@ __global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __rest
   const int steps = load_after_wait(sys_steps + it.sys);
   if (!any || j + ch >= steps) return;  // uniform over the warp: no step j, or no R chain in the last one
   const double* x = after_wait(d.Y + (int64_t)(2 * j + ch) * d.ldY);
-  double* y = d.Y + (int64_t)(2 * j + 2 + ch) * d.ldY;
-  const double* v = d.o_val + b + lane;
-  const int32_t* c = d.o_col + b + lane;
-  const bool both = !it.by_chain && j + 1 < steps;
   const double xi = on ? x[row] : 0.0;
-  double t = dg * xi, xr = 0.0, tr = 0.0;
-  if (!both) {
-    t = row_chain(v, c, width, x, t);
-  } else {
-    const double* r = x + d.ldY;
-    xr = on ? r[row] : 0.0;
-    tr = dg * xr;
-    int k = 0;
-    for (; k + 2 <= width; k += 2) {
-      const int c0 = __ldg(c + kSlice * k), c1 = __ldg(c + kSlice * (k + 1));
-      const double a0 = __ldg(v + kSlice * k), a1 = __ldg(v + kSlice * (k + 1));
-      const double p0 = __ldg(x + c0), p1 = __ldg(x + c1);
-      const double r0 = __ldg(r + c0), r1 = __ldg(r + c1);
-      t = fma(a0, p0, t);
-      tr = fma(a0, r0, tr);
-      t = fma(a1, p1, t);
-      tr = fma(a1, r1, tr);
-    }
-    if (k < width) {
+  const double t = row_chain(d.o_val + b + lane, d.o_col + b + lane, width, x, dg * xi);
+  if (on) d.Y[(int64_t)(2 * j + 2 + ch) * d.ldY + row] = t;
+  if (!emax_all) return;
+  int* em = emax_all + ((int64_t)it.sys * kEmaxCopies + (blockIdx.x & (kEmaxCopies - 1))) * kMaxW + ch;
+  const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(t) : 0u);
+  if (lane == 0) atomicMax(em + 2 * j + 2, (int)e);
+  if (j == 0) {
+    const unsigned e0 = __reduce_max_sync(0xffffffffu, biased_exp(xi));
+    if (lane == 0) atomicMax(em, (int)e0);
+  }
+}
+
+__global__ void __launch_bounds__(kRowItem) mpk_items_both_kernel(const SysDesc* __restrict__ descs,
+                                                                  const RowItem* __restrict__ items,
+                                                                  const int* __restrict__ sys_steps, int j) {
+  pdl_wait();
+  pdl_release();
+  int64_t row;
+  int q;
+  if (!item_row(items, &row, &q)) return;
+  const int steps = load_after_wait(sys_steps + q);
+  if (j >= steps) return;  // uniform over the CTA
+  const SysDesc d = descs[q];
+  const double* pj = d.Y + (int64_t)(2 * j) * d.ldY;
+  const double* rj = d.Y + (int64_t)(2 * j + 1) * d.ldY;
+  const int64_t sl = row >> 5;
+  const int l = (int)(row & 31);
+  const int64_t b = d.o_ptr[sl];
+  const int width = (int)((d.o_ptr[sl + 1] - b) >> 5);
+  const double* v = d.o_val + b + l;
+  const int32_t* c = d.o_col + b + l;
+  const double dg = d.diag[row];
+  double tp = dg * pj[row];
+  if (j + 1 < steps) {
+    double tr = dg * rj[row];
+    for (int k = 0; k < width; ++k) {
       const double a = __ldg(v + kSlice * k);
       const int cc = __ldg(c + kSlice * k);
-      t = fma(a, __ldg(x + cc), t);
-      tr = fma(a, __ldg(r + cc), tr);
+      tp = fma(a, __ldg(pj + cc), tp);
+      tr = fma(a, __ldg(rj + cc), tr);
     }
-    if (on) y[d.ldY + row] = tr;
+    d.Y[(int64_t)(2 * j + 3) * d.ldY + row] = tr;
+  } else {
+    for (int k = 0; k < width; ++k) tp = fma(__ldg(v + kSlice * k), __ldg(pj + __ldg(c + kSlice * k)), tp);
   }
-  if (on) y[row] = t;
-  if (!emax_all) return;
-  // the largest biased exponent of the columns written (and, at step 0, of the
-  // input columns) for the tensor-core Gram: one reduction without return per
-  // warp and column, in place of another pass over the basis
-  int* em = emax_all + (int64_t)it.sys * kMaxW + ch;
-  const auto record = [&](int col, double val) {
-    const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(val) : 0u);
-    if (lane == 0) atomicMax(em + col, (int)e);
-  };
-  record(2 * j + 2, t);
-  if (both) record(2 * j + 3, tr);
-  if (j == 0) {
-    record(0, xi);
-    if (both) record(1, xr);
-  }
+  d.Y[(int64_t)(2 * j + 2) * d.ldY + row] = tp;
 }
 
 // Residual of the systems with sel[q] != 0: into columns 1 (r) and 0 (p) of Y
@@ -216,6 +225,12 @@ cudaError_t launch_mpk_items(const SysDesc* descs, const RowItem* items, int nit
                              int* emax_all, cudaStream_t s) {
   if (nitems < 1) return cudaSuccess;
   return launch_pdl(mpk_items_kernel, nitems, 128, s, descs, items, sys_steps, j, emax_all);
+}
+
+cudaError_t launch_mpk_items_both(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
+                                  cudaStream_t s) {
+  if (nitems < 1) return cudaSuccess;
+  return launch_pdl(mpk_items_both_kernel, nitems, kRowItem, s, descs, items, sys_steps, j);
 }
 
 cudaError_t launch_residual_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sel,

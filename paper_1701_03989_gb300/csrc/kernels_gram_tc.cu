@@ -555,13 +555,14 @@ struct PieceSums {
 // The Gram partial of the chunks ch = c_lo, c_lo + c_step, ... < c_hi of the
 // rows [row_base, row_base + n_local) of the tensor map's matrix (chunk ch
 // starts at row row_base + ch * kTChunk), over the first w columns (the others
-// count as zero) with the column exponents col_emax, written to out[w_out
+// count as zero) with the column exponents (the maximum of `copies` sets of
+// kTW in col_emax), written to out[w_out
 // (w_out + 1) / 2], w <= w_out. Run by a whole CTA of kTcThreads. guard: the
 // wait limit, where a wait that ran out is reported, and the stall test's
 // stage (see TcGuard). ps: this CTA's part in a sum of several (see PieceSums).
 __device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w_out, int w, int64_t row_base, int64_t c_lo,
                                              int64_t c_hi, int64_t c_step, int64_t n_local,
-                                             const int* __restrict__ col_emax, double* __restrict__ out,
+                                             const int* __restrict__ col_emax, int copies, double* __restrict__ out,
                                              const TcGuard guard, const PieceSums ps) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* dstage = smem + kDOff;
@@ -609,7 +610,12 @@ __device__ __forceinline__ void gram_tc_body(const CUtensorMap* ymap_p, int w_ou
   // everything above touches only this CTA: it overlaps the previous kernel
   pdl_wait();
   pdl_release();
-  if (tid < kTW) s_emax[tid] = tid < w ? __ldcg(col_emax + tid) : 0;
+  if (tid < kTW) {
+    int e = 0;
+    if (tid < w)
+      for (int c = 0; c < copies; ++c) e = max(e, __ldcg(col_emax + c * kTW + tid));
+    s_emax[tid] = e;
+  }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -815,7 +821,7 @@ __global__ void __maxnreg__(kTcRegs)
     pdl_wait();
     return;
   }
-  gram_tc_body(&ymap, w, w, 0, blockIdx.x, (n + kTChunk - 1) / kTChunk, gridDim.x, n, col_emax,
+  gram_tc_body(&ymap, w, w, 0, blockIdx.x, (n + kTChunk - 1) / kTChunk, gridDim.x, n, col_emax, 1,
                partials + (int64_t)blockIdx.x * (w * (w + 1) / 2), guard, PieceSums{nullptr, nullptr, 1});
 }
 
@@ -836,8 +842,8 @@ __global__ void __maxnreg__(kTcRegs)
   }
   const int64_t nch = it.nrows / kTChunk;
   const int np = w * (w + 1) / 2;
-  gram_tc_body(&ymap, w, wq, it.row0, 0, nch, 1, nch * kTChunk, emax_all + (int64_t)it.sys * kTW,
-               partials + (int64_t)it.item * np, TcGuard{kWaitLimit, -1, nullptr, nullptr},
+  gram_tc_body(&ymap, w, wq, it.row0, 0, nch, 1, nch * kTChunk, emax_all + (int64_t)it.sys * kEmaxCopies * kTW,
+               kEmaxCopies, partials + (int64_t)it.item * np, TcGuard{kWaitLimit, -1, nullptr, nullptr},
                PieceSums{sums + (int64_t)it.item * 2 * np, tickets + it.item, it.pieces});
 }
 
@@ -874,11 +880,11 @@ __global__ void __launch_bounds__(256) col_exponent_kernel(int64_t n, const doub
 // system) and folds the largest biased exponent of each of its w columns into
 // emax_all[sys * kTW + c] (zeroed before the launch).
 __global__ void __launch_bounds__(256) tc_items_exponent_kernel(int w, const double* __restrict__ Y, int64_t ldY,
-                                                                const GramItem* __restrict__ items,
+                                                                const GramPiece* __restrict__ items,
                                                                 const int* __restrict__ sys_w,
                                                                 int* __restrict__ emax_all) {
   __shared__ unsigned red[8][kTW];
-  const GramItem it = items[blockIdx.x];
+  const GramPiece it = items[blockIdx.x];
   if (sys_w[it.sys] == 0) return;  // uniform over the CTA
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   auto ex = [](double v) { return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu; };
@@ -902,7 +908,7 @@ __global__ void __launch_bounds__(256) tc_items_exponent_kernel(int w, const dou
   if (threadIdx.x < w) {
     unsigned m = 0;
     for (int g = 0; g < 8; ++g) m = max(m, red[g][threadIdx.x]);
-    if (m > 0) atomicMax(emax_all + (int64_t)it.sys * kTW + threadIdx.x, (int)m);
+    if (m > 0) atomicMax(emax_all + (int64_t)it.sys * kEmaxCopies * kTW + threadIdx.x, (int)m);
   }
 }
 
@@ -1313,12 +1319,12 @@ cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t ro
                        emax_all, partials, sums, tickets);
 }
 
-cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramItem* items, int nitems,
+cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramPiece* pieces, int npieces,
                                       const int* sys_w, int nsys, int* emax_all, cudaStream_t s) {
-  if (nitems < 1) return cudaSuccess;
-  const cudaError_t e = cudaMemsetAsync(emax_all, 0, sizeof(int) * kTW * nsys, s);
+  if (npieces < 1) return cudaSuccess;
+  const cudaError_t e = cudaMemsetAsync(emax_all, 0, sizeof(int) * kTW * kEmaxCopies * nsys, s);
   if (e != cudaSuccess) return e;
-  tc_items_exponent_kernel<<<nitems, 256, 0, s>>>(w, Y, ldY, items, sys_w, emax_all);
+  tc_items_exponent_kernel<<<npieces, 256, 0, s>>>(w, Y, ldY, pieces, sys_w, emax_all);
   return cudaGetLastError();
 }
 

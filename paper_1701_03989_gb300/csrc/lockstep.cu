@@ -329,7 +329,7 @@ class Lockstep {
     LS_TRY(dalloc(&d_sums_, (size_t)2 * lanes));
     LS_TRY(dalloc(&d_params_, (size_t)3 * kMaxS));
     LS_TRY(dalloc(&d_spec_, (size_t)lanes * kSpecDoubles));
-    LS_TRY(dalloc(&d_emax_, (size_t)lanes * kMaxW));
+    LS_TRY(dalloc(&d_emax_, (size_t)lanes * kEmaxCopies * kMaxW));
     LS_TRY(dalloc(&d_tickets_, (size_t)lanes));
     if (rcap_) LS_TRY(dalloc(&d_res_hist_, (size_t)lanes * rcap_));
     if (abcap_) LS_TRY(dalloc(&d_ab_hist_, (size_t)lanes * 2 * abcap_));
@@ -361,21 +361,20 @@ class Lockstep {
   static int64_t row_items_of(int64_t n) { return (n + kRowItem - 1) / kRowItem; }
   // Tensor-core Gram items: up to kTcItemRows rows (whole 1024-row chunks) each.
   static constexpr int64_t kTcItemRows = 8192;
-  // Pieces of the items (GramPiece), one CTA each. With few items (at most
-  // kSplitItems) an item is cut into pieces of about a third of the chunks per
-  // SM, so that a handful of systems still covers the SMs: a CTA takes about 5
-  // us for the launch, pipeline fill and epilogue and 9 us per chunk, and with
-  // whole items a 93057-row system alone had 12 CTAs of 78 us. 32 systems of
-  // 1e3..1e5 rows: 190.4 -> 182.2 ms a batch; 16 served requests: 334 -> 330.
+  // Pieces of the items (GramPiece), one CTA each. With few chunks (below six per
+  // SM, in at most kSplitItems items) every chunk is a piece, so that a handful of
+  // systems still covers the SMs: a CTA takes about 5 us for the launch, pipeline
+  // fill and epilogue and 9 us per chunk, and with whole items a 93057-row system
+  // alone had 12 CTAs of 78 us. 32 systems of 1e3..1e5 rows (690 chunks): 190.4 ->
+  // 182.2 ms a batch. With more, whole items: one system of 977 chunks, 60
+  // iterations, 24.6 ms in pieces of two chunks, 23.9 whole.
   static constexpr int kSplitItems = 256;
   static std::vector<GramPiece> pieces_of(const std::vector<GramItem>& items) {
     std::vector<GramPiece> out;
     int64_t chunks = 0;
     for (const GramItem& it : items) chunks += it.nrows / Arena::kRowAlign;
     const int64_t most = kTcItemRows / Arena::kRowAlign;
-    const int64_t per = (int)items.size() > kSplitItems
-                            ? most
-                            : std::max<int64_t>(1, std::min<int64_t>(most, chunks / (3 * gram_grid())));
+    const int64_t per = (int)items.size() <= kSplitItems && chunks < 6 * gram_grid() ? 1 : most;
     const int64_t rows = per * Arena::kRowAlign;
     for (size_t i = 0; i < items.size(); ++i) {
       const int np = (int)((items[i].nrows + rows - 1) / rows);
@@ -619,12 +618,18 @@ class Lockstep {
     int* d_wtc = d_int_ + kWTc * lanes_;
     int* d_tc0 = d_int_ + kTcItem0 * lanes_;
     int* d_tcn = d_int_ + kTcNItems * lanes_;
-    const int nr = (int)ritems_.size(), ng = (int)gitems_.size();
+    const int nr = (int)ritems_.size(), ng = (int)gitems_.size(), nm = (int)mitems_.size();
     const int Wb = 2 * max_sbar + 1;
-    // the steps record the column exponents that the tensor-core Gram needs
-    if (tc_gram) LS_CUDA(cudaMemsetAsync(d_emax_, 0, sizeof(int) * kMaxW * hi_, s_));
-    for (int j = 0; j < max_sbar; ++j)
-      LS_CUDA(launch_mpk_items(d_desc_, d_mitems_, (int)mitems_.size(), d_steps, j, tc_gram ? d_emax_ : nullptr, s_));
+    if (use_both_) {
+      for (int j = 0; j < max_sbar; ++j) LS_CUDA(launch_mpk_items_both(d_desc_, d_mitems_, nm, d_steps, j, s_));
+      if (tc_gram)
+        LS_CUDA(launch_tc_items_exponents(Wb, ybase_, yld_, d_pieces_, (int)pieces_.size(), d_wtc, hi_, d_emax_, s_));
+    } else {
+      // the steps record the column exponents that the tensor-core Gram needs
+      if (tc_gram) LS_CUDA(cudaMemsetAsync(d_emax_, 0, sizeof(int) * kEmaxCopies * kMaxW * hi_, s_));
+      for (int j = 0; j < max_sbar; ++j)
+        LS_CUDA(launch_mpk_items(d_desc_, d_mitems_, nm, d_steps, j, tc_gram ? d_emax_ : nullptr, s_));
+    }
     if (item_gram) {
       // pair groups: enough CTAs to cover the SMs twice
       const int groups = std::max(1, std::min(16, (2 * gram_grid() + ng - 1) / std::max(ng, 1)));
@@ -997,21 +1002,28 @@ class Lockstep {
       for (int64_t r = 0; r < n; r += gr) gitems_.push_back(GramItem{r, (int)std::min<int64_t>(gr, n - r), q});
       h_nitems[q] = (int)gitems_.size() - h_item0[q];
     }
-    // row items, the longest rows first: an item's time is its rows' length, so
-    // the last CTAs of a launch are the short ones
+    int64_t rows_all = 0;
     std::vector<int> order;
-    for (int q = 0; q < hi_; ++q)
-      if (used_[q]) order.push_back(q);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return lane_[a].row_len > lane_[b].row_len; });
-    for (int q : order) {
-      const int64_t n = lane_[q].d.n;
-      for (int64_t r = 0; r < n; r += kRowItem)
-        ritems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(kRowItem, n - r), 0});
-      const bool by_chain = mpk_by_chain(n, lane_[q].row_len);
-      const int64_t mr = by_chain ? kMpkChainRows : kMpkBothRows;
-      for (int64_t r = 0; r < n; r += mr)
-        mitems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(mr, n - r), by_chain ? 1 : 0});
+    for (int q = 0; q < hi_; ++q) {
+      if (!used_[q]) continue;
+      order.push_back(q);
+      rows_all += lane_[q].d.n;
+      for (int64_t r = 0; r < lane_[q].d.n; r += kRowItem)
+        ritems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(kRowItem, lane_[q].d.n - r), 0});
     }
+    // Matrix powers items: from kBothRows rows in all, 256 rows with both chains in
+    // a thread, in system order; below, where latency counts, 64 rows with a warp
+    // per chain, the longest rows first (an item's time is its rows' length, so
+    // the last CTAs of a launch are the short ones). By chain / both in a thread:
+    // 0.69M rows in 32 systems 182 / 236 ms, 11.3M rows in 256 systems 3.74 / 3.42
+    // s, 2.7M rows of one 140^3 system 41 / 28 ms.
+    use_both_ = rows_all >= kBothRows;
+    if (!use_both_)
+      std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return lane_[a].row_len > lane_[b].row_len; });
+    const int64_t mr = use_both_ ? kRowItem : kMpkChainRows;
+    for (int q : order)
+      for (int64_t r = 0; r < lane_[q].d.n; r += mr)
+        mitems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(mr, lane_[q].d.n - r), 0});
     LS_TRY(grow_items((int64_t)ritems_.size(), (int64_t)gitems_.size()));
     LS_TRY(grow_mitems((int64_t)mitems_.size()));
     pieces_ = pieces_of(titems_);
@@ -1038,6 +1050,7 @@ class Lockstep {
     return ASCG_OK;
   }
 
+  static constexpr int64_t kBothRows = (int64_t)1 << 20;
   static constexpr size_t kMaxGraphs = 64;
   void drop_graphs() {
     for (auto& kv : graphs_) cudaGraphExecDestroy(kv.second);
@@ -1070,6 +1083,7 @@ class Lockstep {
   std::vector<GramItem> gitems_;
   std::vector<GramItem> titems_;
   std::vector<RowItem> mitems_;  // matrix powers items
+  bool use_both_ = false;        // of launch_mpk_items_both
   int64_t rcap_items_ = 0, gcap_items_ = 0, mcap_items_ = 0;
   SysDesc* d_desc_ = nullptr;
   BlockState* d_bst_ = nullptr;
@@ -1092,7 +1106,7 @@ class Lockstep {
   unsigned* d_ptick_ = nullptr;            // and their tickets
   int64_t pcap_ = 0;
   double* d_tpart_ = nullptr;     // their partials, tcnp_ each
-  int* d_emax_ = nullptr;         // per-lane column exponents, kMaxW each
+  int* d_emax_ = nullptr;         // per-lane column exponents, kEmaxCopies x kMaxW each
   int64_t tcap_items_ = 0;
   int tcnp_ = 0;
   LaneRun* d_run_ = nullptr;      // device-driven block loop: the lanes' running state
@@ -1546,7 +1560,7 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
   LS_TRY(dalloc(&B.G, (size_t)kMaxW * kMaxW));
   LS_TRY(dalloc(&B.part, (size_t)max_items * np));
   LS_TRY(dalloc(&B.tpart, (size_t)max_titems * np));
-  LS_TRY(dalloc(&B.emax, (size_t)kMaxW));
+  LS_TRY(dalloc(&B.emax, (size_t)kEmaxCopies * kMaxW));
   LS_TRY(dalloc(&B.ints, 5));
   LS_TRY(dalloc(&B.desc, 1));
   LS_TRY(dalloc(&B.items, (size_t)max_items));
@@ -1582,7 +1596,7 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
     LS_CUDA(cudaMemcpyAsync(B.pieces, pieces.data(), sizeof(GramPiece) * pieces.size(), cudaMemcpyHostToDevice, s));
     LS_CUDA(cudaMemcpyAsync(B.ints, ints, sizeof(ints), cudaMemcpyHostToDevice, s));
     // a solve's exponents come from its matrix powers steps: not timed
-    LS_CUDA(launch_tc_items_exponents(w, B.Y, ld, B.titems, nt, B.ints, 1, B.emax, s));
+    LS_CUDA(launch_tc_items_exponents(w, B.Y, ld, B.pieces, (int)pieces.size(), B.ints, 1, B.emax, s));
     LS_CUDA(cudaStreamSynchronize(s));  // the host arrays above are locals
     const int groups = std::max(1, std::min(16, (2 * gram_grid() + ng - 1) / ng));
     std::vector<float> a(kReps), b(kReps);
