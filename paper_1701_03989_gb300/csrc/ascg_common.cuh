@@ -50,10 +50,11 @@ __device__ __forceinline__ unsigned biased_exp(double v) { return ((unsigned)__d
 // the lane's first entry, stride kSlice), one FMA each in stored order. In
 // groups of kRowGroup entries: while a group's FMAs run, the next group's
 // gathers and the loads of A of the group after it are in flight, so that a
-// warp alone on its scheduler waits on its FMA chain and not on memory.
+// warp alone on its scheduler waits on its FMA chain and not on memory. x may
+// have been written by the previous kernel: __ldca (see pdl_wait).
 constexpr int kRowGroup = 4;
 __device__ __forceinline__ double row_chain(const double* __restrict__ v, const int32_t* __restrict__ c, int width,
-                                            const double* __restrict__ x, double t) {
+                                            const double* x, double t) {
   constexpr int G = kRowGroup;
   double a0[G], a1[G], x0[G];
   int c1[G];
@@ -78,7 +79,7 @@ __device__ __forceinline__ double row_chain(const double* __restrict__ v, const 
       }
 #pragma unroll
     for (int q = 0; q < G; ++q)
-      if (q < width) x0[q] = __ldg(x + c0[q]);
+      if (q < width) x0[q] = __ldca(x + c0[q]);
   }
   for (int k = 0; k < width; k += G) {
     double x1[G], a2[G];
@@ -90,7 +91,7 @@ __device__ __forceinline__ double row_chain(const double* __restrict__ v, const 
     }
 #pragma unroll
     for (int q = 0; q < G; ++q)
-      if (k + G + q < width) x1[q] = __ldg(x + c1[q]);
+      if (k + G + q < width) x1[q] = __ldca(x + c1[q]);
 #pragma unroll
     for (int q = 0; q < G; ++q)
       if (k + 2 * G + q < width) {
@@ -147,16 +148,45 @@ inline cudaError_t smem_limit_once(std::atomic<uint64_t>& done, K* kernel, int b
 // no-ops, so the kernels stay correct under any launch. Every kernel launched
 // this way calls pdl_wait() at entry: a kernel that returned before its
 // predecessor finished would let its own successor overtake that predecessor.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// A pointer to what the previous kernel wrote, for use after pdl_wait(): the
-// compiler may move loads it takes for invariant (__ldg, const __restrict__)
-// above the wait, but not above the point where it learns their address.
-template <typename T>
-__device__ __forceinline__ T* after_wait(T* p) {
+//
+// The wait alone does not keep the compiler from moving a load above it: a
+// load that it takes for invariant (through a const __restrict__ parameter) is
+// not ordered with the wait, and neither is any other through a __restrict__
+// pointer, which the wait's memory clobber need not touch. Nor is __ldg right
+// for memory that is written while the kernel is already resident. So what the
+// chain of launches writes is read in one of three ways only:
+//  - by __ldca, __ldcg, __ldcs or load_after_wait: volatile statements like the
+//    wait itself, which keep their order. The kernels that are bound by their
+//    loads do this (the same code as with __ldg; with relearned pointers a matrix
+//    powers step took 12 % longer: Chebyshev, s = 16, 100^3, 531 us against 472;
+//    in classical CG it costs 0.7 % of a 128^3 solve, 43.0 -> 43.3 ms);
+//  - by ordinary loads through a pointer named in pdl_wait(), or in relearn()
+//    after it: the compiler learns its value only there;
+//  - by ordinary loads through a pointer without __restrict__, which the wait's
+//    memory clobber orders.
+// What is constant over the chain (operators, tables, coefficients) may use
+// __ldg and be loaded before the wait, and so may a word that was written
+// several kernels before. tests/test_dependent_launch_cpu.py holds every
+// kernel's pointers to this.
+// relearn() also says that the pointer is one to global memory (never null),
+// which the compiler can no longer see for itself, so that the loads through it
+// need not be generic ones.
+template <typename P>
+__device__ __forceinline__ void relearn(P& p) {
   asm volatile("" : "+l"(p));
-  return p;
+  __builtin_assume(__isGlobal(p));
 }
+template <typename P, typename... Ps>
+__device__ __forceinline__ void relearn(P& p, Ps&... ps) {
+  relearn(p);
+  relearn(ps...);
+}
+template <typename... Ps>
+__device__ __forceinline__ void pdl_wait(Ps&... ps) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if constexpr (sizeof...(Ps) > 0) relearn(ps...);
+}
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // A word that the previous kernel may have written, read after pdl_wait() (not
 // moved above it) and through L1: every CTA reads the same one, and a trip to L2
 // in each cost 7 us per 128^3 step.

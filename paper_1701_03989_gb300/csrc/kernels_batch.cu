@@ -64,11 +64,11 @@ __global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __rest
     width = (int)((d.o_ptr[sl + 1] - b) >> 5);
     if (on) dg = d.diag[row];
   }
-  pdl_wait();  // the step before (its column of Y) and the lanes' tables
+  const double* x = d.Y + (int64_t)(2 * j + ch) * d.ldY;
+  pdl_wait(x);  // the step before (its column of Y) and the lanes' tables
   pdl_release();
   const int steps = load_after_wait(sys_steps + it.sys);
   if (!any || j + ch >= steps) return;  // uniform over the warp: no step j, or no R chain in the last one
-  const double* x = after_wait(d.Y + (int64_t)(2 * j + ch) * d.ldY);
   const double xi = on ? x[row] : 0.0;
   const double t = row_chain(d.o_val + b + lane, d.o_col + b + lane, width, x, dg * xi);
   if (on) d.Y[(int64_t)(2 * j + 2 + ch) * d.ldY + row] = t;
@@ -108,12 +108,12 @@ __global__ void __launch_bounds__(kRowItem) mpk_items_both_kernel(const SysDesc*
     for (int k = 0; k < width; ++k) {
       const double a = __ldg(v + kSlice * k);
       const int cc = __ldg(c + kSlice * k);
-      tp = fma(a, __ldg(pj + cc), tp);
-      tr = fma(a, __ldg(rj + cc), tr);
+      tp = fma(a, __ldca(pj + cc), tp);
+      tr = fma(a, __ldca(rj + cc), tr);
     }
     d.Y[(int64_t)(2 * j + 3) * d.ldY + row] = tr;
   } else {
-    for (int k = 0; k < width; ++k) tp = fma(__ldg(v + kSlice * k), __ldg(pj + __ldg(c + kSlice * k)), tp);
+    for (int k = 0; k < width; ++k) tp = fma(__ldg(v + kSlice * k), __ldca(pj + __ldg(c + kSlice * k)), tp);
   }
   d.Y[(int64_t)(2 * j + 2) * d.ldY + row] = tp;
 }
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kRowItem) recover_items_kernel(const SysDesc* 
   int64_t row;
   int q;
   if (!item_row(items, &row, &q)) return;
-  const int w = sys_w[q];
+  const int w = load_after_wait(sys_w + q);
   if (w == 0) return;  // uniform over the CTA
   const SysDesc d = descs[q];
   const double* cq = coords + (int64_t)q * c_stride;
@@ -190,9 +190,9 @@ __global__ void __launch_bounds__(kRowItem) recover_items_kernel(const SysDesc* 
 #pragma unroll
   for (int c = 0; c < W; ++c) {
     if (c < w) {
-      sx = fma(y[c], __ldg(cq + c), sx);
-      sr = fma(y[c], __ldg(cq + w + c), sr);
-      sp = fma(y[c], __ldg(cq + 2 * w + c), sp);
+      sx = fma(y[c], __ldca(cq + c), sx);
+      sr = fma(y[c], __ldca(cq + w + c), sr);
+      sp = fma(y[c], __ldca(cq + 2 * w + c), sp);
     }
   }
   d.x[row] += sx;

@@ -23,7 +23,7 @@ namespace {
 // is otherwise a gather's latency per entry.
 enum SellMode { kKeep, kStream, kChain };
 template <SellMode MODE = kKeep>
-__device__ __forceinline__ double sell_row(const DevSell& A, int64_t i, const double* __restrict__ x) {
+__device__ __forceinline__ double sell_row(const DevSell& A, int64_t i, const double* x) {
   const int64_t s = i >> 5;
   const int l = (int)(i & 31);
   const int64_t b = A.ptr[s];
@@ -33,9 +33,9 @@ __device__ __forceinline__ double sell_row(const DevSell& A, int64_t i, const do
   if (MODE == kChain) return row_chain(v, c, width, x, 0.0);
   double t = 0.0;
   if (MODE == kStream) {
-    for (int j = 0; j < width; ++j) t = fma(__ldcs(v + kSlice * j), __ldg(x + __ldcs(c + kSlice * j)), t);
+    for (int j = 0; j < width; ++j) t = fma(__ldcs(v + kSlice * j), __ldca(x + __ldcs(c + kSlice * j)), t);
   } else {
-    for (int j = 0; j < width; ++j) t = fma(__ldg(v + kSlice * j), __ldg(x + __ldg(c + kSlice * j)), t);
+    for (int j = 0; j < width; ++j) t = fma(__ldg(v + kSlice * j), __ldca(x + __ldg(c + kSlice * j)), t);
   }
   return t;
 }
@@ -123,21 +123,21 @@ __global__ void __launch_bounds__(256) dot_kernel(const double* __restrict__ u, 
 // reduction and one atomic ticket, so few CTAs keep that overhead small. Each
 // warp-wide FP64 add costs a full FP64 issue slot, however few lanes need it.
 template <SellMode MODE>
-__global__ void __launch_bounds__(kSpmvRows) cg_spmv_dot_kernel(DevSell A, const double* __restrict__ p,
+__global__ void __launch_bounds__(kSpmvRows) cg_spmv_dot_kernel(DevSell A, const double* p,
                                                                 double* __restrict__ q, CGState* st,
                                                                 double* partials, unsigned* counter) {
   __shared__ double red[32];
   __shared__ int flag;
-  pdl_wait();     // the previous kernel's p and state
+  pdl_wait();  // the previous kernel's p and state
   pdl_release();
   const int done = st->done;  // uniform: written by an earlier kernel
   if (blockIdx.x == 0 && threadIdx.x == 0) st->active = !done;  // read by the next two kernels
   if (done) return;
   double part = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * kSpmvRows + threadIdx.x; i < A.n; i += (int64_t)gridDim.x * kSpmvRows) {
-    const double v = sell_row<MODE>(A, i, p);
+    const double v = sell_row<MODE>(A, i, p), pi = p[i];
     q[i] = v;
-    part = fma(p[i], v, part);
+    part = fma(pi, v, part);
   }
   part = block_sum(part, red);
   if (last_block(part, partials, counter, &flag)) {
@@ -169,13 +169,13 @@ __global__ void __launch_bounds__(256) cg_update_kernel(int64_t n, double* __res
                                                         int ab_cap) {
   __shared__ double red[32];
   __shared__ int flag;
-  pdl_wait();     // q and alpha from the SpMV
+  pdl_wait();  // q and alpha from the SpMV
   pdl_release();
   if (!st->active) return;
   const double alpha = st->alpha;
   double s = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double ri = fma(-alpha, q[i], r[i]);  // r -= A q = alpha (A p)
+    const double ri = fma(-alpha, __ldca(q + i), __ldca(r + i));  // r -= A q = alpha (A p)
     r[i] = ri;
     s = fma(ri, ri, s);
   }
@@ -213,14 +213,14 @@ __global__ void __launch_bounds__(256) cg_update_kernel(int64_t n, double* __res
 __global__ void __launch_bounds__(256) cg_pupdate_kernel(int64_t n, double* __restrict__ x,
                                                          const double* __restrict__ r, double* __restrict__ p,
                                                          const CGState* st) {
-  pdl_wait();     // r and beta from the update
+  pdl_wait();  // r and beta from the update
   pdl_release();
   if (!st->active) return;  // this iteration was skipped (solve already done)
   const double alpha = st->alpha, beta = st->beta;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double pi = p[i];
-    x[i] = fma(alpha, pi, x[i]);             // x += q, q = alpha p (the iteration's p)
-    p[i] = fma(beta, pi, r[i]);              // p = r + beta p
+    const double pi = __ldca(p + i);
+    x[i] = fma(alpha, pi, __ldca(x + i));    // x += q, q = alpha p (the iteration's p)
+    p[i] = fma(beta, pi, __ldca(r + i));     // p = r + beta p
   }
 }
 

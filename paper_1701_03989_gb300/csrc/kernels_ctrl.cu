@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(128, 3) block_ctrl_kernel(const double* __rest
                                                          double* __restrict__ ab_hist, int ab_cap, int64_t g_stride,
                                                          int64_t c_stride, double* __restrict__ spec,
                                                          unsigned* counters) {
-  pdl_wait();
+  pdl_wait(G);
   pdl_release();
   const int q = blockIdx.y;
   G += (int64_t)q * g_stride;

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_items_kernel(const SysDe
   pdl_wait();
   pdl_release();
   const GramItem it = items[blockIdx.x];
-  if (sys_w[it.sys] == 0) return;  // uniform over the CTA
+  if (load_after_wait(sys_w + it.sys) == 0) return;  // uniform over the CTA
   const SysDesc& d = descs[it.sys];
   gram_chunks<W, MOM>(it.nrows, d.Y + it.row0, d.ldY, 0, (it.nrows + kChunk - 1) / kChunk,
                       partials + (int64_t)blockIdx.x * NP, (int)blockIdx.y, (int)gridDim.y);
@@ -219,10 +219,10 @@ __global__ void __launch_bounds__(128) gram_items_moment_finalize_kernel(const d
                                                                          const int* __restrict__ sys_nitems,
                                                                          const int* __restrict__ sys_w,
                                                                          double* __restrict__ G, int64_t g_stride) {
-  pdl_wait();
+  pdl_wait(partials);
   pdl_release();
   const int q = blockIdx.x;
-  const int w = sys_w[q];
+  const int w = load_after_wait(sys_w + q);
   if (w == 0) return;
   __shared__ double mu[kMomSlots];
   const int S = (w - 1) / 2;
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(128) gram_items_moment_finalize_kernel(const d
 // is bitwise reproducible.
 __global__ void __launch_bounds__(128) gram_finalize_kernel(int w, const double* __restrict__ partials, int nparts,
                                                             double* __restrict__ G, const int* __restrict__ gate) {
-  pdl_wait();
+  pdl_wait(partials);
   pdl_release();
   if (gate_closed(gate)) return;
   const int np = w * (w + 1) / 2;
@@ -286,10 +286,10 @@ __global__ void __launch_bounds__(256) gram_items_finalize_kernel(int W, const d
                                                                   const int* __restrict__ sys_nitems,
                                                                   const int* __restrict__ sys_w, double* __restrict__ G,
                                                                   int64_t g_stride) {
-  pdl_wait();
+  pdl_wait(partials);
   pdl_release();
   const int q = blockIdx.x;
-  const int w = sys_w[q];
+  const int w = load_after_wait(sys_w + q);
   if (w == 0) return;
   const int NP = W * (W + 1) / 2;
   const int i0 = sys_item0[q], ni = sys_nitems[q];

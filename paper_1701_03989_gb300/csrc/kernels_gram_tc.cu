@@ -1055,7 +1055,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   // everything above touches only this CTA: it overlaps the previous kernel
-  pdl_wait();
+  pdl_wait(x);
   pdl_release();
   if (tid < kTW) s_emax[tid] = tid < w ? __ldcg(col_emax + tid) : 0;
   __syncthreads();

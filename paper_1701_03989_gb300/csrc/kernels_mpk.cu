@@ -39,13 +39,16 @@ namespace {
 // The exponent work always runs (a few integer operations per row); a
 // variant without it measured slower (63.5 us).
 // SIG: 0 no sigma term (j = 0 or sig_j = 0); 1 sig_j = 1 exactly (the
-// Chebyshev basis, where sigma_{j-1} = gamma_j); 2 any other sig_j. The sum
+// Chebyshev basis, where sigma_{j-1} = gamma_j); 2 any other sig_j. Y is not
+// __restrict__: a row's own entries are ordinary loads, ordered after the wait,
+// that the compiler places where they hit L1 (as volatile loads at this point a
+// Chebyshev basis, s = 16, at 100^3 took 532 us, not 472). The sum
 // starts from -sig_j rho_{j-1} and takes the diagonal term as its first FMA,
 // so with SIG = 1 a row costs nnz_row FP64 instructions per chain.
 template <int SIG, bool R>
 __global__ void __launch_bounds__(kSpmvRows, 6)
     mpk_split_step_kernel(DevSell O, const double* __restrict__ oval, const double* __restrict__ dtil, double sig,
-                          double* __restrict__ Y, int64_t ldY, int j, int* emax_part, int64_t emax_ld,
+                          double* Y, int64_t ldY, int j, int* emax_part, int64_t emax_ld,
                           const int* __restrict__ gate) {
   pdl_wait();     // the previous step's columns (and the gate) are written by the kernel before
   pdl_release();  // the next step may be scheduled once every CTA of this one has started
@@ -61,7 +64,7 @@ __global__ void __launch_bounds__(kSpmvRows, 6)
     const int width = (int)((O.ptr[sl + 1] - b) >> 5);
     const double* v = oval + b + l;
     const int32_t* c = O.col + b + l;
-    const double dt = dtil[row];
+    const double dt = __ldca(dtil + row);  // folded by a kernel before step 0, as oval
     // rho_{j+1} = (Dt_j + Ot_j) rho_j - sig_j rho_{j-1}
     double tp, tr = 0.0;
     if (SIG == 0) {
@@ -79,9 +82,9 @@ __global__ void __launch_bounds__(kSpmvRows, 6)
     for (; k + 2 <= width; k += 2) {
       const int c0 = __ldcs(c + kSlice * k), c1 = __ldcs(c + kSlice * (k + 1));
       const double a0 = __ldcs(v + kSlice * k), a1 = __ldcs(v + kSlice * (k + 1));
-      const double p0 = __ldg(pj + c0), p1 = __ldg(pj + c1);
+      const double p0 = __ldca(pj + c0), p1 = __ldca(pj + c1);
       if (R) {
-        const double r0 = __ldg(rj + c0), r1 = __ldg(rj + c1);
+        const double r0 = __ldca(rj + c0), r1 = __ldca(rj + c1);
         tp = fma(a0, p0, tp);
         tr = fma(a0, r0, tr);
         tp = fma(a1, p1, tp);
@@ -94,8 +97,8 @@ __global__ void __launch_bounds__(kSpmvRows, 6)
     if (k < width) {
       const double a = __ldcs(v + kSlice * k);
       const int cc = __ldcs(c + kSlice * k);
-      tp = fma(a, __ldg(pj + cc), tp);
-      if (R) tr = fma(a, __ldg(rj + cc), tr);
+      tp = fma(a, __ldca(pj + cc), tp);
+      if (R) tr = fma(a, __ldca(rj + cc), tr);
     }
     Y[(int64_t)(2 * j + 2) * ldY + row] = tp;
     if (R) Y[(int64_t)(2 * j + 3) * ldY + row] = tr;
@@ -146,27 +149,30 @@ __global__ void __launch_bounds__(128, 8)
   // wait on the previous step. (Before step 0 the operator itself may have
   // been written by the kernel just before, the folding of the coefficients.)
   if (j == 0) pdl_wait();
+  const double* v = oval;
+  relearn(v);
   int64_t b = 0;
   int width = 0;
   double dt = 0.0;
   if (any) {
     b = O.ptr[sl];
     width = (int)((O.ptr[sl + 1] - b) >> 5);
-    if (on) dt = dtil[row];
+    if (on) dt = __ldcg(dtil + row);
   }
   if (j > 0) pdl_wait();
+  const double* x = Y + (int64_t)(2 * j + ch) * ldY;
+  relearn(x);
   pdl_release();
   if (!any || gate_closed(gate)) return;  // uniform over the warp
-  const double* x = after_wait(Y + (int64_t)(2 * j + ch) * ldY);
   const double xi = on ? x[row] : 0.0;
   double t;
   if (SIG == 0) {
     t = dt * xi;
   } else {
-    const double z = on ? Y[(int64_t)(2 * j - 2 + ch) * ldY + row] : 0.0;
+    const double z = on ? __ldcg(Y + (int64_t)(2 * j - 2 + ch) * ldY + row) : 0.0;
     t = fma(dt, xi, SIG == 1 ? -z : -sig * z);
   }
-  t = row_chain(oval + b + lane, O.col + b + lane, width, x, t);
+  t = row_chain(v + b + lane, O.col + b + lane, width, x, t);
   if (on) Y[(int64_t)(2 * j + 2 + ch) * ldY + row] = t;
   if (!emax_part) return;
   const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(t) : 0u);
@@ -176,7 +182,7 @@ __global__ void __launch_bounds__(128, 8)
     const unsigned e0 = __reduce_max_sync(0xffffffffu, on ? biased_exp(xi) : 0u);
     if (lane == 0) emax_part[(int64_t)ch * emax_ld + sl] = (int)e0;
     if (!R) {
-      const unsigned e1 = __reduce_max_sync(0xffffffffu, on ? biased_exp(Y[ldY + row]) : 0u);
+      const unsigned e1 = __reduce_max_sync(0xffffffffu, on ? biased_exp(__ldcg(Y + ldY + row)) : 0u);
       if (lane == 0) emax_part[emax_ld + sl] = (int)e1;
     }
   }
@@ -251,14 +257,14 @@ template <int W>
 __global__ void __launch_bounds__(256, 6) recover_kernel(int64_t n, const double* Y, int64_t ldY,
                                                          const double* __restrict__ coords, double* x, double* r,
                                                          double* p, const int* __restrict__ gate) {
-  pdl_wait();
+  pdl_wait(coords);
   pdl_release();
   if (gate_closed(gate)) return;
   __shared__ double cx[W], cr[W], cp[W];
   if (threadIdx.x < W) {
-    cx[threadIdx.x] = __ldcg(coords + threadIdx.x);
-    cr[threadIdx.x] = __ldcg(coords + W + threadIdx.x);
-    cp[threadIdx.x] = __ldcg(coords + 2 * W + threadIdx.x);
+    cx[threadIdx.x] = coords[threadIdx.x];
+    cr[threadIdx.x] = coords[W + threadIdx.x];
+    cp[threadIdx.x] = coords[2 * W + threadIdx.x];
   }
   __syncthreads();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
