@@ -922,54 +922,42 @@ class Lockstep {
     return c;
   }
 
-  ascg_status grow_titems(int64_t titems, int64_t pieces) {
-    if (titems > tcap_items_) {
-      LS_CUDA(cudaStreamSynchronize(s_));
-      dfree(d_tpart_);
-      tcap_items_ = std::max<int64_t>(titems, 2 * tcap_items_);
-      LS_TRY(dalloc(&d_tpart_, (size_t)tcap_items_ * tcnp_));
-    }
-    if (pieces > pcap_) {
-      LS_CUDA(cudaStreamSynchronize(s_));
-      dfree(d_pieces_);
-      pcap_ = std::max<int64_t>(pieces, 2 * pcap_);
-      LS_TRY(dalloc(&d_pieces_, (size_t)pcap_));
-    }
-    if (!d_psums_) {  // the sums of split items, left zero by every block
-      LS_TRY(dalloc(&d_psums_, (size_t)kSplitItems * 2 * tcnp_));
-      LS_TRY(dalloc(&d_ptick_, (size_t)kSplitItems));
-      LS_CUDA(cudaMemsetAsync(d_psums_, 0, sizeof(unsigned long long) * kSplitItems * 2 * tcnp_, s_));
-      LS_CUDA(cudaMemsetAsync(d_ptick_, 0, sizeof(unsigned) * kSplitItems, s_));
-    }
+  // A table of at least `need` entries of `per` elements, its contents not kept.
+  // The capacity counts as zero until the new table is there, so a growth that
+  // fails is made up for by the next call.
+  template <class T>
+  ascg_status regrow(T** p, int64_t* cap, int64_t need, int64_t per = 1) {
+    if (need <= *cap) return ASCG_OK;
+    LS_CUDA(cudaStreamSynchronize(s_));
+    const int64_t want = std::max<int64_t>(need, 2 * *cap);
+    *cap = 0;
+    dfree(*p);
+    LS_TRY(dalloc(p, (size_t)(want * per)));
+    *cap = want;
     return ASCG_OK;
   }
 
-  ascg_status grow_mitems(int64_t mitems) {
-    if (mitems > mcap_items_) {
-      LS_CUDA(cudaStreamSynchronize(s_));
-      dfree(d_mitems_);
-      mcap_items_ = std::max<int64_t>(mitems, 2 * mcap_items_);
-      LS_TRY(dalloc(&d_mitems_, (size_t)mcap_items_));
+  ascg_status grow_titems(int64_t titems, int64_t pieces) {
+    LS_TRY(regrow(&d_tpart_, &tcap_items_, titems, tcnp_));
+    LS_TRY(regrow(&d_pieces_, &pcap_, pieces));
+    if (!d_ptick_) {  // the sums of split items and their tickets, left zero by every block
+      const size_t nsums = (size_t)kSplitItems * 2 * tcnp_;
+      if (!d_psums_) LS_TRY(dalloc(&d_psums_, nsums));
+      unsigned* tick = nullptr;
+      LS_TRY(dalloc(&tick, (size_t)kSplitItems));
+      cudaError_t e = cudaMemsetAsync(d_psums_, 0, sizeof(unsigned long long) * nsums, s_);
+      if (e == cudaSuccess) e = cudaMemsetAsync(tick, 0, sizeof(unsigned) * kSplitItems, s_);
+      if (e != cudaSuccess) dfree(tick);
+      LS_CUDA(e);
+      d_ptick_ = tick;
     }
     return ASCG_OK;
   }
 
   ascg_status grow_items(int64_t ritems, int64_t gitems) {
-    if (ritems > rcap_items_) {
-      LS_CUDA(cudaStreamSynchronize(s_));
-      dfree(d_ritems_);
-      rcap_items_ = std::max<int64_t>(ritems, 2 * rcap_items_);
-      LS_TRY(dalloc(&d_ritems_, (size_t)rcap_items_));
-    }
-    if (gitems > gcap_items_) {
-      LS_CUDA(cudaStreamSynchronize(s_));
-      dfree(d_gitems_);
-      dfree(d_partials_);
-      gcap_items_ = std::max<int64_t>(gitems, 2 * gcap_items_);
-      LS_TRY(dalloc(&d_gitems_, (size_t)gcap_items_));
-      LS_TRY(dalloc(&d_partials_, (size_t)gcap_items_ * npw_));
-    }
-    return ASCG_OK;
+    LS_TRY(regrow(&d_ritems_, &rcap_items_, ritems));
+    LS_TRY(regrow(&d_gitems_, &gcap_items_, gitems));
+    return regrow(&d_partials_, &parcap_items_, gitems, npw_);
   }
 
   // Row items, Gram items and descriptors of the held lanes, in lane order.
@@ -977,6 +965,7 @@ class Lockstep {
   // copies below (every caller synchronises, or waits for the block's end,
   // before it changes the lanes again).
   ascg_status rebuild_tables() {
+    dirty_ = true;  // until every table is in place: a failed call is repeated by refresh()
     ritems_.clear();
     mitems_.clear();
     gitems_.clear();
@@ -1025,7 +1014,7 @@ class Lockstep {
       for (int64_t r = 0; r < lane_[q].d.n; r += mr)
         mitems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(mr, lane_[q].d.n - r), 0});
     LS_TRY(grow_items((int64_t)ritems_.size(), (int64_t)gitems_.size()));
-    LS_TRY(grow_mitems((int64_t)mitems_.size()));
+    LS_TRY(regrow(&d_mitems_, &mcap_items_, (int64_t)mitems_.size()));
     pieces_ = pieces_of(titems_);
     LS_TRY(grow_titems((int64_t)titems_.size(), (int64_t)pieces_.size()));
     if (!pieces_.empty())
@@ -1084,7 +1073,7 @@ class Lockstep {
   std::vector<GramItem> titems_;
   std::vector<RowItem> mitems_;  // matrix powers items
   bool use_both_ = false;        // of launch_mpk_items_both
-  int64_t rcap_items_ = 0, gcap_items_ = 0, mcap_items_ = 0;
+  int64_t rcap_items_ = 0, gcap_items_ = 0, parcap_items_ = 0, mcap_items_ = 0;
   SysDesc* d_desc_ = nullptr;
   BlockState* d_bst_ = nullptr;
   double* d_G_ = nullptr;
@@ -1343,7 +1332,20 @@ struct ascg_server_s {
       if (pick[gi].empty()) continue;
       Group& g = group[gi];
       std::vector<int> lanes;
-      LS_TRY(g.eng.admit(pick[gi], &lanes));
+      const ascg_status st = g.eng.admit(pick[gi], &lanes);
+      if (st != ASCG_OK) {
+        // a table could not grow: the requests that are not running yet go back to
+        // the head of the queue, and the next step tries again
+        cudaStreamSynchronize(g.stream);  // nothing of theirs is still written
+        g.eng.retire(lanes);
+        for (int gj = kGroups - 1; gj >= gi; --gj)
+          for (auto it = pick[gj].rbegin(); it != pick[gj].rend(); ++it) {
+            arena.give(it->off);
+            queue.push_front(*it);
+            --running;
+          }
+        return st;
+      }
       const double t = now_ms();
       for (int q : lanes) {
         g.eng.lane(q).t_admit = t;
