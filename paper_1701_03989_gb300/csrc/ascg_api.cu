@@ -15,6 +15,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "ascg_common.cuh"
 
 using namespace ascg;
@@ -66,12 +68,14 @@ void dev_free(T*& p) {
 // went to cudaMalloc and cudaFree. A call takes a block (device memory, and a
 // page of pinned host memory) for itself and gives it back after it has
 // synchronised its stream, so a block is never shared between threads or
-// streams. At most kKeepBlocks idle blocks are kept per process; they are
+// streams. Nor between contexts (a program may use several on one device, each
+// with addresses of its own): a block is used, and freed, only in the context it
+// was made in. At most kKeepBlocks idle blocks are kept per process; they are
 // freed when the last operator is destroyed.
 constexpr size_t kScratchBytes = (size_t)1 << 20, kScratchHost = 4096;
 constexpr size_t kKeepBlocks = 4;
 struct ScratchBlock {
-  int dev = -1;
+  unsigned long long ctx = 0;  // its context's id (unique in the process); 0: unknown, not kept
   size_t bytes = 0;
   unsigned char* d = nullptr;
   unsigned char* h = nullptr;
@@ -85,10 +89,50 @@ ScratchPool& scratch_pool() {
   static ScratchPool* p = new ScratchPool();  // never destroyed: calls may outlive static destruction
   return *p;
 }
+// The current context's id, 0 if it cannot be told.
+unsigned long long context_id() {
+  struct Driver {
+    CUresult (*get_current)(CUcontext*) = nullptr;
+    CUresult (*get_id)(CUcontext, unsigned long long*) = nullptr;
+    Driver() {
+      void *a = nullptr, *b = nullptr;
+      cudaDriverEntryPointQueryResult q, r;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+          cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &r) == cudaSuccess &&
+          q == cudaDriverEntryPointSuccess && r == cudaDriverEntryPointSuccess) {
+        get_current = reinterpret_cast<CUresult (*)(CUcontext*)>(a);
+        get_id = reinterpret_cast<CUresult (*)(CUcontext, unsigned long long*)>(b);
+      }
+    }
+  };
+  static const Driver drv;
+  CUcontext c = nullptr;
+  unsigned long long id = 0;
+  if (!drv.get_current || !drv.get_id) return 0;
+  if (drv.get_current(&c) != CUDA_SUCCESS) return 0;
+  // a thread's first call: the runtime has not made the device's context current yet
+  if (!c && (cudaFree(nullptr) != cudaSuccess || drv.get_current(&c) != CUDA_SUCCESS)) return 0;
+  return c && drv.get_id(c, &id) == CUDA_SUCCESS ? id : 0;
+}
 void scratch_free(ScratchBlock& b) {
   if (b.d) cudaFree(b.d);
   if (b.h) cudaFreeHost(b.h);
   b = ScratchBlock();
+}
+// Frees the idle blocks of the current context.
+void scratch_drop_idle() {
+  ScratchPool& p = scratch_pool();
+  const unsigned long long ctx = context_id();
+  std::vector<ScratchBlock> drop;
+  {
+    std::lock_guard<std::mutex> lock(p.mu);
+    for (size_t i = p.idle.size(); i-- > 0;)
+      if (p.idle[i].ctx == ctx) {
+        drop.push_back(p.idle[i]);
+        p.idle.erase(p.idle.begin() + (std::ptrdiff_t)i);
+      }
+  }
+  for (ScratchBlock& b : drop) scratch_free(b);
 }
 void scratch_op_created() {
   ScratchPool& p = scratch_pool();
@@ -97,12 +141,12 @@ void scratch_op_created() {
 }
 void scratch_op_destroyed() {
   ScratchPool& p = scratch_pool();
-  std::vector<ScratchBlock> drop;
+  bool last = false;
   {
     std::lock_guard<std::mutex> lock(p.mu);
-    if (--p.ops == 0) drop.swap(p.idle);
+    last = --p.ops == 0;
   }
-  for (ScratchBlock& b : drop) scratch_free(b);
+  if (last) scratch_drop_idle();
 }
 
 // One call's scratch, carved front to back in 256-byte steps.
@@ -111,7 +155,7 @@ class Scratch {
   ~Scratch() {
     if (!b_.d) return;
     ScratchPool& p = scratch_pool();
-    if (clean_) {
+    if (clean_ && b_.ctx != 0) {
       std::lock_guard<std::mutex> lock(p.mu);
       if (p.idle.size() < kKeepBlocks) {
         p.idle.push_back(b_);
@@ -121,19 +165,18 @@ class Scratch {
     scratch_free(b_);  // waits for the device where the call could not
   }
   ascg_status open(size_t bytes) {
-    int dev = 0;
-    ASCG_CUDA(cudaGetDevice(&dev));
+    const unsigned long long ctx = context_id();
     ScratchPool& p = scratch_pool();
-    {
+    if (ctx != 0) {
       std::lock_guard<std::mutex> lock(p.mu);
       for (size_t i = p.idle.size(); i-- > 0;)
-        if (p.idle[i].dev == dev && p.idle[i].bytes >= bytes) {
+        if (p.idle[i].ctx == ctx && p.idle[i].bytes >= bytes) {
           b_ = p.idle[i];
           p.idle.erase(p.idle.begin() + (std::ptrdiff_t)i);
           return ASCG_OK;
         }
     }
-    b_.dev = dev;
+    b_.ctx = ctx;
     b_.bytes = bytes > kScratchBytes ? bytes : kScratchBytes;
     cudaError_t e = cudaMalloc((void**)&b_.d, b_.bytes);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&b_.h, kScratchHost);
