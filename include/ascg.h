@@ -19,10 +19,13 @@
  *    stream). Calls that report results on the host or use scratch of the
  *    library's (ascg_solve*, ascg_block_step, ascg_newton_shifts,
  *    ascg_matrix_powers, ascg_gram*, ascg_recover_tc; not ascg_gram_noalloc)
- *    synchronise that stream before they return. Scratch blocks (1 MB of
- *    device memory) are kept between calls, at most four idle ones per
- *    process, until the last operator is destroyed. The others return
- *    as soon as their work is enqueued.
+ *    synchronise that stream before they return. The others return as soon
+ *    as their work is enqueued.
+ *  - Device memory kept between calls. Scratch blocks of the single-step calls
+ *    (1 MB and a page of pinned host memory each): at most four idle ones per
+ *    process, until the last operator is destroyed or ascg_trim is called. An
+ *    operator's workspace, which grows with what is called on it: until it is
+ *    destroyed or trimmed.
  *  - Sizes are int64_t. Matrices have n >= 1 rows and nnz < 2^31 nonzeros.
  *  - All arithmetic is IEEE double. eps = 2^-53.
  *  - An ascg_op is not safe for concurrent use from several threads or
@@ -207,6 +210,11 @@ ascg_status ascg_op_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr,
 /* Frees the operator and its workspace. NULL is accepted. */
 ascg_status ascg_op_destroy(ascg_op op);
 
+/* Frees what is kept for later calls: op's workspace (op may be NULL; no call
+ * on it may be running), and the idle scratch blocks of the current context.
+ * The next calls allocate again. */
+ascg_status ascg_trim(ascg_op op);
+
 /* n and nnz of the operator (host out-pointers may be NULL). */
 ascg_status ascg_op_size(ascg_op op, int64_t* n, int64_t* nnz);
 
@@ -285,7 +293,10 @@ ascg_status ascg_spmv(ascg_op op, const double* x, double* y, void* cuda_stream)
  * two distinct gamma values other than 1). 1 <= s <= 16. The coefficients are
  * folded into the operator first ((D - theta_j)/gamma_j and O/gamma_j for
  * A = D + O), exactly as ascg_solve does, so this call runs the solver's own
- * kernel. */
+ * kernel. The folded operator stays in op's workspace (until ascg_op_destroy
+ * or ascg_trim): 8 n bytes per distinct (theta, gamma) other than (0, 1), at
+ * most 8 n s, and a copy of O's values (8 bytes per entry, each slice of 32
+ * rows padded to its longest) per distinct gamma other than 1, at most two. */
 ascg_status ascg_matrix_powers(ascg_op op, int s, const double* theta, const double* sigma,
                                const double* gamma, double* Y, int64_t ldY, void* cuda_stream);
 

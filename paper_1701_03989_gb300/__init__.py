@@ -94,6 +94,7 @@ def _load():
         "ascg_options_default": (C.c_int, [C.POINTER(ascg_options)]),
         "ascg_op_create_csr": (C.c_int, [I64, I64, P, P, P, C.c_int, C.POINTER(P)]),
         "ascg_op_destroy": (C.c_int, [P]),
+        "ascg_trim": (C.c_int, [P]),
         "ascg_op_size": (C.c_int, [P, C.POINTER(I64), C.POINTER(I64)]),
         "ascg_solve": (C.c_int, [P, P, P, C.POINTER(ascg_options), C.POINTER(ascg_result), P]),
         "ascg_solve_host": (C.c_int, [P, P, P, C.POINTER(ascg_options), C.POINTER(ascg_result), P]),
@@ -184,6 +185,11 @@ def ascg_op_create_csr(n, nnz, rowptr, colind, val, on_device=0):
 
 def ascg_op_destroy(op):
     _check(_lib.ascg_op_destroy(op), "ascg_op_destroy")
+
+
+def ascg_trim(op=None):
+    """Frees what is kept for later calls: op's workspace and the idle scratch blocks."""
+    _check(_lib.ascg_trim(op), "ascg_trim")
 
 
 def ascg_op_size(op):
@@ -412,7 +418,7 @@ def block_infos(count: int):
     return (ascg_block_info * count)()
 
 
-EXPORTED = ["ascg_options_default", "ascg_op_create_csr", "ascg_op_destroy", "ascg_op_size", "ascg_solve",
+EXPORTED = ["ascg_options_default", "ascg_op_create_csr", "ascg_op_destroy", "ascg_trim", "ascg_op_size", "ascg_solve",
             "ascg_solve_host", "ascg_solve_batch", "ascg_spmv", "ascg_matrix_powers", "ascg_gram", "ascg_gram_noalloc", "ascg_gram_moments",
             "ascg_block_step", "ascg_recover", "ascg_recover_tc",
             "ascg_newton_shifts", "ascg_server_create", "ascg_server_submit", "ascg_server_step",

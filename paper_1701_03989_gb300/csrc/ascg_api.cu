@@ -71,7 +71,8 @@ void dev_free(T*& p) {
 // streams. Nor between contexts (a program may use several on one device, each
 // with addresses of its own): a block is used, and freed, only in the context it
 // was made in. At most kKeepBlocks idle blocks are kept per process; they are
-// freed when the last operator is destroyed.
+// freed when the last operator is destroyed, and by ascg_trim: a program without
+// operators has no other way to have them back.
 constexpr size_t kScratchBytes = (size_t)1 << 20, kScratchHost = 4096;
 constexpr size_t kKeepBlocks = 4;
 struct ScratchBlock {
@@ -1140,6 +1141,13 @@ ascg_status ascg_op_destroy(ascg_op op) {
   op->free_device();
   delete op;
   scratch_op_destroyed();
+  return ASCG_OK;
+}
+
+ascg_status ascg_trim(ascg_op op) {
+  g_err.clear();
+  if (op) op->ws.release();
+  scratch_drop_idle();
   return ASCG_OK;
 }
 

@@ -1,8 +1,7 @@
-"""Scratch blocks kept between single-step calls: contexts, threads, and what gives them back."""
+"""Scratch blocks kept between single-step calls: contexts, and what gives them back."""
 import os
 import subprocess
 import sys
-import threading
 
 import numpy as np
 import pytest
@@ -44,3 +43,60 @@ print("ok")
 def test_blocks_stay_in_their_context():
     r = subprocess.run([sys.executable, "-c", TWO_CONTEXTS % ROOT], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
+
+
+# A program that never creates an operator: what its calls keep comes back by ascg_trim, and they go on working.
+NO_OPERATOR = r"""
+import sys
+import torch
+sys.path.insert(0, %r)
+import paper_1701_03989_gb300 as P
+Y = torch.rand((5, 2048), dtype=torch.float64, device="cuda")
+G = torch.empty((5, 5), dtype=torch.float64, device="cuda")
+def gram():
+    P.ascg_gram(2048, 5, Y, 2048, G)
+    return G.cpu()  # compared on the host: torch's own kernels would load, and take device memory, on first use
+first = gram()
+P.ascg_trim()
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+for _ in range(3):
+    assert torch.equal(gram(), first)
+    P.ascg_trim()
+assert torch.cuda.mem_get_info()[0] == free
+print("ok")
+"""
+
+
+def test_trim_without_an_operator():
+    r = subprocess.run([sys.executable, "-c", NO_OPERATOR % ROOT], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
+
+
+def test_trim_gives_an_operators_workspace_back():
+    """Matrix powers keep at most the folded operator that the header states; trimming gives it back and changes no bit."""
+    import paper_1701_03989_gb300 as P
+
+    n, s = 1 << 20, 16  # tridiagonal: O has two entries a row
+    cols = np.arange(n)[:, None] + np.array([-1, 0, 1])[None, :]
+    keep = (cols >= 0) & (cols < n)
+    vals = np.broadcast_to(np.array([-1.0, 4.0, -1.0]), (n, 3))
+    rowptr = np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int64)
+    op = P.ascg_op_create_csr(n, int(rowptr[-1]), rowptr, cols[keep].astype(np.int32), vals[keep], 0)
+    th, sg, gm = np.linspace(0.5, 3.5, s), np.full(s, 0.25), np.array([1.0] + [0.5] * (s - 1))
+    Y = torch.zeros((2 * s + 1, n), dtype=torch.float64, device="cuda")
+    Y[:2] = torch.rand((2, n), dtype=torch.float64, device="cuda")
+    P.ascg_matrix_powers(op, s, th, sg, gm, Y, n)
+    want = Y.cpu()
+    torch.cuda.synchronize()
+    P.ascg_trim(op)
+    free = torch.cuda.mem_get_info()[0]
+    P.ascg_matrix_powers(op, s, th, sg, gm, Y, n)
+    kept = free - torch.cuda.mem_get_info()[0]
+    assert 0 < kept <= 8 * n * s + 8 * 2 * n + (4 << 20)  # one gamma other than 1; allocations come in 2 MB
+    assert torch.equal(Y.cpu(), want)
+    P.ascg_trim(op)
+    assert torch.cuda.mem_get_info()[0] == free
+    b, x = torch.rand(n, dtype=torch.float64, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda")
+    assert P.ascg_solve(op, b, x, P.make_options(s_max=4)).status == P.ASCG_OK
+    P.ascg_op_destroy(op)
