@@ -1,7 +1,8 @@
-"""Scratch blocks kept between single-step calls: contexts, and what gives them back."""
+"""Scratch blocks kept between single-step calls: contexts, threads, and what gives them back."""
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -100,3 +101,59 @@ def test_trim_gives_an_operators_workspace_back():
     b, x = torch.rand(n, dtype=torch.float64, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda")
     assert P.ascg_solve(op, b, x, P.make_options(s_max=4)).status == P.ASCG_OK
     P.ascg_op_destroy(op)
+
+
+def test_mixed_calls_from_threads():
+    """Calls that stage through the pinned page, on a stream each: every one of them runs, with the bits it has alone."""
+    import paper_1701_03989_gb300 as P
+
+    n, w, s = 4096, 17, 8
+    g = torch.Generator(device="cuda").manual_seed(1)
+    Y = torch.rand((w, n), dtype=torch.float64, device="cuda", generator=g) - 0.5
+    G0 = (Y @ Y.T).contiguous()
+    coords = torch.rand(3 * w, dtype=torch.float64, device="cuda", generator=g)
+    rng = np.random.default_rng(2)
+
+    def gram(k, st):
+        G = torch.empty((w, w), dtype=torch.float64, device="cuda")
+        P.ascg_gram(n, w, Y, n, G, stream=st)
+        return G.cpu().numpy()
+
+    def block(k, st):
+        c = torch.zeros(3 * w, dtype=torch.float64, device="cuda")
+        info, hist = P.ascg_block_step(s, G0, P.ASCG_ADAPTIVE, np.full(s, 0.1 * k), np.zeros(s), np.ones(s), n, 1e-9, 1.0,
+                                       1, 100, 1.0, c, stream=st)
+        return np.concatenate([np.array(info.sqrt_kappa), hist.ravel(), c.cpu().numpy()])
+
+    al, be = rng.uniform(0.3, 3.0, (8, 16)), rng.uniform(0.01, 1.5, (8, 15))
+
+    def shifts(k, st):
+        return P.ascg_newton_shifts(al[k], be[k], 16, 16, stream=st)
+
+    def recover(k, st):
+        v = torch.zeros((3, n), dtype=torch.float64, device="cuda")
+        P.ascg_recover_tc(n, w, Y, n, coords, v[0], v[1], v[2], stream=st)
+        return v.cpu().numpy()
+
+    calls = [gram, block, shifts, recover]
+    alone = {(f, k): f(k, None) for f in calls for k in range(8)}
+    done, errors = [0] * 8, []
+
+    def work(k):
+        try:
+            st = torch.cuda.Stream()
+            with torch.cuda.stream(st):
+                for i in range(40):
+                    f = calls[(k + i) % 4]
+                    assert np.array_equal(f(k, st), alone[f, k]), (f, k)
+                    done[k] += 1
+        except BaseException as e:  # a thread's failure is the test's
+            errors.append((k, repr(e)))
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors and done == [40] * 8
