@@ -386,9 +386,9 @@ struct GramPiece {
 cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t rows, const GramPiece* pieces,
                                  int npieces, const int* sys_w, const int* emax_all, double* partials,
                                  unsigned long long* sums, unsigned* tickets, cudaStream_t s);
-// The column exponents of every piece's system (emax_all zeroed here), by a pass over Y.
+// The column exponents of the pieces' systems (emax_all zeroed before), by a pass over their rows of Y.
 cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramPiece* pieces, int npieces,
-                                      const int* sys_w, int nsys, int* emax_all, cudaStream_t s);
+                                      const int* sys_w, int* emax_all, cudaStream_t s);
 // Recovery (eq. coords) on the tensor cores: x += Y x', r = Y r', p = Y p' in
 // one pass, with the Gram's digit split of Y (col_emax: the Gram's column
 // exponents, device int[kMaxW]) and coefficients (coords: device double[3w],
@@ -425,20 +425,21 @@ struct RowItem {
   int sys;
   int row0;
   int nrows;
-  int pad_;
+  int by_chain;  // matrix powers: kMpkChainRows rows, a warp per slice and chain
 };
 // Copies of a system's column exponents (kMaxW ints each) that its CTAs spread
 // their maxima over: atomics on one address take about 1 ns each, and with one
 // copy and one per warp a 140^3 system's steps took 41 ms instead of 28.
 constexpr int kEmaxCopies = 8;
-// Rows of a matrix powers item with a warp per chain.
-constexpr int kMpkChainRows = 64;
-// Matrix powers step j (monomial basis) of every system q with j < sys_steps[q].
-// items: kMpkChainRows rows each, a warp per chain. emax_all (nsys x kEmaxCopies x kMaxW ints, zeroed before
-// step 0, or nullptr): the largest biased exponent of every column formed, and
-// of columns 0 and 1, is the maximum over the system's copies.
+// Rows of a matrix powers item with a warp per chain, and of one with both chains
+// in a thread in the same launch.
+constexpr int kMpkChainRows = 64, kMpkMixedRows = 128;
+// Matrix powers step j (monomial basis) of every system q with j < sys_steps[q]. items: by chain (kMpkChainRows
+// rows each) and, if mixed, also with both chains in a thread (kMpkMixedRows). emax_all (nsys x kEmaxCopies x kMaxW
+// ints, zeroed before step 0, or nullptr): of the systems by chain, the largest biased exponent of every column formed,
+// and of columns 0 and 1, is the maximum over the system's copies.
 cudaError_t launch_mpk_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
-                             int* emax_all, cudaStream_t s);
+                             bool mixed, int* emax_all, cudaStream_t s);
 // The same with kRowItem rows per item and both chains in a thread, without exponents.
 cudaError_t launch_mpk_items_both(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
                                   cudaStream_t s);

@@ -22,37 +22,39 @@ __device__ __forceinline__ bool item_row(const RowItem* items, int64_t* row, int
 // eq. (polybasiscg)) for every system q with j < sys_steps[q]: column 2j+2 =
 // A column 2j and, while j + 1 < sbar_q, column 2j+3 = A column 2j+1, A = D + O.
 //
-// Two kernels. mpk_items_kernel: one warp per 32-row
-// slice and chain (P or R), an item of 64 rows per CTA of 128 threads; the
-// second warp of a slice finds A in L1. A row's sum is one chain of dependent
-// FMAs, 64 cycles each on GB300, so a long row costs its length in latency
-// however idle the GPU is: the two chains on two warps halve that, and small
-// CTAs spread a small system over more SMs. row_chain keeps two groups of A and
-// one of gathers in flight. 8 CTAs per SM (64 registers) beat 7 (72) by 4 % and
-// 10 (48, spilling) by 18 %. FP64-bound: 1.71M warp FMAs (10 systems, two banded
-// of 117 and 129 entries a row) take 111 us, 0.79 of the FP64 pipe. 32 systems of
-// 1e3..1e5 rows, targets 1e-8 and 1e-12: 236.4 -> 195.1 ms a batch with the
-// exponents folded in below (one thread per row with both chains in 256-row
-// CTAs, and a pass over the bases for the exponents before).
-// It records the largest biased exponent of the columns written (and, at step 0,
-// of the input columns) for the tensor-core Gram, in place of another pass over
-// the basis: one atomic without return per warp, into one of the system's
-// kEmaxCopies copies.
+// Two ways of summing a row, chosen per system (items_by_chain). By chain: one
+// warp per 32-row slice and chain (P or R), an item of 64 rows per CTA of 128
+// threads; the second warp of a slice finds A in L1. A row's sum is one chain of
+// dependent FMAs, 64 cycles each on GB300, so a long row costs its length in
+// latency however idle the GPU is: the two chains on two warps halve that, and
+// small CTAs spread a small system over more SMs. row_chain keeps two groups of A
+// and one of gathers in flight. 8 CTAs per SM (64 registers) beat 7 (72) by 4 %
+// and 10 (48, spilling) by 18 %. FP64-bound: 1.71M warp FMAs (10 systems, two
+// banded of 117 and 129 entries a row) take 111 us, 0.79 of the FP64 pipe at its
+// nominal rate. 32 systems of 1e3..1e5 rows, targets 1e-8 and 1e-12: 236.4 -> 195.1
+// ms a batch with the exponents folded in below (one thread per row with both
+// chains in 256-row CTAs, and a pass over the bases for the exponents before).
+// Such an item records the largest biased exponent of the columns written (and,
+// at step 0, of the input columns) for the tensor-core Gram, in place of another
+// pass over the basis: one atomic without return per warp, into one of the
+// system's kEmaxCopies copies.
 //
-// mpk_items_both_kernel: 256 rows, both chains in one thread, for batches with so
-// many rows that the GPU is full anyway (Lockstep::rebuild_tables): A is read
-// once, the items stay in system order, which mixes FP64-bound long rows with
-// HBM-bound short ones, and the exponents take a pass of their own (recording
-// them here, even once per CTA, was slower: 140^3, 60 iterations, 29.7 ms
-// against 27.8).
+// Both chains in a thread: A and its indices are read once, for short rows in
+// batches that fill the GPU, where the doubled loads are what counts. The
+// exponents of such systems take a pass of their own (recording them here, even
+// once per CTA, was slower: 140^3, 60 iterations, 29.7 ms against 27.8). In a
+// batch that has both kinds (MIXED) such an item is 128 rows of the same kernel;
+// a batch that has no other takes mpk_items_both_kernel, 256 rows.
+template <bool MIXED>
 __global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __restrict__ descs,
                                                            const RowItem* __restrict__ items,
                                                            const int* __restrict__ sys_steps, int j,
                                                            int* __restrict__ emax_all) {
   const RowItem it = items[blockIdx.x];
   const SysDesc d = descs[it.sys];
+  const bool chain = !MIXED || it.by_chain;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ch = warp & 1, first = kSlice * (warp >> 1);
+  const int ch = chain ? warp & 1 : 0, first = kSlice * (chain ? warp >> 1 : warp);
   const bool any = first < it.nrows, on = first + lane < it.nrows;
   const int64_t row = (int64_t)it.row0 + first + lane;
   int64_t b = 0;
@@ -69,10 +71,25 @@ __global__ void __launch_bounds__(128, 8) mpk_items_kernel(const SysDesc* __rest
   pdl_release();
   const int steps = load_after_wait(sys_steps + it.sys);
   if (!any || j + ch >= steps) return;  // uniform over the warp: no step j, or no R chain in the last one
+  const double* v = d.o_val + b + lane;
+  const int32_t* c = d.o_col + b + lane;
   const double xi = on ? x[row] : 0.0;
-  const double t = row_chain(d.o_val + b + lane, d.o_col + b + lane, width, x, dg * xi);
+  double t = dg * xi;
+  if (MIXED && !chain && j + 1 < steps) {
+    const double* r = x + d.ldY;
+    double tr = dg * (on ? r[row] : 0.0);
+    for (int k = 0; k < width; ++k) {
+      const double a = __ldg(v + kSlice * k);
+      const int cc = __ldg(c + kSlice * k);
+      t = fma(a, __ldca(x + cc), t);
+      tr = fma(a, __ldca(r + cc), tr);
+    }
+    if (on) d.Y[(int64_t)(2 * j + 3) * d.ldY + row] = tr;
+  } else {
+    t = row_chain(v, c, width, x, t);
+  }
   if (on) d.Y[(int64_t)(2 * j + 2 + ch) * d.ldY + row] = t;
-  if (!emax_all) return;
+  if (!emax_all || !chain) return;
   int* em = emax_all + ((int64_t)it.sys * kEmaxCopies + (blockIdx.x & (kEmaxCopies - 1))) * kMaxW + ch;
   const unsigned e = __reduce_max_sync(0xffffffffu, on ? biased_exp(t) : 0u);
   if (lane == 0) atomicMax(em + 2 * j + 2, (int)e);
@@ -222,9 +239,10 @@ cudaError_t launch_fill_uniform(double* v, int64_t count, uint64_t seed, cudaStr
 }
 
 cudaError_t launch_mpk_items(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,
-                             int* emax_all, cudaStream_t s) {
+                             bool mixed, int* emax_all, cudaStream_t s) {
   if (nitems < 1) return cudaSuccess;
-  return launch_pdl(mpk_items_kernel, nitems, 128, s, descs, items, sys_steps, j, emax_all);
+  if (mixed) return launch_pdl(mpk_items_kernel<true>, nitems, 128, s, descs, items, sys_steps, j, emax_all);
+  return launch_pdl(mpk_items_kernel<false>, nitems, 128, s, descs, items, sys_steps, j, emax_all);
 }
 
 cudaError_t launch_mpk_items_both(const SysDesc* descs, const RowItem* items, int nitems, const int* sys_steps, int j,

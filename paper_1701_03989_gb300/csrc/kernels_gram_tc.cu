@@ -1320,10 +1320,8 @@ cudaError_t launch_gram_tc_items(int w, const double* Y, int64_t ldY, int64_t ro
 }
 
 cudaError_t launch_tc_items_exponents(int w, const double* Y, int64_t ldY, const GramPiece* pieces, int npieces,
-                                      const int* sys_w, int nsys, int* emax_all, cudaStream_t s) {
+                                      const int* sys_w, int* emax_all, cudaStream_t s) {
   if (npieces < 1) return cudaSuccess;
-  const cudaError_t e = cudaMemsetAsync(emax_all, 0, sizeof(int) * kTW * kEmaxCopies * nsys, s);
-  if (e != cudaSuccess) return e;
   tc_items_exponent_kernel<<<npieces, 256, 0, s>>>(w, Y, ldY, pieces, sys_w, emax_all);
   return cudaGetLastError();
 }

@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "ascg_common.cuh"
+#include "dispatch.cuh"
 
 namespace ascg {
 
@@ -620,16 +621,19 @@ class Lockstep {
     int* d_tcn = d_int_ + kTcNItems * lanes_;
     const int nr = (int)ritems_.size(), ng = (int)gitems_.size(), nm = (int)mitems_.size();
     const int Wb = 2 * max_sbar + 1;
-    if (use_both_) {
-      for (int j = 0; j < max_sbar; ++j) LS_CUDA(launch_mpk_items_both(d_desc_, d_mitems_, nm, d_steps, j, s_));
-      if (tc_gram)
-        LS_CUDA(launch_tc_items_exponents(Wb, ybase_, yld_, d_pieces_, (int)pieces_.size(), d_wtc, hi_, d_emax_, s_));
-    } else {
-      // the steps record the column exponents that the tensor-core Gram needs
-      if (tc_gram) LS_CUDA(cudaMemsetAsync(d_emax_, 0, sizeof(int) * kEmaxCopies * kMaxW * hi_, s_));
-      for (int j = 0; j < max_sbar; ++j)
-        LS_CUDA(launch_mpk_items(d_desc_, d_mitems_, nm, d_steps, j, tc_gram ? d_emax_ : nullptr, s_));
+    // the steps by chain record the column exponents that the tensor-core Gram
+    // needs; those of the other systems take a pass over their rows
+    if (tc_gram) LS_CUDA(cudaMemsetAsync(d_emax_, 0, sizeof(int) * kEmaxCopies * kMaxW * hi_, s_));
+    for (int j = 0; j < max_sbar; ++j) {
+      if (chain_lanes_ == 0)
+        LS_CUDA(launch_mpk_items_both(d_desc_, d_mitems_, nm, d_steps, j, s_));
+      else
+        LS_CUDA(launch_mpk_items(d_desc_, d_mitems_, nm, d_steps, j, chain_lanes_ < nused_, tc_gram ? d_emax_ : nullptr,
+                                 s_));
     }
+    if (tc_gram)
+      LS_CUDA(launch_tc_items_exponents(Wb, ybase_, yld_, d_pieces_ + chain_pieces_,
+                                        (int)pieces_.size() - chain_pieces_, d_wtc, d_emax_, s_));
     if (item_gram) {
       // pair groups: enough CTAs to cover the SMs twice
       const int groups = std::max(1, std::min(16, (2 * gram_grid() + ng - 1) / std::max(ng, 1)));
@@ -991,31 +995,40 @@ class Lockstep {
       for (int64_t r = 0; r < n; r += gr) gitems_.push_back(GramItem{r, (int)std::min<int64_t>(gr, n - r), q});
       h_nitems[q] = (int)gitems_.size() - h_item0[q];
     }
-    int64_t rows_all = 0;
+    BatchRows rows;
     std::vector<int> order;
     for (int q = 0; q < hi_; ++q) {
       if (!used_[q]) continue;
       order.push_back(q);
-      rows_all += lane_[q].d.n;
+      rows.rows += lane_[q].d.n;
+      rows.mean_len += lane_[q].row_len * (double)lane_[q].d.n;
+      rows.max_len = std::max(rows.max_len, lane_[q].row_len);
       for (int64_t r = 0; r < lane_[q].d.n; r += kRowItem)
         ritems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(kRowItem, lane_[q].d.n - r), 0});
     }
-    // Matrix powers items: from kBothRows rows in all, 256 rows with both chains in
-    // a thread, in system order; below, where latency counts, 64 rows with a warp
-    // per chain, the longest rows first (an item's time is its rows' length, so
-    // the last CTAs of a launch are the short ones). By chain / both in a thread:
-    // 0.69M rows in 32 systems 182 / 236 ms, 11.3M rows in 256 systems 3.74 / 3.42
-    // s, 2.7M rows of one 140^3 system 41 / 28 ms.
-    use_both_ = rows_all >= kBothRows;
-    if (!use_both_)
+    if (rows.rows > 0) rows.mean_len /= (double)rows.rows;
+    // Matrix powers items (items_by_chain says how each system's rows are summed).
+    // With items by chain the longest rows go first (an item's time is its rows'
+    // length, so the last CTAs of a launch are the short ones).
+    std::vector<char> chain(hi_, 0);
+    chain_lanes_ = 0;
+    for (int q : order) {
+      chain[q] = items_by_chain(rows, lane_[q].row_len);
+      chain_lanes_ += chain[q];
+    }
+    if (chain_lanes_ > 0)
       std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return lane_[a].row_len > lane_[b].row_len; });
-    const int64_t mr = use_both_ ? kRowItem : kMpkChainRows;
-    for (int q : order)
+    const int64_t both_rows = chain_lanes_ == 0 ? kRowItem : kMpkMixedRows;
+    for (int q : order) {
+      const int64_t mr = chain[q] ? kMpkChainRows : both_rows;
       for (int64_t r = 0; r < lane_[q].d.n; r += mr)
-        mitems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(mr, lane_[q].d.n - r), 0});
+        mitems_.push_back(RowItem{q, (int)r, (int)std::min<int64_t>(mr, lane_[q].d.n - r), chain[q]});
+    }
     LS_TRY(grow_items((int64_t)ritems_.size(), (int64_t)gitems_.size()));
     LS_TRY(regrow(&d_mitems_, &mcap_items_, (int64_t)mitems_.size()));
-    pieces_ = pieces_of(titems_);
+    pieces_ = pieces_of(titems_);  // those of the systems by chain first
+    chain_pieces_ = (int)(std::stable_partition(pieces_.begin(), pieces_.end(),
+                                                [&](const GramPiece& p) { return chain[p.sys] != 0; }) - pieces_.begin());
     LS_TRY(grow_titems((int64_t)titems_.size(), (int64_t)pieces_.size()));
     if (!pieces_.empty())
       LS_CUDA(cudaMemcpyAsync(d_pieces_, pieces_.data(), sizeof(GramPiece) * pieces_.size(), cudaMemcpyHostToDevice,
@@ -1039,7 +1052,6 @@ class Lockstep {
     return ASCG_OK;
   }
 
-  static constexpr int64_t kBothRows = (int64_t)1 << 20;
   static constexpr size_t kMaxGraphs = 64;
   void drop_graphs() {
     for (auto& kv : graphs_) cudaGraphExecDestroy(kv.second);
@@ -1072,7 +1084,8 @@ class Lockstep {
   std::vector<GramItem> gitems_;
   std::vector<GramItem> titems_;
   std::vector<RowItem> mitems_;  // matrix powers items
-  bool use_both_ = false;        // of launch_mpk_items_both
+  int chain_lanes_ = 0;          // held lanes whose matrix powers items are by chain
+  int chain_pieces_ = 0;         // their Gram pieces, the first of pieces_
   int64_t rcap_items_ = 0, gcap_items_ = 0, parcap_items_ = 0, mcap_items_ = 0;
   SysDesc* d_desc_ = nullptr;
   BlockState* d_bst_ = nullptr;
@@ -1598,7 +1611,8 @@ ascg_status ascg_tune_gram_schedule(int s_max, int64_t* tc_lane_rows, double* ta
     LS_CUDA(cudaMemcpyAsync(B.pieces, pieces.data(), sizeof(GramPiece) * pieces.size(), cudaMemcpyHostToDevice, s));
     LS_CUDA(cudaMemcpyAsync(B.ints, ints, sizeof(ints), cudaMemcpyHostToDevice, s));
     // a solve's exponents come from its matrix powers steps: not timed
-    LS_CUDA(launch_tc_items_exponents(w, B.Y, ld, B.pieces, (int)pieces.size(), B.ints, 1, B.emax, s));
+    LS_CUDA(cudaMemsetAsync(B.emax, 0, sizeof(int) * kEmaxCopies * kMaxW, s));
+    LS_CUDA(launch_tc_items_exponents(w, B.Y, ld, B.pieces, (int)pieces.size(), B.ints, B.emax, s));
     LS_CUDA(cudaStreamSynchronize(s));  // the host arrays above are locals
     const int groups = std::max(1, std::min(16, (2 * gram_grid() + ng - 1) / ng));
     std::vector<float> a(kReps), b(kReps);

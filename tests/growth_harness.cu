@@ -90,7 +90,7 @@ bool gram_tc_aligned(const double*, int64_t) { return true; }
 // every table a launch is given has to be there
 int missing = 0;
 void want(const void* p) { missing += p == nullptr; }
-cudaError_t launch_mpk_items(const SysDesc* a, const RowItem* b, int, const int* c, int, int*, cudaStream_t) {
+cudaError_t launch_mpk_items(const SysDesc* a, const RowItem* b, int, const int* c, int, bool, int*, cudaStream_t) {
   want(a), want(b), want(c);
   return cudaSuccess;
 }
@@ -98,7 +98,7 @@ cudaError_t launch_mpk_items_both(const SysDesc* a, const RowItem* b, int, const
   want(a), want(b), want(c);
   return cudaSuccess;
 }
-cudaError_t launch_tc_items_exponents(int, const double*, int64_t, const GramPiece* a, int, const int*, int, int*,
+cudaError_t launch_tc_items_exponents(int, const double*, int64_t, const GramPiece* a, int, const int*, int*,
                                       cudaStream_t) {
   want(a);
   return cudaSuccess;
