@@ -40,4 +40,28 @@ inline bool items_by_chain(const BatchRows& b, double row_len) {
   return row_len >= 40.0 || b.rows < 196608 || (row_len >= 7.0 && b.rows <= 400000);
 }
 
+// Whether classical CG's product sums its rows with pipelined loads (row_chain) or
+// an entry at a time, with A kept in L2 up to 32 MiB of values and columns and
+// streamed past it above. Pipelined hides the gathers' latency but holds four CTAs
+// of 256 rows per SM, and keeps A in L2. us for 60 iterations, an entry at a time /
+// pipelined, by rows and entries a row:
+//   20000   13 1206 / 1166, 81 1859 / 1497     40000   13 1266 / 1268, 81 2759 / 1859
+//   70000   13 1351 / 1395, 49 2217 / 1666     90000   21 1484 / 1530, 33 1870 / 1666
+//   100000  33 1951 / 1845, 201 7164 / 4924    110000  21 1486 / 1837, 61 2407 / 2619
+//   116000  61 2872 / 2583                     130000  21 1660 / 1879, 81 3868 / 3067
+//   150000  33 2000 / 2122, 49 2634 / 2468     160000  21 2449 / 1995, 81 4353 / 4093
+//   175000  49 3613 / 3189, 61 3794 / 3850     200000  33 3270 / 2756, 49 3451 / 3693
+//   230000  33 3242 / 2844, 49 3519 / 3746     262144  21 2665 / 2482, 33 2929 / 3159
+// Up to 50000 rows latency is all. To four CTAs per SM (155648 rows) an entry at a
+// time is better where A stays in L2, also streamed up to 80 MiB once there are
+// more than 102400 rows. Beyond, pipelined is better as long as A, which it reads
+// from L2, and what the iteration streams through it fit in its 129 MB.
+inline bool cg_rows_pipelined(int64_t n, int64_t nnz) {
+  if (nnz < 12 * n || n > 262144) return false;
+  const int64_t a = 12 * nnz, mib = (int64_t)1 << 20;
+  if (n <= 50000) return true;
+  if (n <= 155648) return a > 32 * mib && (n <= 102400 || a >= 80 * mib);
+  return a + 128 * n <= 128000000 || (n <= 163840 && a >= 80 * mib);
+}
+
 }  // namespace ascg

@@ -9,6 +9,7 @@
 // to finish (by an atomic ticket) adds the partials in index order. There are
 // no spin-waits.
 #include "ascg_common.cuh"
+#include "dispatch.cuh"
 
 namespace ascg {
 
@@ -265,10 +266,7 @@ cudaError_t launch_dot(const double* u, const double* v, int64_t n, double* out,
 cudaError_t launch_cg_spmv_dot(const DevSell& A, int64_t nnz, const double* p, double* q, CGState* st,
                                double* partials, unsigned* counter, cudaStream_t s) {
   const int g = grid_for(A.n, kSpmvRows, 152 * 8);
-  // long rows: us per iteration, an entry at a time / pipelined: n = 20011 of 13
-  // entries a row 14.0 / 13.5, of 81 25.1 / 18.8, n = 100003 of 33 27.5 / 25.4,
-  // n = 300007 of 81 (streamed past L2) 73.6 / 75.9
-  if (nnz >= 12 * A.n && A.n <= 262144)
+  if (cg_rows_pipelined(A.n, nnz))
     return launch_pdl(cg_spmv_dot_kernel<kChain>, g, kSpmvRows, s, A, p, q, st, partials, counter);
   // A's values and columns (12 bytes per entry) beyond a quarter of the 129 MB
   // L2: stream them past it

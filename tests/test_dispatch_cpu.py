@@ -36,3 +36,16 @@ def test_items_by_chain(tmp_path, systems, want):
         body += "b.rows += %d; b.mean_len += %r * %d; b.max_len = b.max_len > %r ? b.max_len : %r;\n" % (n, l, n, l, l)
     body += "b.mean_len /= (double)b.rows;\n" + "".join('std::printf("%%d ", (int)items_by_chain(b, %r));\n' % l for _, l in systems)
     assert "".join(_run(tmp_path, body)) == want
+
+
+# classical CG: rows, entries a row, pipelined row sums?
+CG_ROWS = [(20000, 13, 1), (20000, 81, 1), (50000, 49, 1), (20000, 5, 0), (70000, 13, 0), (70000, 49, 1), (80000, 21, 0), (90000, 33, 1),
+           (100000, 13, 0), (100000, 49, 1), (110000, 13, 0), (110000, 21, 0), (110000, 61, 0), (116000, 61, 1), (130000, 21, 0),
+           (130000, 81, 1), (150000, 13, 0), (150000, 33, 0), (150000, 49, 1), (160000, 13, 1), (160000, 81, 1), (175000, 49, 1),
+           (190000, 33, 1), (190000, 61, 0), (200000, 49, 0), (200000, 201, 0), (230000, 33, 1), (262144, 21, 1), (262144, 33, 0),
+           (262144, 201, 0), (300000, 21, 0), (600000, 81, 0)]
+
+
+def test_cg_rows_pipelined(tmp_path):
+    got = _run(tmp_path, "".join('std::printf("%%d ", (int)cg_rows_pipelined(%d, %d));\n' % (n, n * k) for n, k, _ in CG_ROWS))
+    assert [int(v) for v in got] == [w for _, _, w in CG_ROWS]
