@@ -555,7 +555,8 @@ class Lockstep {
     const bool item_gram = n_tc < count_active();
     const bool tc_gram = n_tc > 0;
     const int Wb = 2 * max_sbar + 1;
-    int nl = max_sbar + 2 + (item_gram ? 2 : 0) + (tc_gram ? 2 : 0);
+    // the exponent pass of the systems that are not summed by chain is a launch too
+    int nl = max_sbar + 2 + (item_gram ? 2 : 0) + (tc_gram ? (chain_pieces_ < (int)pieces_.size() ? 3 : 2) : 0);
     // The block's work: the state records in, the matrix powers steps, the
     // Gram (item launch and tensor-core lanes), the controller, the recovery,
     // the state records out. The host fills the pinned records before each

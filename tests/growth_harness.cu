@@ -1,7 +1,11 @@
-// Host-only run of the solve server's admission with a fake CUDA runtime: device
-// memory is host memory, launches do nothing, and the k-th allocation after the
-// server's creation fails. Prints one line per k: what the failed step left behind
-// and how the retry ended. Compiled and read by tests/test_growth_cpu.py.
+// Host-only run of the lockstep engine with a fake CUDA runtime: device memory is
+// host memory and launches are only counted. Compiled and read by
+// tests/test_growth_cpu.py.
+//   growth   the k-th allocation after the server's creation fails; one line per k:
+//            what the failed step left behind and how the retry ended
+//   count    the launches that ascg_server_info reports, and those made, for a server
+//            with one system of each size
+//   tune     the exponent passes and tensor-core Grams that the autotuner makes, by rows
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -60,6 +64,8 @@ cudaError_t copy(void* d, const void* s, size_t n) {
 #define cudaStreamWaitEvent(...) fake::ok()
 #define cudaStreamBeginCapture(s, m) cudaErrorNotSupported
 #define cudaEventCreateWithFlags(p, f) (*(p) = nullptr, cudaSuccess)
+#define cudaEventCreate(p) (*(p) = nullptr, fake::ok())
+#define cudaEventElapsedTime(p, a, b) (*(p) = 1.0f, fake::ok())
 #define cudaEventRecord(...) fake::ok()
 #define cudaEventQuery(e) fake::ok()
 #define cudaEventSynchronize(e) fake::ok()
@@ -89,32 +95,41 @@ bool gram_tc_applies(int w) { return w >= kGramTcMinW && w <= kMaxW; }
 bool gram_tc_aligned(const double*, int64_t) { return true; }
 // every table a launch is given has to be there
 int missing = 0;
+int64_t calls = 0, exponents = 0, grams = 0;
 void want(const void* p) { missing += p == nullptr; }
 cudaError_t launch_mpk_items(const SysDesc* a, const RowItem* b, int, const int* c, int, bool, int*, cudaStream_t) {
+  ++calls;
   want(a), want(b), want(c);
   return cudaSuccess;
 }
 cudaError_t launch_mpk_items_both(const SysDesc* a, const RowItem* b, int, const int* c, int, cudaStream_t) {
+  ++calls;
   want(a), want(b), want(c);
   return cudaSuccess;
 }
-cudaError_t launch_tc_items_exponents(int, const double*, int64_t, const GramPiece* a, int, const int*, int*,
+cudaError_t launch_tc_items_exponents(int, const double*, int64_t, const GramPiece* a, int n, const int*, int*,
                                       cudaStream_t) {
+  exponents += n > 0;
+  calls += n > 0;
   want(a);
   return cudaSuccess;
 }
 cudaError_t launch_gram_items(int, const SysDesc*, const GramItem* a, int, const int*, double* b, int, bool,
                               cudaStream_t) {
+  ++calls;
   want(a), want(b);
   return cudaSuccess;
 }
 cudaError_t launch_gram_items_finalize(int, const double* a, const int*, const int*, const int*, int, double*, int64_t,
                                        bool, cudaStream_t) {
+  ++calls;
   want(a);
   return cudaSuccess;
 }
 cudaError_t launch_gram_tc_items(int, const double*, int64_t, int64_t, const GramPiece* a, int, const int*, const int*,
                                  double* b, unsigned long long* c, unsigned* d, cudaStream_t) {
+  ++grams;
+  ++calls;
   want(a), want(b), want(c), want(d);
   return cudaSuccess;
 }
@@ -122,6 +137,7 @@ cudaError_t launch_gram_tc_items(int, const double*, int64_t, int64_t, const Gra
 cudaError_t launch_block_ctrl_batch(const double*, int64_t, const double*, const double*, const double*, BlockState* st,
                                     int count, int, int, double*, int64_t, double*, int, double*, int, double*,
                                     unsigned*, cudaStream_t) {
+  ++calls;
   for (int q = 0; q < count; ++q) {
     st[q].s_k = st[q].active ? 1 : 0;
     st[q].converged = st[q].m + 1 >= 6;
@@ -130,22 +146,57 @@ cudaError_t launch_block_ctrl_batch(const double*, int64_t, const double*, const
 }
 cudaError_t launch_recover_items(int, const SysDesc*, const RowItem* a, int, const int*, const double*, int64_t,
                                  cudaStream_t) {
+  ++calls;
   want(a);
   return cudaSuccess;
 }
 cudaError_t launch_residual_items(const SysDesc*, const RowItem* a, int, const int*, int, cudaStream_t) {
+  ++calls;
   want(a);
   return cudaSuccess;
 }
 // ||b||^2 = ||r||^2 = 1: every system needs blocks
 cudaError_t launch_seg_sumsq(const SysDesc*, const int* list, int n, int, double* out, cudaStream_t) {
+  ++calls;
   for (int i = 0; i < n; ++i) out[list[i]] = 1.0;
   return cudaSuccess;
 }
 cudaError_t launch_fill_uniform(double*, int64_t, uint64_t, cudaStream_t) { return cudaSuccess; }
 }  // namespace ascg
 
-int main() {
+int count_launches() {
+  for (int64_t n : {700, 3000, 250000, 1100000}) {
+    ascg_options o{};
+    o.method = ASCG_ADAPTIVE;
+    o.s_max = o.s0 = o.f = 8;
+    o.max_iters = 100;
+    ascg_server srv = nullptr;
+    if (ascg_server_create(&o, (int64_t)1 << 30, 4, nullptr, &srv) != ASCG_OK) return 2;
+    ascg::calls = 0;
+    ascg_completion c[8];
+    int nd = 0, na = 1, np = 0;
+    double b = 0, x = 0;
+    if (ascg_server_submit(srv, (ascg_op)(uintptr_t)n, &b, &x, 1e-8, 1) != ASCG_OK) return 3;
+    while (na + np > 0)
+      if (ascg_server_step(srv, c, 8, &nd, &na, &np) != ASCG_OK) return 4;
+    ascg_server_stats st;
+    ascg_server_info(srv, &st);
+    std::printf("n %lld reported %lld made %lld\n", (long long)n, (long long)st.launches, (long long)ascg::calls);
+    ascg_server_destroy(srv);
+  }
+  return 0;
+}
+
+int tune() {
+  int64_t rows = 0;
+  double table[3 * 16];
+  int nrow = 0;
+  if (ascg_tune_gram_schedule(4, &rows, table, 16, &nrow, nullptr) != ASCG_OK) return 2;
+  std::printf("sizes %d grams %lld exponents %lld\n", nrow, (long long)ascg::grams, (long long)ascg::exponents);
+  return 0;
+}
+
+int growth() {
   for (int k = 1; k < 40; ++k) {
     ascg_options o{};
     o.method = ASCG_ADAPTIVE;
@@ -186,4 +237,9 @@ int main() {
   }
   std::printf("leaked %zu\n", fake::live.size());
   return 0;
+}
+
+int main(int argc, char** argv) {
+  const std::string what = argc > 1 ? argv[1] : "";
+  return what == "growth" ? growth() : what == "count" ? count_launches() : what == "tune" ? tune() : 1;
 }

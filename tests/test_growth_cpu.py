@@ -1,4 +1,4 @@
-"""Solve server under failing device allocations, on the CPU: the engine with a fake CUDA runtime (growth_harness.cu).
+"""The lockstep engine on the CPU, with a fake CUDA runtime (growth_harness.cu): failing allocations, and what is launched.
 
 A step whose tables cannot grow returns ASCG_ERR_OOM. No launch may then get a table that is not there, the requests
 that were not yet running are queued again, and later steps finish all of them.
@@ -14,17 +14,22 @@ ROOT = os.path.dirname(HERE)
 
 
 @pytest.fixture(scope="module")
-def lines(tmp_path_factory):
+def run(tmp_path_factory):
     exe = str(tmp_path_factory.mktemp("growth") / "growth")
     nvcc = "/usr/local/cuda/bin/nvcc" if os.path.exists("/usr/local/cuda/bin/nvcc") else "nvcc"
     subprocess.run([nvcc, "-std=c++17", "-w", "-gencode", "arch=compute_103a,code=sm_103a", "--expt-relaxed-constexpr",
                     "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_1701_03989_gb300", "csrc"),
                     os.path.join(HERE, "growth_harness.cu"), "-o", exe], check=True)
-    return subprocess.run([exe], check=True, capture_output=True, text=True, timeout=120).stdout.splitlines()
+    return lambda what: subprocess.run([exe, what], check=True, capture_output=True, text=True, timeout=120).stdout.splitlines()
 
 
-def test_failed_growth_is_made_up_for(lines):
-    rows = [dict(zip(m[0::2], map(int, m[1::2]))) for m in (re.split(r"\s+", l) for l in lines[:-1])]
+def _rows(lines):
+    return [dict(zip(m[0::2], map(int, m[1::2]))) for m in (re.split(r"\s+", l) for l in lines)]
+
+
+def test_failed_growth_is_made_up_for(run):
+    lines = run("growth")
+    rows = _rows(lines[:-1])
     assert len(rows) > 5 and [r["hit"] for r in rows] == [1] * (len(rows) - 1) + [0]
     for r in rows:
         assert r["status"] == (2 if r["hit"] else 0)       # ASCG_ERR_OOM
@@ -33,3 +38,12 @@ def test_failed_growth_is_made_up_for(lines):
         if r["hit"]:
             assert r["queued"] >= 1 and r["running"] + r["queued"] == 4
     assert lines[-1] == "leaked 0"
+
+
+def test_reported_launches_are_those_made(run):
+    """Systems below the tensor-core line, with exponents recorded by the steps, with both chains in a thread (the exponents
+    take a launch), and from 2^20 rows."""
+    rows = _rows(run("count"))
+    assert [r["n"] for r in rows] == [700, 3000, 250000, 1100000]
+    for r in rows:
+        assert r["reported"] == r["made"] > 0, r
