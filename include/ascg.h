@@ -527,10 +527,12 @@ ascg_status ascg_server_destroy(ascg_server srv);
 /* Autotuner of the batched Gram schedule. For w = 2 s_max + 1 and sizes
  * n = 2^12, 2^13, ..., 2^22, times on this GPU the Gram of one system of n
  * rows (random basis) in the FP64 item launch and in the tensor-core item
- * launch (kernel, finalize; the column exponents come from the matrix powers
- * steps in a solve), each the median of several runs. In a batch each launch covers all its systems and fills the GPU, so
- * a system costs the per-row rate at full load (taken at the largest size)
- * times the rows read: n in FP64, round_up(n, 1024) on the tensor cores.
+ * launch (kernel, finalize, and from 2^20 rows the pass for the column
+ * exponents, which in smaller batches the matrix powers steps may record),
+ * each the median of several runs. In a batch each launch covers all its
+ * systems and fills the GPU, so a system costs the per-row rate at full load
+ * (taken at the largest size) times the rows read: n in FP64, round_up(n,
+ * 1024) on the tensor cores.
  * Writes to *tc_lane_rows the smallest power of two >= 256 from which the
  * tensor cores cost less at every larger size (or -1 if they never do), for
  * ascg_options.tc_lane_rows. table (host, may be NULL): up to table_cap rows

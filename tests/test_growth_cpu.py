@@ -47,3 +47,10 @@ def test_reported_launches_are_those_made(run):
     assert [r["n"] for r in rows] == [700, 3000, 250000, 1100000]
     for r in rows:
         assert r["reported"] == r["made"] > 0, r
+
+
+def test_tuner_times_the_exponents_of_large_batches(run):
+    """11 sizes, six Grams each; one exponent pass to prepare each size, and one with every Gram of the three sizes of at
+    least 2^20 rows, in whose batches no system's steps record the exponents."""
+    (r,) = _rows(run("tune"))
+    assert r == {"sizes": 11, "grams": 66, "exponents": 11 + 3 * 6}
