@@ -451,14 +451,20 @@ typedef struct {
 
 /* Creates a server. opts: as for ascg_solve_batch (an s-step method, the
  * MONOMIAL basis; s_seq is copied), history buffers NULL; eps_target is per
- * request. hbm_budget: device bytes the server may hold for running
- * systems. A system of n rows holds (2 s_max + 1) 8 round_up(n, 1024) bytes
+ * request. hbm_budget: device bytes for the bases and the Gram partials of
+ * the running systems. A system of n rows holds (2 s_max + 1) 8 round_up(n, 1024) bytes
  * of basis (a row range of one shared matrix) plus (2 s_max + 1)(s_max + 1)
  * 8 bytes of Gram partials per FP64 Gram item (1024 to 8192 rows, about n/16
  * as a power of two) and per tensor-core Gram item (8192 rows). The basis
- * matrix takes the budget less the partials' share and is allocated here;
- * the partial and row-table buffers (at most 80 bytes per 256 rows) grow on
- * demand within that share.
+ * matrix takes the budget less the partials' share, which is what the most
+ * rows it could hold would need, and is allocated here. The partials are
+ * allocated as systems come; the buffers of a size class (there are three)
+ * double when they grow, so they hold up to twice what the systems that it
+ * ran at once have needed. Beside the budget the server holds, by the same
+ * rule, tables of at most 96 bytes per 256 rows or part of them and, per
+ * tensor-core Gram item, up to 256 items a class, 16 (2 s_max + 1)(s_max + 1)
+ * + 4 bytes of exact sums; and, from its creation, 25 kB per possible system
+ * (max_systems) in each class.
  * max_systems: most systems running at once (1 .. 2^20). cuda_stream: the
  * caller's stream, which orders submissions after the caller's work; the
  * server runs its blocks on streams of its own. The operators are the

@@ -945,16 +945,19 @@ class Lockstep {
   ascg_status grow_titems(int64_t titems, int64_t pieces) {
     LS_TRY(regrow(&d_tpart_, &tcap_items_, titems, tcnp_));
     LS_TRY(regrow(&d_pieces_, &pcap_, pieces));
-    if (!d_ptick_) {  // the sums of split items and their tickets, left zero by every block
-      const size_t nsums = (size_t)kSplitItems * 2 * tcnp_;
-      if (!d_psums_) LS_TRY(dalloc(&d_psums_, nsums));
-      unsigned* tick = nullptr;
-      LS_TRY(dalloc(&tick, (size_t)kSplitItems));
-      cudaError_t e = cudaMemsetAsync(d_psums_, 0, sizeof(unsigned long long) * nsums, s_);
-      if (e == cudaSuccess) e = cudaMemsetAsync(tick, 0, sizeof(unsigned) * kSplitItems, s_);
-      if (e != cudaSuccess) dfree(tick);
-      LS_CUDA(e);
-      d_ptick_ = tick;
+    // the sums of split items and their tickets, left zero by every block
+    const int64_t split = std::min<int64_t>(titems, kSplitItems);
+    if (split > scap_) {
+      const int64_t want = std::min<int64_t>(std::max(split, 2 * scap_), kSplitItems);
+      LS_CUDA(cudaStreamSynchronize(s_));
+      scap_ = 0;
+      dfree(d_psums_);
+      dfree(d_ptick_);
+      LS_TRY(dalloc(&d_psums_, (size_t)(want * 2 * tcnp_)));
+      LS_TRY(dalloc(&d_ptick_, (size_t)want));
+      LS_CUDA(cudaMemsetAsync(d_psums_, 0, sizeof(unsigned long long) * (size_t)(want * 2 * tcnp_), s_));
+      LS_CUDA(cudaMemsetAsync(d_ptick_, 0, sizeof(unsigned) * (size_t)want, s_));
+      scap_ = want;
     }
     return ASCG_OK;
   }
@@ -1107,7 +1110,7 @@ class Lockstep {
   GramPiece* d_pieces_ = nullptr;  // tensor-core Gram items (row ranges in the shared matrix) in pieces
   unsigned long long* d_psums_ = nullptr;  // integer sums of split items
   unsigned* d_ptick_ = nullptr;            // and their tickets
-  int64_t pcap_ = 0;
+  int64_t pcap_ = 0, scap_ = 0;
   double* d_tpart_ = nullptr;     // their partials, tcnp_ each
   int* d_emax_ = nullptr;         // per-lane column exponents, kEmaxCopies x kMaxW each
   int64_t tcap_items_ = 0;

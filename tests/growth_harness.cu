@@ -5,6 +5,7 @@
 //            what the failed step left behind and how the retry ended
 //   count    the launches that ascg_server_info reports, and those made, for a server
 //            with one system of each size
+//   memory   the most device bytes held while systems run, beside what they need
 //   tune     the exponent passes and tensor-core Grams that the autotuner makes, by rows
 #include <cuda_runtime.h>
 
@@ -18,23 +19,26 @@
 #include <deque>
 #include <iterator>
 #include <map>
-#include <set>
 #include <string>
 #include <vector>
 
 namespace fake {
 int count = 0, fail_at = -1;
-std::set<void*> live;
+std::map<void*, size_t> live;
+size_t held = 0, peak = 0;
 cudaError_t alloc(void** p, size_t n) {
   if (++count == fail_at) {
     *p = nullptr;
     return cudaErrorMemoryAllocation;
   }
   *p = std::calloc(1, n ? n : 1);
-  live.insert(*p);
+  live[*p] = n;
+  held += n;
+  peak = held > peak ? held : peak;
   return cudaSuccess;
 }
 cudaError_t release(void* p) {
+  if (p) held -= live[p];
   live.erase(p);
   std::free(p);
   return cudaSuccess;
@@ -187,6 +191,45 @@ int count_launches() {
   return 0;
 }
 
+// Rounds of requests on one server, each drained before the next comes.
+int memory() {
+  const std::vector<std::vector<int64_t>> rounds = {
+      std::vector<int64_t>(16, 1000), {64000, 65000, 30000}, {200000, 120000}, {600000}, std::vector<int64_t>(16, 5000)};
+  for (int s : {2, 8, 16}) {
+    ascg_options o{};
+    o.method = ASCG_ADAPTIVE;
+    o.s_max = o.s0 = o.f = s;
+    o.max_iters = 100;
+    ascg_server srv = nullptr;
+    fake::peak = fake::held;
+    const size_t before = fake::held;
+    if (ascg_server_create(&o, (int64_t)1 << 30, 16, nullptr, &srv) != ASCG_OK) return 2;
+    int64_t git[3] = {0, 0, 0}, tit[3] = {0, 0, 0}, units[3] = {0, 0, 0};
+    double b = 0, x = 0;
+    for (const auto& r : rounds) {
+      for (int64_t n : r)
+        if (ascg_server_submit(srv, (ascg_op)(uintptr_t)n, &b, &x, 1e-8, 1) != ASCG_OK) return 3;
+      ascg_completion c[32];
+      int nd = 0, na = 1, np = 0;
+      while (na + np > 0) {
+        if (ascg_server_step(srv, c, 32, &nd, &na, &np) != ASCG_OK) return 4;
+        for (int g = 0; g < 3; ++g) {
+          const ascg::Lockstep& e = srv->group[g].eng;
+          git[g] = std::max(git[g], (int64_t)e.gitems_.size());
+          tit[g] = std::max(tit[g], (int64_t)e.titems_.size());
+          units[g] = std::max(units[g], (int64_t)e.ritems_.size());
+        }
+      }
+    }
+    std::printf("s %d arena %zu peak %zu gitems %lld titems %lld units %lld split %lld\n", s, srv->arena.bytes_total(),
+                fake::peak - before, (long long)(git[0] + git[1] + git[2]), (long long)(tit[0] + tit[1] + tit[2]),
+                (long long)(units[0] + units[1] + units[2]),
+                (long long)(std::min<int64_t>(tit[0], 256) + std::min<int64_t>(tit[1], 256) + std::min<int64_t>(tit[2], 256)));
+    ascg_server_destroy(srv);
+  }
+  return 0;
+}
+
 int tune() {
   int64_t rows = 0;
   double table[3 * 16];
@@ -241,5 +284,5 @@ int growth() {
 
 int main(int argc, char** argv) {
   const std::string what = argc > 1 ? argv[1] : "";
-  return what == "growth" ? growth() : what == "count" ? count_launches() : what == "tune" ? tune() : 1;
+  return what == "growth" ? growth() : what == "count" ? count_launches() : what == "memory" ? memory() : what == "tune" ? tune() : 1;
 }

@@ -54,3 +54,18 @@ def test_tuner_times_the_exponents_of_large_batches(run):
     least 2^20 rows, in whose batches no system's steps record the exponents."""
     (r,) = _rows(run("tune"))
     assert r == {"sizes": 11, "grams": 66, "exponents": 11 + 3 * 6}
+
+
+def test_server_memory_is_what_the_header_states(run):
+    """A 1 GB budget, 16 systems at once: the basis matrix and the partials' first buffers as at creation, buffers at most
+    twice what the systems have needed, tables, sums and records as the header gives them."""
+    for r in _rows(run("memory")):
+        w = 2 * r["s"] + 1
+        pairs = w * (w + 1) // 2
+        budget = 1 << 30
+        first = (budget // (8 * w) // 1024 + 16) // 3 + 1          # partials per class at creation
+        assert r["arena"] <= budget
+        partials = 8 * pairs * max(2 * r["gitems"], 3 * first) + 8 * pairs * 2 * r["titems"]
+        tables = 2 * 96 * r["units"] + 3 * (1024 * 16 + first * 16)
+        sums = 2 * r["split"] * (16 * pairs + 4)
+        assert r["peak"] <= r["arena"] + partials + tables + sums + 3 * 16 * 25000, r
