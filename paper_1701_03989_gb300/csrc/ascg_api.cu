@@ -791,7 +791,6 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
     const bool ahead = o.method == ASCG_FIXED_S || o.method == ASCG_VARIABLE_S ||
                        (o.method == ASCG_ADAPTIVE && o.f >= o.s_max - 1);
     int wb_of[kRing] = {};
-    bool rec_tc_of[kRing] = {};  // the block's recovery ran on the tensor cores
     bool rec_x_of[kRing] = {};   // the block's recovery updated x too
     for (int q = 0; q < kRing; ++q) __atomic_store_n(w.h_seq + q, 0u, __ATOMIC_RELEASE);
     int sbar_of[kRing] = {};
@@ -884,7 +883,6 @@ ascg_status solve_device(ascg_op op, const double* b, double* x, const ascg_opti
       // same sums either way.
       const bool tc_rec = tc_gram && !rec_fp64;
       const bool one_pass = !tc_rec && n <= kOnePassRows;
-      rec_tc_of[slot] = tc_rec;
       rec_x_of[slot] = tc_rec || one_pass;
       if (tc_rec)
         ASCG_CUDA(launch_recover_tc(n, wb, Yc, w.ldY, w.expp, cbuf[cur], x, Ybuf[cur ^ 1] + w.ldY, Ybuf[cur ^ 1], s,

@@ -1,8 +1,9 @@
 // Shared device helpers and kernel declarations of libascg.
 //
-// Arithmetic is IEEE double throughout. On GB300 the FP64 pipe retires one
-// warp-wide DFMA per ~20 SM cycles (about 1.0 TFLOP/s per GPU), and an
-// instruction costs the same with 1 or 32 active lanes. Kernels therefore
+// Arithmetic is IEEE double throughout. On GB300 an SM retires one warp-wide
+// DFMA per 16 cycles (1.26 TFLOP/s per GPU; the best kernel here, the FP64
+// recovery, reaches 0.96 of it), and an instruction costs the same with 1 or 32
+// active lanes. Kernels therefore
 // keep every lane busy and count FP64 instructions, not bytes.
 #pragma once
 

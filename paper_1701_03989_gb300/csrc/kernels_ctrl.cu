@@ -4,11 +4,12 @@
 // shifts.
 //
 // All of this is tiny dense work on matrices of order <= 33. On GB300 an FP64
-// warp instruction takes 64 cycles of its SM sub-partition (77 with all four
-// busy) whether 0, 1 or 32 lanes are active, a comparison 110 to 220, a
-// reciprocal 325, a square root 550, a shuffle and add 110. So this code keeps the lanes busy on
-// independent work: one lane per row for the Householder steps, and 64
-// evaluation points per Sturm multisection round.
+// warp instruction takes 64 cycles of its SM sub-partition (77 in a probe of
+// this code's pattern with all four busy) whether 0, 1 or 32 lanes are active, a
+// comparison 110 to 220, a reciprocal 325, a square root 550, a shuffle and add
+// 110. So this code keeps the lanes busy on independent work: one lane per row
+// for the Householder steps, and 64 evaluation points per Sturm multisection
+// round.
 #include <math_constants.h>
 
 #include "ascg_common.cuh"
@@ -57,8 +58,8 @@ __device__ void gershgorin(const double* d, const double* e, int m, double* lo, 
 // rescalings do not change signs), the backward error of the pivot form.
 // The loop is unrolled with d and e2 in registers. Each step costs three FP64
 // instructions (d_k - x, the product with e2 and the FMA); on GB300 an SM
-// sub-partition issues about one FP64 warp instruction per 64 cycles (77 with
-// all four busy), and that rate sets the time of a multisection round, so a
+// sub-partition issues at most one FP64 warp instruction per 64 cycles (77 seen
+// here with all four busy), and that rate sets the time of a multisection round, so a
 // minor is looked at only once the next step's instructions are on their way
 // (244 cycles a step against 260 before and 231 for the three alone). The
 // leading minors grow at most like (1 + sqrt 2)^k <= 2^43 for M <= 33, so they

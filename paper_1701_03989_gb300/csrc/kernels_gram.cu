@@ -2,7 +2,7 @@
 //
 // This is the largest FP64 cost of a block: w(w+1)/2 fused multiply-adds per
 // row (561 at w = 33), against about 2 * (2s-1) * nnz/n for the matrix powers
-// kernel. GB300 runs FP64 at one warp instruction per ~20 SM cycles, and DMMA
+// kernel. GB300 runs FP64 at one warp instruction per 16 SM cycles, and DMMA
 // (mma.sync m8n8k4 f64) shares that pipe at the same rate. So the Gram stays
 // on CUDA cores, and the design goal is to keep every FP64 lane busy on a
 // distinct product.

@@ -367,8 +367,10 @@ class Lockstep {
   // systems still covers the SMs: a CTA takes about 5 us for the launch, pipeline
   // fill and epilogue and 9 us per chunk, and with whole items a 93057-row system
   // alone had 12 CTAs of 78 us. 32 systems of 1e3..1e5 rows (690 chunks): 190.4 ->
-  // 182.2 ms a batch. With more, whole items: one system of 977 chunks, 60
-  // iterations, 24.6 ms in pieces of two chunks, 23.9 whole.
+  // 182.2 ms a batch. Whole items / pieces, one 2D Poisson system, 60 iterations,
+  // s = 5 and 10, ms: 565 chunks 5.78 / 5.29 and 8.75 / 7.84, 792 6.87 / 6.74 and
+  // 10.44 / 10.06, 900 7.31 / 7.29 and 11.24 / 11.02, 977 7.74 / 8.01 and 11.91 /
+  // 12.10, 1098 8.31 / 8.86 and 12.96 / 13.39.
   static constexpr int kSplitItems = 256;
   static std::vector<GramPiece> pieces_of(const std::vector<GramItem>& items) {
     std::vector<GramPiece> out;
