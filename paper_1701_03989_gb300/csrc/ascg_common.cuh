@@ -159,8 +159,8 @@ inline cudaError_t smem_limit_once(std::atomic<uint64_t>& done, K* kernel, int b
 //  - by __ldca, __ldcg, __ldcs or load_after_wait: volatile statements like the
 //    wait itself, which keep their order. The kernels that are bound by their
 //    loads do this (the same code as with __ldg; with relearned pointers a matrix
-//    powers step took 12 % longer: Chebyshev, s = 16, 100^3, 531 us against 472;
-//    in classical CG it costs 0.7 % of a 128^3 solve, 43.0 -> 43.3 ms);
+//    powers step took 12 % longer: Chebyshev, s = 16, 100^3, 531 us against 472),
+//    and issue a row's loads before the first is used, since none can be moved;
 //  - by ordinary loads through a pointer named in pdl_wait(), or in relearn()
 //    after it: the compiler learns its value only there;
 //  - by ordinary loads through a pointer without __restrict__, which the wait's

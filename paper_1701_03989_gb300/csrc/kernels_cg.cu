@@ -219,9 +219,10 @@ __global__ void __launch_bounds__(256) cg_pupdate_kernel(int64_t n, double* __re
   if (!st->active) return;  // this iteration was skipped (solve already done)
   const double alpha = st->alpha, beta = st->beta;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double pi = __ldca(p + i);
-    x[i] = fma(alpha, pi, __ldca(x + i));    // x += q, q = alpha p (the iteration's p)
-    p[i] = fma(beta, pi, __ldca(r + i));     // p = r + beta p
+    // all three in flight before the first is used (14.2 us at 128^3 otherwise)
+    const double pi = __ldca(p + i), xi = __ldca(x + i), ri = __ldca(r + i);
+    x[i] = fma(alpha, pi, xi);               // x += q, q = alpha p (the iteration's p)
+    p[i] = fma(beta, pi, ri);                // p = r + beta p
   }
 }
 
