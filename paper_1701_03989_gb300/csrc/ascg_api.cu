@@ -248,7 +248,6 @@ struct Workspace {
   double* h_scal = nullptr;
   cudaEvent_t ev[8] = {};
   cudaEvent_t ev_blk[kRing][5] = {};  // per record slot: the phase boundaries of a block (timing)
-  bool events = false;
   cudaStream_t side = nullptr;  // x += Y x' of the previous block
   cudaEvent_t ev_gram = nullptr, ev_x[2] = {};
 
@@ -263,18 +262,17 @@ struct Workspace {
     if (h_cgs) cudaFreeHost(h_cgs);
     if (h_scal) cudaFreeHost(h_scal);
     h_bst = nullptr; h_seq = nullptr; h_cgs = nullptr; h_scal = nullptr;
-    if (events) {
-      for (auto& e : ev) cudaEventDestroy(e);
-      for (auto& row : ev_blk)
-        for (auto& e : row) cudaEventDestroy(e);
-      cudaEventDestroy(ev_gram);
-      for (auto& e : ev_x) cudaEventDestroy(e);
-      if (side) cudaStreamDestroy(side);
-    }
-    events = false;
+    auto drop = [](cudaEvent_t& e) {
+      if (e) cudaEventDestroy(e);
+      e = nullptr;
+    };
+    for (auto& e : ev) drop(e);
+    for (auto& row : ev_blk)
+      for (auto& e : row) drop(e);
+    drop(ev_gram);
+    for (auto& e : ev_x) drop(e);
+    if (side) cudaStreamDestroy(side);
     side = nullptr;
-    ev_gram = nullptr;
-    ev_x[0] = ev_x[1] = nullptr;
     n = 0; wcols = 0; ldY = 0; partials_cap = 0; res_cap = 0; ab_cap = 0; emax_ld = 0; dt_rows = 0;
   }
 };
@@ -375,7 +373,7 @@ constexpr int64_t kOnePassRows = 131072;
 
 // Ensures the workspace can hold n rows, wcols basis columns and histories of
 // res_cap entries.
-ascg_status ensure(ascg_op op, int wcols, int res_cap) {
+ascg_status ensure_all(ascg_op op, int wcols, int res_cap) {
   Workspace& w = op->ws;
   const int64_t n = op->n;
   if (!w.counter) {
@@ -399,7 +397,6 @@ ascg_status ensure(ascg_op op, int wcols, int res_cap) {
     ASCG_CUDA(cudaEventCreateWithFlags(&w.ev_gram, cudaEventDisableTiming));
     for (auto& e : w.ev_x) ASCG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     ASCG_CUDA(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
-    w.events = true;
   }
   if (w.n != n || w.wcols < wcols) {
     dev_free(w.Y); dev_free(w.Y2); dev_free(w.q);
@@ -435,6 +432,13 @@ ascg_status ensure(ascg_op op, int wcols, int res_cap) {
     w.ab_cap = res_cap;
   }
   return ASCG_OK;
+}
+// A workspace that could not grow is given up, so that the next call starts from
+// an empty one and not from the parts that were there.
+ascg_status ensure(ascg_op op, int wcols, int res_cap) {
+  const ascg_status st = ensure_all(op, wcols, res_cap);
+  if (st != ASCG_OK) op->ws.release();
+  return st;
 }
 
 // ||B_{k,s}||_2 of eq. (AVVB) for the basis coefficients th, sg, gm. B is

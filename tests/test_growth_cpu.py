@@ -13,13 +13,18 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 
 
-@pytest.fixture(scope="module")
-def run(tmp_path_factory):
-    exe = str(tmp_path_factory.mktemp("growth") / "growth")
+def _compile(tmp, name, *extra):
+    exe = str(tmp.mktemp(name) / name)
     nvcc = "/usr/local/cuda/bin/nvcc" if os.path.exists("/usr/local/cuda/bin/nvcc") else "nvcc"
     subprocess.run([nvcc, "-std=c++17", "-w", "-gencode", "arch=compute_103a,code=sm_103a", "--expt-relaxed-constexpr",
                     "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_1701_03989_gb300", "csrc"),
-                    os.path.join(HERE, "growth_harness.cu"), "-o", exe], check=True)
+                    os.path.join(HERE, name + "_harness.cu"), "-o", exe, *extra], check=True)
+    return exe
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    exe = _compile(tmp_path_factory, "growth")
     return lambda what: subprocess.run([exe, what], check=True, capture_output=True, text=True, timeout=120).stdout.splitlines()
 
 
@@ -69,3 +74,19 @@ def test_server_memory_is_what_the_header_states(run):
         tables = 2 * 96 * r["units"] + 3 * (1024 * 16 + first * 16)
         sums = 2 * r["split"] * (16 * pairs + 4)
         assert r["peak"] <= r["arena"] + partials + tables + sums + 3 * 16 * 25000, r
+
+
+def test_workspace_after_a_failed_growth(tmp_path_factory):
+    """An operator's workspace whose k-th allocation failed: a later, smaller call finds every part, whether the workspace
+    was new or already there. The kernels' launchers come from the library; none is called."""
+    import __graft_entry__
+    __graft_entry__.build()
+    lib = os.path.join(ROOT, "paper_1701_03989_gb300")
+    exe = _compile(tmp_path_factory, "workspace", "-L", lib, "-l:libascg.so", "-Xlinker", "-rpath," + lib)
+    lines = subprocess.run([exe], check=True, capture_output=True, text=True, timeout=120).stdout.splitlines()
+    rows = _rows(lines[:-1])
+    for grown in (0, 1):
+        r = [q for q in rows if q["grown"] == grown]
+        assert len(r) > 3 and [q["status"] for q in r] == [2] * (len(r) - 1) + [0]  # ASCG_ERR_OOM until nothing fails
+    assert all(q["again"] == 0 and q["missing"] == 0 for q in rows)
+    assert lines[-1] == "leaked 0"
